@@ -1,0 +1,280 @@
+"""The work that users of this library have it do, as cases to be timed and compared.
+
+A case is one attention layer of a video diffusion transformer: which entry points it calls ("path"), batch,
+heads, channels per head, the latent grid T x Hs x Ws whose N = T*Hs*Ws tokens attend each other, and the kept
+lists (3-D windows, irregular lists, Top-K, 1-D windows of ST-SWA, or all blocks).  Everything a user's program
+keeps between calls -- static lists, rotation table, weights, workspace -- is made in prepare(); what it makes
+anew for each layer and denoising step is made in run().
+
+    fused    salad_fused_fwd                          window, irregular or all-kept lists
+    layer    salad_dynamic_scale, salad_fused_fwd     with the post-tuning threshold (one of two batch items dropped)
+    linear   salad_linear_attn_fwd                    the linear branch alone
+    rope     salad_fused_rope_fwd                     rotary linear branch
+    topk     salad_topk_mask_build, salad_fused_fwd   lists made from Q and K in every call
+    stswa    salad_fused_stswa_fwd                    every second head temporal
+    proj     salad_fused_proj_fwd                     one d x d projection block per head
+    fullproj salad_sparse_attn_fwd, salad_linear_attn_fwd, salad_proj_combine_fwd   the head-mixing projection
+"""
+from __future__ import annotations
+
+import math
+
+import torch
+
+from paper_2601_16515_b200 import salad
+
+EPS = 1e-6
+TAU = 0.5
+
+
+def _case(name, path, B, H, d, grid, window=None, lists="window", Bq=128):
+    T, Hs, Ws = grid
+    wt, wh, ww = window or (0, 0, 0)
+    c = dict(path=path, B=B, H=H, d=d, T=T, Hs=Hs, Ws=Ws, Bq=Bq, lists=lists, wt=wt, wh=wh, ww=ww)
+    if name:
+        c["name"] = name
+    return c
+
+
+def listed():
+    return [
+        # The smallest call: the tiny configuration (d = 64, 64 x 64 blocks, 1024 tokens, own frame / own row
+        # band per head), what a unit test or a toy model runs: launches and host time are all of it.
+        _case("tiny", "fused", 1, 2, 64, (4, 16, 16), lists="tiny", Bq=64),
+        # A short, small clip: a ragged grid of 2310 tokens, the 12 heads of the 1.3B model.  Fewer work items
+        # than the chip takes at once.
+        _case("clip-short", "fused", 1, 12, 128, (5, 21, 22), (1, 5, 11)),
+        # The headline workload: the 1.3B layer at 480p, 90 % block sparsity.
+        _case("wan1.3b-90", "fused", 1, 12, 128, (21, 30, 52), (2, 5, 24)),
+        # The same layer under per-head irregular lists of 5 to 15 % of the key blocks.
+        _case("wan1.3b-irregular", "fused", 1, 12, 128, (21, 30, 52), lists="irregular"),
+        # The 14B-shaped layer at 720p: the largest sparse call.
+        _case("wan14b-90", "fused", 1, 40, 128, (21, 45, 80), (2, 10, 36)),
+        # Classifier-free guidance pair at 95 % sparsity with the dynamic scale made in the call and branch
+        # dropping: a conditional item that keeps its linear branch and an unconditional one that loses it.
+        _case("cfg-95-drop", "layer", 2, 12, 128, (21, 30, 52), (1, 4, 24)),
+        # The same pair with all blocks kept: the steps that run with full attention.
+        _case("cfg-dense", "fused", 2, 12, 128, (21, 30, 52), lists="all"),
+        # The linear branch alone (the tuning and ablation runs time and test it by itself).
+        _case("linear-480p", "linear", 1, 12, 128, (21, 30, 52)),
+        # Rotary linear branch, on an odd grid of another clip length (17 x 31 x 53).
+        _case("rope-odd", "rope", 1, 12, 128, (17, 31, 53), (2, 5, 24)),
+        # Dynamic Top-K lists at 90 % sparsity, made from the call's own Q and K.
+        _case("topk-90", "topk", 1, 12, 128, (21, 30, 52), lists="topk"),
+        # The paper's ST-SWA, temporal heads re-ordered inside the call, a window of a tenth of the sequence.
+        _case("stswa-480p", "stswa", 1, 12, 128, (21, 30, 52), lists="stswa"),
+        # The full head-mixing projection on the linear branch: both branches, then the projection and the sum.
+        _case("fullproj-480p", "fullproj", 1, 12, 128, (21, 30, 52), (2, 5, 24)),
+    ]
+
+
+def draw(rng):
+    """One more case: clips of about 500 to 75600 tokens, B = 1 or 2, up to 40 heads, d = 64 or 128, every path."""
+    path = rng.choice(("fused", "fused", "fused", "layer", "linear", "rope", "topk", "stswa", "proj", "fullproj"))
+    while True:
+        n = math.exp(rng.uniform(math.log(500), math.log(75600)))
+        T = rng.randint(1, 21)
+        aspect = rng.uniform(0.5, 2.0)
+        Hs = max(2, round(math.sqrt(n / T / aspect)))
+        Ws = max(2, round(n / T / Hs))
+        N = T * Hs * Ws
+        B, d = rng.choice((1, 1, 2)), rng.choice((128, 128, 128, 64))
+        H = rng.choice((2, 5, 8, 12, 12, 16, 24, 40))
+        Bq = rng.choice((128, 128, 128, 64)) if path in ("fused", "rope", "proj") else 128
+        window = (round(T * rng.uniform(0.04, 0.2)), round(Hs * rng.uniform(0.1, 0.3)), round(Ws * rng.uniform(0.2, 0.6)))
+        lists = {"topk": "topk", "stswa": "stswa"}.get(path, "window")
+        if path == "fused":
+            lists = rng.choice(("window", "window", "irregular", "all"))
+        if not 400 <= N <= 75600 or B * H * N * d * 2 > 8e8:
+            continue
+        reach = math.prod(min(1.0, (2 * x + 2) / n) for x, n in zip(window, (T, Hs, Ws)))
+        kept = {"all": 1.0, "window": min(1.0, 1.5 * reach)}.get(lists, 0.15)
+        if B * H * d * 4.0 * N * N * kept <= 1.0e13:
+            return _case(None, path, B, H, d, (T, Hs, Ws), window, lists, Bq)
+
+
+def _sizes(case):
+    N = case["T"] * case["Hs"] * case["Ws"]
+    return case["B"], case["H"], case["d"], N, case["Bq"], -(-N // case["Bq"]), -(-N // 64)
+
+
+def _topk(nKb):
+    return max(1, round(0.1 * nKb))
+
+
+def _temporal(H):
+    return [h % 2 for h in range(H)]
+
+
+def _half_width(N):
+    return max(1, N // 20)
+
+
+def _lists(case, generator):
+    """(row_ptr, col_idx, Hm) of the kept lists that a program has before the call; None where the call makes them."""
+    B, H, d, N, Bq, nQb, nKb = _sizes(case)
+    grid = (case["T"], case["Hs"], case["Ws"])
+    kind = case["lists"]
+    if case["path"] == "linear" or kind == "topk":
+        return None
+    if kind == "stswa":
+        return (*salad.salad_stswa_mask_build(grid, _temporal(H), [_half_width(N)] * H), H)
+    if kind == "tiny":
+        return (*salad.salad_mask_build(*grid, Bq, 64, [(0, 15, 15), (3, 0, 0)]), 2)
+    if kind == "window":
+        return (*salad.salad_mask_build(*grid, Bq, 64, [(case["wt"], case["wh"], case["ww"])]), 1)
+    if kind == "all":
+        row_ptr = torch.arange(nQb + 1, dtype=torch.int32, device="cuda") * nKb
+        return row_ptr, torch.arange(nKb, dtype=torch.int32, device="cuda").repeat(nQb), 1
+    # irregular: every query block keeps the key blocks of its own tokens and others drawn at random, 5 to 15 % in all
+    rows = H * nQb
+    score = torch.rand((rows, nKb), generator=generator, device="cuda")
+    first = torch.arange(nQb, device="cuda") * Bq // 64
+    last = (torch.clamp((torch.arange(nQb, device="cuda") + 1) * Bq, max=N) - 1) // 64
+    j = torch.arange(nKb, device="cuda")
+    own = ((j >= first[:, None]) & (j <= last[:, None])).repeat(H, 1)
+    score.masked_fill_(own, 2.0)
+    lo, hi = max(1, round(0.05 * nKb)), max(2, round(0.15 * nKb))
+    length = torch.randint(lo, hi + 1, (rows,), generator=generator, device="cuda")
+    length = torch.clamp(torch.maximum(length, own.sum(1)), max=nKb)
+    rank = score.argsort(dim=1, descending=True).argsort(dim=1)
+    keep = rank < length[:, None]
+    row_ptr = torch.zeros(rows + 1, dtype=torch.int32, device="cuda")
+    row_ptr[1:] = torch.cumsum(length, 0)
+    return row_ptr, keep.nonzero()[:, 1].to(torch.int32).contiguous(), H
+
+
+def _field(case, generator):
+    """A smooth spatio-temporal field [B, H, N, d] (nearby tokens are alike), four plane waves per head."""
+    B, H, d, N = _sizes(case)[:4]
+    n = torch.arange(N, device="cuda", dtype=torch.float32)
+    t, h, w = n // (case["Hs"] * case["Ws"]), (n // case["Ws"]) % case["Hs"], n % case["Ws"]
+    pos = torch.stack((t / case["T"], h / case["Hs"], w / case["Ws"]))
+    freq = torch.randint(1, 4, (B * H, 4, 3), generator=generator, device="cuda").float()
+    angle = 2 * math.pi * (freq @ pos)                                            # [B*H, 4, N]
+    psi = 2 * math.pi * torch.rand((B * H, d, 4), generator=generator, device="cuda")
+    basis = torch.cat((angle.sin(), angle.cos()), 1).transpose(1, 2).bfloat16()
+    mix = torch.cat((psi.cos(), psi.sin()), 2).transpose(1, 2).bfloat16()
+    return (0.25 * (basis @ mix)).view(B, H, N, d)
+
+
+def prepare(case, seed):
+    B, H, d, N, Bq, nQb, nKb = _sizes(case)
+    g = torch.Generator(device="cuda").manual_seed(seed)
+
+    def noise(*shape, dtype=torch.bfloat16):
+        return torch.randn(shape, generator=g, device="cuda", dtype=dtype)
+
+    # Q, K, V as the transformer hands them to attention: unit noise, and a smooth field that Q and K share
+    # (nearby tokens score higher); the tiny configuration has half the noise and no field
+    if case["lists"] == "tiny":
+        q, k, v = (noise(B, H, N, d) * 0.5 for _ in range(3))
+    else:
+        shared = _field(case, g)
+        q, k = noise(B, H, N, d).add_(shared), noise(B, H, N, d).add_(shared)
+        v = noise(B, H, N, d).add_(_field(case, g))
+    s = dict(case=case, q=q, k=k, v=v, ws=salad.alloc_workspace(B, H, N, d, Bq, 64))
+    lists = _lists(case, g)
+    if lists is not None:
+        s["rp"], s["ci"], s["Hm"] = lists
+    # scales: lambda of a tuned layer, s_b of this timestep
+    s["lam"] = torch.rand(H, generator=g, device="cuda")
+    s["sb"] = torch.sigmoid(torch.randn(B, generator=g, device="cuda"))
+    path = case["path"]
+    if path == "layer":
+        s["w"] = noise(H * d, dtype=torch.float32) / math.sqrt(H * d)
+        s["x"] = noise(B, N, H * d)
+        for b in range(B):                                 # item 0 well above the threshold, item 1 well below
+            s["x"][b] += ((0.8 if b % 2 == 0 else -0.8) * s["w"]).bfloat16()
+    elif path == "rope":
+        s["rope"] = salad.salad_rope3d_table_build(case["T"], case["Hs"], case["Ws"], d)
+    elif path == "stswa":
+        s["flags"] = _temporal(H)
+    elif path == "proj":
+        s["blocks"] = noise(H, d, d) / math.sqrt(d)
+    elif path == "fullproj":
+        s["weight"] = noise(H * d, H * d) / math.sqrt(H * d)
+        s["bias"] = noise(H * d, dtype=torch.float32) * 0.1
+    return s
+
+
+def run(s):
+    case = s["case"]
+    path, Bq, q, k, v, ws = case["path"], case["Bq"], s["q"], s["k"], s["v"], s["ws"]
+    if path == "fused":
+        return salad.salad_fused_fwd(q, k, v, s["rp"], s["ci"], s["Hm"], s["lam"], s["sb"], Bq=Bq, eps=EPS, workspace=ws)
+    if path == "layer":
+        scale = salad.salad_dynamic_scale(s["x"], s["w"])
+        out = salad.salad_fused_fwd(q, k, v, s["rp"], s["ci"], s["Hm"], s["lam"], scale, eps=EPS, workspace=ws, drop_tau=TAU)
+        return scale, out
+    if path == "linear":
+        return salad.salad_linear_attn_fwd(q, k, v, eps=EPS, workspace=ws)
+    if path == "rope":
+        return salad.salad_fused_rope_fwd(q, k, v, s["rp"], s["ci"], s["Hm"], s["lam"], s["sb"], s["rope"], Bq=Bq, eps=EPS,
+                                          workspace=ws)
+    if path == "topk":
+        B, H, nKb = q.shape[0], q.shape[1], -(-q.shape[2] // 64)
+        rp, ci = salad.salad_topk_mask_build(q, k, _topk(nKb))
+        return rp, ci, salad.salad_fused_fwd(q, k, v, rp, ci, B * H, s["lam"], s["sb"], eps=EPS, workspace=ws)
+    if path == "stswa":
+        grid = (case["T"], case["Hs"], case["Ws"])
+        return salad.salad_fused_stswa_fwd(q, k, v, grid, s["flags"], s["rp"], s["ci"], s["lam"], s["sb"], eps=EPS)
+    if path == "proj":
+        return salad.salad_fused_proj_fwd(q, k, v, s["rp"], s["ci"], s["Hm"], s["blocks"], s["sb"], Bq=Bq, eps=EPS,
+                                          workspace=ws)
+    o_s = salad.salad_sparse_attn_fwd(q, k, v, s["rp"], s["ci"], s["Hm"], workspace=ws)
+    o_l = salad.salad_linear_attn_fwd(q, k, v, eps=EPS, workspace=ws)
+    return salad.salad_proj_combine_fwd(o_s, o_l, s["weight"], s["sb"], s["bias"])
+
+
+def work(case):
+    """Q, K, V (and X, the weights, the table) read once, the output written once; the products of the kept
+    blocks (ragged blocks at their valid size), of the linear state and of its application."""
+    B, H, d, N, Bq, nQb, nKb = _sizes(case)
+    path = case["path"]
+    nbytes, flops = 4.0 * B * H * N * d * 2, 0.0
+    if path != "linear":
+        if case["lists"] == "topk":
+            pairs = B * H * nQb * _topk(nKb) * (N / nQb) * (N / nKb)
+            nbytes += 4.0 * B * H * nQb * _topk(nKb)
+        else:
+            rp, ci, Hm = _lists(case, torch.Generator(device="cuda").manual_seed(1))
+            nbytes += 4.0 * (rp.numel() + ci.numel())
+            rows = (rp.numel() - 1) // Hm
+            if case["lists"] == "stswa":         # blocks of whole spatial positions in the temporal heads
+                T = case["T"]
+                q_rows, k_rows = [128, (128 // T) * T], [64, (64 // T) * T]
+                kind = _temporal(H)
+            else:
+                q_rows, k_rows, kind = [Bq], [64], [0] * Hm
+            counts = (rp[1:] - rp[:-1]).long()
+            row = torch.repeat_interleave(torch.arange(Hm * rows, device="cuda"), counts)
+            head = torch.tensor(kind, device="cuda")[row // rows]
+            qr, kr = torch.tensor(q_rows, device="cuda")[head], torch.tensor(k_rows, device="cuda")[head]
+            vq = torch.minimum(qr, N - (row % rows) * qr).double()
+            vk = torch.minimum(kr, N - ci.long() * kr).double()
+            pairs = float((vq * vk).sum()) * B * H / Hm
+        flops += 4.0 * d * pairs
+    kept_items = (B + 1) // 2 if path == "layer" else B          # items whose linear branch is not dropped
+    flops += 4.0 * kept_items * H * N * d * d
+    if path == "layer":
+        nbytes += 2.0 * B * N * H * d
+        flops += 2.0 * B * N * H * d
+    elif path == "rope":
+        nbytes += 2.0 * N * d
+    elif path == "proj":
+        nbytes += 2.0 * H * d * d
+    elif path == "fullproj":
+        nbytes += 2.0 * (H * d) ** 2
+        flops += 2.0 * B * N * (H * d) ** 2
+    return {"bytes": nbytes, "flops": flops}
+
+
+def tolerance(case):
+    # Outputs are bf16 with bf16 probabilities and a bf16 linear state inside.  Against the same layers in 64 bits
+    # (small grids of every kind of list, the linear branch, the projection) they are off by 1.8e-3 to 2.3e-3 in
+    # the 2-norm and by up to 1.5e-2 at one value; four times that.
+    if case["path"] == "topk":
+        # the scores of two key blocks can agree to fp32 rounding: either may be kept
+        return {"rel": 9e-3, "max": 6e-2, "differ": 1e-3}
+    return {"rel": 9e-3, "max": 6e-2}
