@@ -227,6 +227,94 @@ def run(s):
     return salad.salad_proj_combine_fwd(o_s, o_l, s["weight"], s["sb"], s["bias"])
 
 
+def _attention64(s, perms, q_rows, k_rows, lists):
+    """Softmax attention over the kept blocks in 64 bits, [B, H, N, d].  Head h takes its tokens in the order
+    perms[h % len], cut into blocks of q_rows[h % len] x k_rows[h % len] tokens."""
+    q, k, v = s["q"], s["k"], s["v"]
+    B, H, N, d = q.shape
+    rp, ci, Hm = lists
+    rows = (rp.numel() - 1) // Hm
+    counts = (rp[1:] - rp[:-1]).long()
+    row = torch.repeat_interleave(torch.arange(Hm * rows, device="cuda"), counts)
+    out = torch.empty((B, H, N, d), dtype=torch.float64, device="cuda")
+    keep = None
+    for b in range(B):
+        for h in range(H):
+            i = h % len(perms)
+            hm = 0 if Hm == 1 else h if Hm == H else b * H + h
+            if keep is None or Hm > 1:
+                mine = (row // rows) == hm
+                keep = torch.zeros((rows, -(-N // k_rows[i])), dtype=torch.bool, device="cuda")
+                keep[row[mine] % rows, ci[mine].long()] = True
+                keep = keep.repeat_interleave(k_rows[i], dim=1)[:, :N]
+            order = perms[i]
+            kk, vv, qq = k[b, h, order].double(), v[b, h, order].double(), q[b, h, order].double()
+            for n0 in range(0, N, 4096):
+                x = qq[n0:n0 + 4096] @ kk.T / math.sqrt(d)
+                x.masked_fill_(~keep[torch.arange(n0, n0 + x.shape[0], device="cuda") // q_rows[i]], -math.inf)
+                x -= x.amax(1, keepdim=True)
+                x.exp_()
+                out[b, h, order[n0:n0 + 4096]] = (x @ vv) / x.sum(1, keepdim=True)
+    return out
+
+
+def _linear64(s):
+    """ReLU linear attention in 64 bits, [B, H, N, d]; with a rotation table, rotated in the numerator alone."""
+    out = torch.empty(s["q"].shape, dtype=torch.float64, device="cuda")
+    for b in range(out.shape[0]):
+        for h in range(out.shape[1]):
+            q, k, v = (s[name][b, h].double() for name in ("q", "k", "v"))
+            q, k = q.clamp_min(0), k.clamp_min(0)
+            den = q @ k.sum(0) + EPS
+            if "rope" in s:
+                c, sn = s["rope"][..., 0].double(), s["rope"][..., 1].double()
+                q, k = (torch.stack((c * x[:, 0::2] - sn * x[:, 1::2], sn * x[:, 0::2] + c * x[:, 1::2]), 2).flatten(1)
+                        for x in (q, k))
+            out[b, h] = (q @ (k.T @ v)) / den[:, None]
+    return out
+
+
+def exact(case, seed):
+    """What run() returns for these inputs (lists and rotation table among them), in 64 bits."""
+    s = prepare(case, seed)
+    B, H, d, N, Bq, nQb, nKb = _sizes(case)
+    path, dev = case["path"], "cuda"
+    if path == "linear":
+        return _linear64(s)
+    tokens = torch.arange(N, device=dev)
+    perms, q_rows, k_rows = [tokens], [Bq], [64]
+    if path == "topk":
+        def means(x, block):
+            x = torch.nn.functional.pad(x.double(), (0, 0, 0, -N % block)).view(B * H, -1, block, d).sum(2)
+            size = torch.clamp(N - torch.arange(x.shape[1], device=dev) * block, max=block)
+            return x / size[:, None]
+        score = means(s["q"], Bq) @ means(s["k"], 64).transpose(1, 2)
+        kept = score.argsort(dim=2, descending=True, stable=True)[..., :_topk(nKb)].sort(dim=2).values
+        lists = (torch.arange(B * H * nQb + 1, device=dev) * kept.shape[2], kept.flatten(), B * H)
+    else:
+        lists = (s["rp"], s["ci"], s["Hm"])
+    if path == "stswa":
+        T = case["T"]
+        perms.append(tokens.view(T, -1).T.flatten())             # m = s * T + t
+        q_rows.append(128 // T * T)
+        k_rows.append(64 // T * T)
+    o_s = _attention64(s, perms, q_rows, k_rows, lists)
+    o_l = _linear64(s)
+    sb = s["sb"].double().view(B, 1, 1, 1)
+    if path == "proj":
+        return o_s + sb * torch.einsum("hca,bhna->bhnc", s["blocks"].double(), o_l)
+    if path == "fullproj":
+        mixed = o_l.transpose(1, 2).reshape(B, N, H * d) @ s["weight"].double().T + s["bias"].double()
+        return o_s + sb * mixed.view(B, N, H, d).transpose(1, 2)
+    lam = s["lam"].double().view(1, H, 1, 1)
+    if path == "layer":
+        scale = torch.stack([torch.sigmoid(x.double() @ s["w"].double()).mean() for x in s["x"]])
+        kept = torch.where(scale < TAU, 0.0, scale).view(B, 1, 1, 1)
+        return scale, o_s + kept * lam * o_l
+    out = o_s + sb * lam * o_l
+    return (None, None, out) if path == "topk" else out
+
+
 def work(case):
     """Q, K, V (and X, the weights, the table) read once, the output written once; the products of the kept
     blocks (ragged blocks at their valid size), of the linear state and of its application."""
