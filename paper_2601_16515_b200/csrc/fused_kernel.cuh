@@ -132,10 +132,10 @@ salad_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     const uint32_t s_base = smem_u32(smem);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    // The work order comes from the first kernel of the call.  Without a linear branch that is the kernel
-    // before this one.  With one, the state kernels lie between, and this kernel does not wait for them
-    // here: it runs beside them (each of their CTAs has passed its own wait for the first kernel before
-    // a CTA of this one is placed) and waits only where it first touches the state, in the epilogue.
+    // The work order (and the verdict on the lists) comes from the first kernel of the call.  Without a linear
+    // branch that is the kernel before this one.  With one, it is the state kernel, whose ordering CTAs let the kernels
+    // after it go only when their results are in the L2; this kernel reads them from there and does not wait for
+    // the state kernels here: it runs beside them and waits only where it first touches the state, in the epilogue.
     if ((p.mode & MODE_LINEAR) == 0 || p.wait_at_top) grid_dependency_wait();
     grid_launch_dependents();
 
@@ -146,7 +146,7 @@ salad_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
     const int rank = blockIdx.x % p.nQb, bh = blockIdx.x / p.nQb;
     const int h = bh % p.H, b = bh / p.H;
     const int hm = (p.Hm == 1) ? 0 : (p.Hm == p.H ? h : bh);   // one mask, one per head, or one per (batch, head)
-    const int qb = p.order ? __ldg(p.order + size_t(hm) * p.nQb + rank) : rank;
+    const int qb = p.order ? __ldcg(p.order + size_t(hm) * p.nQb + rank) : rank;
     // temporal head: blocks of spatial positions, fetched through the 4-D maps
     const bool perm = p.th.T > 0 && ((p.th.flags[h >> 5] >> (h & 31)) & 1u);
     const int q_rows = perm ? p.th.kq * p.th.T : p.Bq;          // rows of the 128-row tile that hold queries

@@ -27,6 +27,7 @@
 // the K tile in the stage; those accumulator rows are ignored.
 #pragma once
 #include "ptx.cuh"
+#include "work_order_kernel.cuh"
 
 namespace salad {
 
@@ -52,7 +53,11 @@ struct StateParams {
     float* z_part;        // [BH][chunks][D]
     int32_t* ws_status;
     int32_t* user_status;
-    int clear_status;         // 1: this kernel is the first of its call and clears the status words itself
+    int clear_status;         // 1: this call's status words are cleared here (by the first state CTA, or with the ordering)
+    // calls with a sparse branch: the first order_ctas CTAs (one per mask head) order the kept lists
+    const int32_t* row_ptr;
+    int32_t* order;
+    int order_ctas, nQb;
     const float* dyn_scale;   // [B] or null: with drop_tau, batch items whose scale is below it are skipped
     float drop_tau;
     int H;
@@ -78,26 +83,32 @@ salad_linear_state_kernel(const __grid_constant__ CUtensorMap map_k, const __gri
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     const uint32_t s_base = smem_u32(smem);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int chunk = blockIdx.x, bh = blockIdx.y;
+    if (int(blockIdx.x) < p.order_ctas) {
+        // Ordering CTA.  Its results are written, and pushed to the L2, before it lets the kernels after this one go:
+        // the attention kernel reads them (from the L2) without a wait of its own.
+        grid_dependency_wait();        // (the list validator, if there is one)
+        order_lists<C::THREADS>(p.row_ptr, p.nQb, p.order_ctas, blockIdx.x, p.order, p.ws_status, p.user_status,
+                                p.clear_status, reinterpret_cast<int*>(smem));
+        __threadfence();
+        __syncthreads();
+        grid_launch_dependents();
+        return;
+    }
+    const int chunk = (blockIdx.x - p.order_ctas) % p.chunks, bh = (blockIdx.x - p.order_ctas) / p.chunks;
     // First kernel of a linear-only call (an ordinary launch, so everything before it in the stream is done):
     // its first CTA, which is in the first wave, clears the status words at once; a CTA sets them only after
-    // a bounded wait of a second has run out.  No CTA of this kernel reads them (there is no earlier kernel of
-    // the call whose failure it would have to honour).
-    if (p.clear_status && chunk == 0 && bh == 0 && tid == 0) {
+    // a bounded wait of a second has run out.  No state CTA reads them.
+    if (p.order_ctas == 0 && p.clear_status && chunk == 0 && bh == 0 && tid == 0) {
         p.ws_status[0] = 0; p.ws_status[1] = 0;
         if (p.user_status) *p.user_status = 0;
     }
-    if (branch_dropped(p.dyn_scale, p.drop_tau, bh / p.H)) {           // whole CTA, before any allocation
-        grid_dependency_wait();        // an exit releases the kernels after this one: not before the kernel before it is done
-        return;
-    }
+    if (branch_dropped(p.dyn_scale, p.drop_tau, bh / p.H)) return;     // whole CTA, before any allocation
     const int kb0 = chunk * p.blocks_per_chunk;
     const int kb1 = min(p.nKb, kb0 + p.blocks_per_chunk);
     const int nblk = max(0, kb1 - kb0);
 
-    // K and V are inputs of the call, not products of the kernel before this one in the stream: the
-    // producer thread starts the first loads at once, ahead of the set-up below and of the dependency
-    // wait (this kernel is launched so that it may begin while its predecessor still runs).
+    // K and V are inputs of the call, not products of the kernel before this one (the list validator, if any): the
+    // producer thread starts the first loads at once, ahead of the set-up below.
     auto load_stage = [&](int g) {
         const int s = g % C::STAGES;
         const uint32_t bar = smem_u32(&full[s]);
@@ -127,15 +138,9 @@ salad_linear_state_kernel(const __grid_constant__ CUtensorMap map_k, const __gri
         reinterpret_cast<uint32_t*>(smem + C::OFF_ONES)[i] = 0x3F803F80u;
     fence_proxy_async_smem();
     if (warp == 1) { tmem_alloc(smem_u32(&tmem_base_slot), C::TMEM_COLS); tmem_relinquish(); }
-    // Invariant the attention kernel of a fused call relies on: this kernel releases its dependents only AFTER
-    // its own dependency wait (here, and in the early exit of a dropped batch item above).  The attention
-    // kernel reads the launch order and the status word, both written by the first kernel of the call,
-    // without a wait of its own; it can be placed only once every CTA of the finalize kernel has started,
-    // which needs every CTA of this kernel to have got here, i.e. past the wait for that first kernel.
-    grid_dependency_wait();            // the status word is cleared by the kernel before
+    grid_dependency_wait();            // (nothing to wait for in an ordinary launch)
     grid_launch_dependents();
-    // 2: the first kernel of the call has reported a failure (a rejected mask): do nothing, report nothing
-    if (tid == 0) abort_flag = (!p.clear_status && *reinterpret_cast<volatile int32_t*>(p.ws_status) != 0) ? 2 : 0;
+    if (tid == 0) abort_flag = 0;
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();

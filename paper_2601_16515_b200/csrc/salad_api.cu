@@ -256,7 +256,7 @@ int list_rows_of(const Problem& P) {
 }
 
 template <int D>
-int launch_state(const Problem& P, const Workspace& w, const DeviceInfo& dev) {
+int launch_state(const Problem& P, const Workspace& w, const DeviceInfo& dev, int list_rows, bool validated) {
     const int BH = P.B * P.H;
     const int nKb = (P.N + 63) / 64;
     int chunks = dev.sms / BH;          // one CTA per SM (its stage ring takes most of the shared memory)
@@ -281,14 +281,19 @@ int launch_state(const Problem& P, const Workspace& w, const DeviceInfo& dev) {
     // Fused calls: the short-ring variant, which shares its SM with a CTA of the attention kernel.  With a
     // rotation table the state pass keeps the SM to itself (full ring, eight ReLU warps): sharing the SM with
     // the attention kernel was measured no faster.
-    // In a linear-only call this is the first kernel: an ordinary launch (it must not start before the call
-    // before it has ended), which clears the status words itself.
-    sp.clear_status = (P.mode & MODE_SPARSE) ? 0 : 1;
+    // The first kernel of its call (unless the list validator runs before it): an ordinary launch, which must not
+    // start before the call before it has ended.  Calls with a sparse branch: the CTAs that order the kept lists come
+    // first in the grid, so that they start first.
+    sp.clear_status = validated ? 0 : 1;
+    sp.row_ptr = P.row_ptr; sp.order = reinterpret_cast<int32_t*>(ws + w.off_order);
+    sp.nQb = list_rows;
+    sp.order_ctas = (P.mode & MODE_SPARSE) ? P.Hm : 0;
     auto launch = [&](auto kernel, int threads, int smem) {
-        if (sp.clear_status)
-            kernel<<<dim3(chunks, BH), dim3(threads), size_t(smem), P.stream>>>(mk, mv, mr, sp);
-        else
-            launch_dependent(kernel, dim3(chunks, BH), dim3(threads), size_t(smem), P.stream, mk, mv, mr, sp);
+        const dim3 grid(unsigned(sp.order_ctas + int64_t(chunks) * BH));
+        SALAD_LOGF("salad_linear_state_kernel grid %d + %d x %d%s", sp.order_ctas, chunks, BH,
+                   validated ? " after csr_validate_kernel" : "");
+        if (!validated) kernel<<<grid, dim3(threads), size_t(smem), P.stream>>>(mk, mv, mr, sp);
+        else launch_dependent(kernel, grid, dim3(threads), size_t(smem), P.stream, mk, mv, mr, sp);
     };
     if (P.rope)
         launch(salad_linear_state_kernel<D, false, true>, StateCfg<D, false, true>::THREADS,
@@ -430,12 +435,11 @@ int run(const Problem& P) {
     if (rc != SALAD_OK) return rc;
     const Workspace w = carve(P.B, P.H, P.N, P.d, P.Bq, list_rows_of(P));
     uint8_t* ws = static_cast<uint8_t*>(P.ws);
+    const int nQb = list_rows_of(P) > 0 ? list_rows_of(P) : (P.N + P.Bq - 1) / P.Bq;
+    const bool state = (P.mode & MODE_LINEAR) && !P.prepared;
+    bool validated = false;
     if (P.mode & MODE_SPARSE) {
-        // first kernel of the call: longest work items first (the mask is an input of every call,
-        // so is its order); it also clears the status words
-        const int nQb = list_rows_of(P) > 0 ? list_rows_of(P) : (P.N + P.Bq - 1) / P.Bq;
         int32_t* ws_status = reinterpret_cast<int32_t*>(ws + w.off_status);
-        int clear_status = 1;
         if (g_validate_capacity > 0) {
             // opt-in check of the lists (salad_set_mask_validation): it owns the status words of this call
             int nkb_bound = (P.N + 63) / 64;
@@ -444,16 +448,20 @@ int run(const Problem& P) {
             rc = launch_csr_validate(P.row_ptr, P.col_idx, g_validate_capacity, int64_t(P.Hm) * nQb, nkb_bound,
                                      ws_status, P.d_status, P.stream);
             if (rc != SALAD_OK) return rc;
-            clear_status = 0;
+            validated = true;
         }
-        SALAD_LOGF("work_order_kernel grid %d block 1024 (nQb %d)%s", P.Hm, nQb, clear_status ? "" : " after csr_validate_kernel");
-        work_order_kernel<<<P.Hm, 1024, 0, P.stream>>>(P.row_ptr, nQb, P.Hm,
-                                                      reinterpret_cast<int32_t*>(ws + w.off_order), ws_status,
-                                                      P.d_status, clear_status);
-        if (check_launch() != SALAD_OK) return SALAD_ERR_CUDA;
+        if (!state) {
+            // first kernel of a call without a state pass: longest work items first (the mask is an input of
+            // every call, so is its order); it also clears the status words
+            SALAD_LOGF("work_order_kernel grid %d block 1024 (nQb %d)%s", P.Hm, nQb, validated ? " after csr_validate_kernel" : "");
+            work_order_kernel<<<P.Hm, 1024, 0, P.stream>>>(P.row_ptr, nQb, P.Hm,
+                                                          reinterpret_cast<int32_t*>(ws + w.off_order), ws_status,
+                                                          P.d_status, validated ? 0 : 1);
+            if (check_launch() != SALAD_OK) return SALAD_ERR_CUDA;
+        }
     }
-    if ((P.mode & MODE_LINEAR) && !P.prepared) {
-        rc = (P.d == 128) ? launch_state<128>(P, w, dev) : launch_state<64>(P, w, dev);
+    if (state) {
+        rc = (P.d == 128) ? launch_state<128>(P, w, dev, nQb, validated) : launch_state<64>(P, w, dev, nQb, validated);
         if (rc != SALAD_OK) return rc;
     }
     if (P.state_only) return SALAD_OK;
@@ -1030,7 +1038,7 @@ SALAD_EXPORT int salad_linear_attn_fwd_noalloc(const void* q, const void* k, con
     P.ws = scratch; P.ws_bytes = kNoAllocBytes; P.d_status = d_status;
     P.stream = static_cast<cudaStream_t>(stream);
     // (the array keeps the last call's contents: the state kernel, first of the call, clears the status words)
-    rc = (d == 128) ? launch_state<128>(P, w, dev) : launch_state<64>(P, w, dev);
+    rc = (d == 128) ? launch_state<128>(P, w, dev, 0, false) : launch_state<64>(P, w, dev, 0, false);
     if (rc != SALAD_OK) return rc;
     return (d == 128) ? launch_apply<128>(P, w, dev) : launch_apply<64>(P, w, dev);
 }
