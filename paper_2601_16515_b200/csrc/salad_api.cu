@@ -255,8 +255,15 @@ int list_rows_of(const Problem& P) {
     return (P.st_T > 0 && stswa_geometry(P.st_T, P.st_Hs, P.st_Ws, &sg)) ? sg.rows : 0;
 }
 
+// The maps of K and V in 64-token boxes, which the state kernel and the attention kernel share.
+struct KvMaps { CUtensorMap k, v; };
+bool make_kv_maps(const Problem& P, KvMaps* m) {
+    return make_tmap_bf16_3d(&m->k, P.k, P.d, P.N, int64_t(P.B) * P.H, 64) &&
+           make_tmap_bf16_3d(&m->v, P.v, P.d, P.N, int64_t(P.B) * P.H, 64);
+}
+
 template <int D>
-int launch_state(const Problem& P, const Workspace& w, const DeviceInfo& dev, int list_rows, bool validated) {
+int launch_state(const Problem& P, const KvMaps& kv, const Workspace& w, const DeviceInfo& dev, int list_rows, bool validated) {
     const int BH = P.B * P.H;
     const int nKb = (P.N + 63) / 64;
     int chunks = dev.sms / BH;          // one CTA per SM (its stage ring takes most of the shared memory)
@@ -265,10 +272,7 @@ int launch_state(const Problem& P, const Workspace& w, const DeviceInfo& dev, in
     if (int64_t(chunks) * BH > w.slots) chunks = w.slots / BH;
     const int bpc = (nKb + chunks - 1) / chunks;
     uint8_t* ws = static_cast<uint8_t*>(P.ws);
-    CUtensorMap mk, mv;
-    if (!make_tmap_bf16_3d(&mk, P.k, D, P.N, BH, 64) || !make_tmap_bf16_3d(&mv, P.v, D, P.N, BH, 64))
-        return SALAD_ERR_CUDA;
-    CUtensorMap mr = mk;          // unused without a rotation table
+    CUtensorMap mr = kv.k;          // unused without a rotation table
     if (P.rope && !make_tmap_f16_rows(&mr, P.rope, D, P.N, 64)) return SALAD_ERR_CUDA;
     StateParams sp;
     sp.N = P.N; sp.nKb = nKb; sp.chunks = chunks; sp.blocks_per_chunk = bpc;
@@ -292,8 +296,8 @@ int launch_state(const Problem& P, const Workspace& w, const DeviceInfo& dev, in
         const dim3 grid(unsigned(sp.order_ctas + int64_t(chunks) * BH));
         SALAD_LOGF("salad_linear_state_kernel grid %d + %d x %d%s", sp.order_ctas, chunks, BH,
                    validated ? " after csr_validate_kernel" : "");
-        if (!validated) kernel<<<grid, dim3(threads), size_t(smem), P.stream>>>(mk, mv, mr, sp);
-        else launch_dependent(kernel, grid, dim3(threads), size_t(smem), P.stream, mk, mv, mr, sp);
+        if (!validated) kernel<<<grid, dim3(threads), size_t(smem), P.stream>>>(kv.k, kv.v, mr, sp);
+        else launch_dependent(kernel, grid, dim3(threads), size_t(smem), P.stream, kv.k, kv.v, mr, sp);
     };
     if (P.rope)
         launch(salad_linear_state_kernel<D, false, true>, StateCfg<D, false, true>::THREADS,
@@ -322,12 +326,12 @@ int launch_state(const Problem& P, const Workspace& w, const DeviceInfo& dev, in
 }
 
 template <int D>
-int launch_fused(const Problem& P, const Workspace& w, const DeviceInfo& dev) {
+int launch_fused(const Problem& P, const KvMaps& kv, const Workspace& w, const DeviceInfo& dev) {
     const int BH = P.B * P.H;
     uint8_t* ws = static_cast<uint8_t*>(P.ws);
-    CUtensorMap mq, mk, mv, mo, ms;
-    if (!make_tmap_bf16_3d(&mq, P.q, D, P.N, BH, P.Bq) || !make_tmap_bf16_3d(&mk, P.k, D, P.N, BH, 64) ||
-        !make_tmap_bf16_3d(&mv, P.v, D, P.N, BH, 64) || !make_tmap_bf16_3d(&mo, P.o, D, P.N, BH, P.Bq) ||
+    const CUtensorMap &mk = kv.k, &mv = kv.v;
+    CUtensorMap mq, mo, ms;
+    if (!make_tmap_bf16_3d(&mq, P.q, D, P.N, BH, P.Bq) || !make_tmap_bf16_3d(&mo, P.o, D, P.N, BH, P.Bq) ||
         !make_tmap_bf16_3d(&ms, ws + w.off_kvt, D, D, BH, D))
         return SALAD_ERR_CUDA;
     FusedParams fp;
@@ -460,15 +464,17 @@ int run(const Problem& P) {
             if (check_launch() != SALAD_OK) return SALAD_ERR_CUDA;
         }
     }
+    KvMaps kv;
+    if (!make_kv_maps(P, &kv)) return SALAD_ERR_CUDA;
     if (state) {
-        rc = (P.d == 128) ? launch_state<128>(P, w, dev, nQb, validated) : launch_state<64>(P, w, dev, nQb, validated);
+        rc = (P.d == 128) ? launch_state<128>(P, kv, w, dev, nQb, validated) : launch_state<64>(P, kv, w, dev, nQb, validated);
         if (rc != SALAD_OK) return rc;
     }
     if (P.state_only) return SALAD_OK;
     // linear-only calls: the stand-alone apply kernel
     if (P.mode == MODE_LINEAR)
         return (P.d == 128) ? launch_apply<128>(P, w, dev) : launch_apply<64>(P, w, dev);
-    return (P.d == 128) ? launch_fused<128>(P, w, dev) : launch_fused<64>(P, w, dev);
+    return (P.d == 128) ? launch_fused<128>(P, kv, w, dev) : launch_fused<64>(P, kv, w, dev);
 }
 
 // ---------------------------------------------------------------------------------------
@@ -1038,7 +1044,9 @@ SALAD_EXPORT int salad_linear_attn_fwd_noalloc(const void* q, const void* k, con
     P.ws = scratch; P.ws_bytes = kNoAllocBytes; P.d_status = d_status;
     P.stream = static_cast<cudaStream_t>(stream);
     // (the array keeps the last call's contents: the state kernel, first of the call, clears the status words)
-    rc = (d == 128) ? launch_state<128>(P, w, dev, 0, false) : launch_state<64>(P, w, dev, 0, false);
+    KvMaps kv;
+    if (!make_kv_maps(P, &kv)) return SALAD_ERR_CUDA;
+    rc = (d == 128) ? launch_state<128>(P, kv, w, dev, 0, false) : launch_state<64>(P, kv, w, dev, 0, false);
     if (rc != SALAD_OK) return rc;
     return (d == 128) ? launch_apply<128>(P, w, dev) : launch_apply<64>(P, w, dev);
 }

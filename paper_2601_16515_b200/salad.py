@@ -118,13 +118,30 @@ def _check(rc: int, where: str):
 
 
 def _ptr(t: Optional[torch.Tensor]):
-    return None if t is None else ctypes.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
-def _stream(stream) -> ctypes.c_void_p:
+# A call is issued on the device of its tensors, on that device's current stream unless the caller names one.  The
+# handles come straight from torch's C layer: the Python device context and Stream objects cost 6 us a call, more than
+# the launches of the smallest calls.
+_current_device = torch._C._cuda_getDevice
+_current_raw_stream = torch._C._cuda_getCurrentRawStream
+
+
+def _call(name: str, anchor: torch.Tensor, stream, *args):
+    """One library call whose last argument is the stream, on the device of `anchor`."""
+    index = anchor.get_device()
     if stream is None:
-        stream = torch.cuda.current_stream()
-    return ctypes.c_void_p(stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream))
+        stream = _current_raw_stream(index)
+    else:
+        stream = stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
+    if _current_device() == index:
+        rc = getattr(_lib, name)(*args, stream)
+    else:
+        with torch.cuda.device(index):
+            rc = getattr(_lib, name)(*args, stream)
+    if rc != SALAD_OK:
+        raise SaladError(rc, name)
 
 
 def _bf16_4d(name: str, t: torch.Tensor):
@@ -154,12 +171,10 @@ def salad_mask_build(T: int, Hs: int, Ws: int, Bq: int, Bk: int,
     nQb = -(-N // Bq)
     row_ptr = torch.empty(Hm * nQb + 1, dtype=torch.int32, device=device)
     nnz = ctypes.c_int64(-1)
-    with torch.cuda.device(row_ptr.device):
-        _check(_lib.salad_mask_build(T, Hs, Ws, Bq, Bk, Hm, h_win, _ptr(row_ptr), None, 0,
-                                     ctypes.byref(nnz), _stream(stream)), "salad_mask_build")
-        col_idx = torch.empty(max(1, nnz.value), dtype=torch.int32, device=device)
-        _check(_lib.salad_mask_build(T, Hs, Ws, Bq, Bk, Hm, h_win, _ptr(row_ptr), _ptr(col_idx),
-                                     col_idx.numel(), ctypes.byref(nnz), _stream(stream)), "salad_mask_build")
+    _call("salad_mask_build", row_ptr, stream, T, Hs, Ws, Bq, Bk, Hm, h_win, _ptr(row_ptr), None, 0, ctypes.byref(nnz))
+    col_idx = torch.empty(max(1, nnz.value), dtype=torch.int32, device=device)
+    _call("salad_mask_build", row_ptr, stream, T, Hs, Ws, Bq, Bk, Hm, h_win, _ptr(row_ptr), _ptr(col_idx),
+          col_idx.numel(), ctypes.byref(nnz))
     return row_ptr, col_idx[:nnz.value]
 
 
@@ -169,9 +184,8 @@ def salad_csr_validate(row_ptr, col_idx, nKb: int, status=None, stream=None):
     _i32("row_ptr", row_ptr); _i32("col_idx", col_idx)
     if status is None:
         status = torch.zeros(1, dtype=torch.int32, device=row_ptr.device)
-    with torch.cuda.device(row_ptr.device):
-        _check(_lib.salad_csr_validate(_ptr(row_ptr), _ptr(col_idx), col_idx.numel(), row_ptr.numel() - 1, int(nKb),
-                                       _ptr(status), _stream(stream)), "salad_csr_validate")
+    _call("salad_csr_validate", row_ptr, stream, _ptr(row_ptr), _ptr(col_idx), col_idx.numel(), row_ptr.numel() - 1,
+          int(nKb), _ptr(status))
     return status
 
 
@@ -217,11 +231,8 @@ def salad_sparse_attn_fwd(q, k, v, row_ptr, col_idx, Hm: int, Bq: int = 128, Bk:
     _i32("row_ptr", row_ptr); _i32("col_idx", col_idx)
     if out is None:
         out = torch.empty_like(q)
-    with torch.cuda.device(q.device):
-        _check(_lib.salad_sparse_attn_fwd(_ptr(q), _ptr(k), _ptr(v), _ptr(out), _ptr(lse), B, H, N, d, Bq, Bk,
-                                          _ptr(row_ptr), _ptr(col_idx), Hm, float(softmax_scale),
-                                          _ptr(workspace), workspace.numel(), _ptr(status), _stream(stream)),
-               "salad_sparse_attn_fwd")
+    _call("salad_sparse_attn_fwd", q, stream, _ptr(q), _ptr(k), _ptr(v), _ptr(out), _ptr(lse), B, H, N, d, Bq, Bk,
+          _ptr(row_ptr), _ptr(col_idx), Hm, float(softmax_scale), _ptr(workspace), workspace.numel(), _ptr(status))
     return out
 
 
@@ -232,10 +243,8 @@ def salad_linear_attn_fwd(q, k, v, eps: float = 1e-6, out=None, kv_out=None, z_o
     B, H, N, d, workspace = _common(q, k, v, 128, 64, workspace)
     if out is None:
         out = torch.empty_like(q)
-    with torch.cuda.device(q.device):
-        _check(_lib.salad_linear_attn_fwd(_ptr(q), _ptr(k), _ptr(v), _ptr(out), _ptr(kv_out), _ptr(z_out),
-                                          B, H, N, d, float(eps), _ptr(workspace), workspace.numel(),
-                                          _ptr(status), _stream(stream)), "salad_linear_attn_fwd")
+    _call("salad_linear_attn_fwd", q, stream, _ptr(q), _ptr(k), _ptr(v), _ptr(out), _ptr(kv_out), _ptr(z_out), B, H, N,
+          d, float(eps), _ptr(workspace), workspace.numel(), _ptr(status))
     return out
 
 
@@ -252,9 +261,7 @@ def salad_rope3d_table_build(T: int, Hs: int, Ws: int, d: int, base: float = 100
     if out is None:
         out = torch.empty((T * Hs * Ws, d // 2, 2), dtype=torch.float16, device=device or "cuda")
     _rope_table(out, T * Hs * Ws, d)
-    with torch.cuda.device(out.device):
-        _check(_lib.salad_rope3d_table_build(T, Hs, Ws, d, float(base), _ptr(out), _stream(stream)),
-               "salad_rope3d_table_build")
+    _call("salad_rope3d_table_build", out, stream, T, Hs, Ws, d, float(base), _ptr(out))
     return out
 
 
@@ -266,11 +273,8 @@ def salad_linear_attn_rope_fwd(q, k, v, rope, eps: float = 1e-6, out=None, kv_ou
     _rope_table(rope, N, d)
     if out is None:
         out = torch.empty_like(q)
-    with torch.cuda.device(q.device):
-        _check(_lib.salad_linear_attn_rope_fwd(_ptr(q), _ptr(k), _ptr(v), _ptr(out), _ptr(kv_out), _ptr(z_out),
-                                               B, H, N, d, _ptr(rope), float(eps), _ptr(workspace),
-                                               workspace.numel(), _ptr(status), _stream(stream)),
-               "salad_linear_attn_rope_fwd")
+    _call("salad_linear_attn_rope_fwd", q, stream, _ptr(q), _ptr(k), _ptr(v), _ptr(out), _ptr(kv_out), _ptr(z_out), B,
+          H, N, d, _ptr(rope), float(eps), _ptr(workspace), workspace.numel(), _ptr(status))
     return out
 
 
@@ -287,12 +291,9 @@ def salad_fused_rope_fwd(q, k, v, row_ptr, col_idx, Hm: int, static_scale, dyn_s
     if out is None:
         out = torch.empty_like(q)
     tau = float("-inf") if drop_tau is None else float(drop_tau)
-    with torch.cuda.device(q.device):
-        _check(_lib.salad_fused_rope_fwd(_ptr(q), _ptr(k), _ptr(v), _ptr(out), B, H, N, d, Bq, Bk,
-                                         _ptr(row_ptr), _ptr(col_idx), Hm, _ptr(static_scale), _ptr(dyn_scale),
-                                         _ptr(rope), tau, float(softmax_scale), float(eps), _ptr(workspace),
-                                         workspace.numel(), _ptr(status), _stream(stream)),
-               "salad_fused_rope_fwd")
+    _call("salad_fused_rope_fwd", q, stream, _ptr(q), _ptr(k), _ptr(v), _ptr(out), B, H, N, d, Bq, Bk, _ptr(row_ptr),
+          _ptr(col_idx), Hm, _ptr(static_scale), _ptr(dyn_scale), _ptr(rope), tau, float(softmax_scale), float(eps),
+          _ptr(workspace), workspace.numel(), _ptr(status))
     return out
 
 
@@ -304,9 +305,8 @@ def salad_linear_state_fwd(k, v, workspace, kv_out=None, z_out=None, status=None
     if k.shape != v.shape:
         raise ValueError("k and v must have the same shape")
     B, H, N, d = k.shape
-    with torch.cuda.device(k.device):
-        _check(_lib.salad_linear_state_fwd(_ptr(k), _ptr(v), _ptr(kv_out), _ptr(z_out), B, H, N, d, _ptr(workspace),
-                                           workspace.numel(), _ptr(status), _stream(stream)), "salad_linear_state_fwd")
+    _call("salad_linear_state_fwd", k, stream, _ptr(k), _ptr(v), _ptr(kv_out), _ptr(z_out), B, H, N, d, _ptr(workspace),
+          workspace.numel(), _ptr(status))
     return workspace
 
 
@@ -322,11 +322,9 @@ def salad_fused_prepared_fwd(q, k, v, row_ptr, col_idx, Hm: int, static_scale, d
     if out is None:
         out = torch.empty_like(q)
     tau = float("-inf") if drop_tau is None else float(drop_tau)
-    with torch.cuda.device(q.device):
-        _check(_lib.salad_fused_prepared_fwd(_ptr(q), _ptr(k), _ptr(v), _ptr(out), B, H, N, d, Bq, Bk,
-                                             _ptr(row_ptr), _ptr(col_idx), Hm, _ptr(static_scale), _ptr(dyn_scale), tau,
-                                             float(softmax_scale), float(eps), _ptr(workspace), workspace.numel(),
-                                             _ptr(status), _stream(stream)), "salad_fused_prepared_fwd")
+    _call("salad_fused_prepared_fwd", q, stream, _ptr(q), _ptr(k), _ptr(v), _ptr(out), B, H, N, d, Bq, Bk,
+          _ptr(row_ptr), _ptr(col_idx), Hm, _ptr(static_scale), _ptr(dyn_scale), tau, float(softmax_scale), float(eps),
+          _ptr(workspace), workspace.numel(), _ptr(status))
     return out
 
 
@@ -345,11 +343,9 @@ def salad_fused_proj_fwd(q, k, v, row_ptr, col_idx, Hm: int, proj_blocks, dyn_sc
     if out is None:
         out = torch.empty_like(q)
     tau = float("-inf") if drop_tau is None else float(drop_tau)
-    with torch.cuda.device(q.device):
-        _check(_lib.salad_fused_proj_fwd(_ptr(q), _ptr(k), _ptr(v), _ptr(out), B, H, N, d, Bq, Bk,
-                                         _ptr(row_ptr), _ptr(col_idx), Hm, _ptr(proj_blocks), _ptr(dyn_scale), tau,
-                                         float(softmax_scale), float(eps), _ptr(workspace), workspace.numel(),
-                                         _ptr(status), _stream(stream)), "salad_fused_proj_fwd")
+    _call("salad_fused_proj_fwd", q, stream, _ptr(q), _ptr(k), _ptr(v), _ptr(out), B, H, N, d, Bq, Bk, _ptr(row_ptr),
+          _ptr(col_idx), Hm, _ptr(proj_blocks), _ptr(dyn_scale), tau, float(softmax_scale), float(eps), _ptr(workspace),
+          workspace.numel(), _ptr(status))
     return out
 
 
@@ -370,10 +366,8 @@ def salad_linear_attn_fwd_noalloc(q, k, v, eps: float = 1e-6, out=None, kv_out=N
     B, H, N, d = q.shape
     if out is None:
         out = torch.empty_like(q)
-    with torch.cuda.device(q.device):
-        _check(_lib.salad_linear_attn_fwd_noalloc(_ptr(q), _ptr(k), _ptr(v), _ptr(out), _ptr(kv_out), _ptr(z_out),
-                                                  B, H, N, d, float(eps), _ptr(status), _stream(stream)),
-               "salad_linear_attn_fwd_noalloc")
+    _call("salad_linear_attn_fwd_noalloc", q, stream, _ptr(q), _ptr(k), _ptr(v), _ptr(out), _ptr(kv_out), _ptr(z_out),
+          B, H, N, d, float(eps), _ptr(status))
     return out
 
 
@@ -397,10 +391,8 @@ def salad_topk_mask_build(q, k, topk: int, Bq: int = 128, Bk: int = 64, row_ptr=
     if workspace is None:
         nbytes = int(_lib.salad_topk_workspace_bytes(B, H, N, d, Bq, Bk))
         workspace = torch.empty(max(nbytes, 256), dtype=torch.uint8, device=q.device)
-    with torch.cuda.device(q.device):
-        _check(_lib.salad_topk_mask_build(_ptr(q), _ptr(k), B, H, N, d, Bq, Bk, int(topk), _ptr(row_ptr),
-                                          _ptr(col_idx), col_idx.numel(), _ptr(workspace), workspace.numel(),
-                                          _stream(stream)), "salad_topk_mask_build")
+    _call("salad_topk_mask_build", q, stream, _ptr(q), _ptr(k), B, H, N, d, Bq, Bk, int(topk), _ptr(row_ptr),
+          _ptr(col_idx), col_idx.numel(), _ptr(workspace), workspace.numel())
     return row_ptr, col_idx[:rows * kk]
 
 
@@ -415,9 +407,7 @@ def salad_permute_tokens(x, grid, head_flags, inverse: bool = False, out=None, s
         raise ValueError("head_flags must have one entry per head")
     if out is None:
         out = torch.empty_like(x)
-    with torch.cuda.device(x.device):
-        _check(_lib.salad_permute_tokens(_ptr(x), _ptr(out), B, H, N, d, T, Hs, Ws, flags, int(bool(inverse)),
-                                         _stream(stream)), "salad_permute_tokens")
+    _call("salad_permute_tokens", x, stream, _ptr(x), _ptr(out), B, H, N, d, T, Hs, Ws, flags, int(bool(inverse)))
     return out
 
 
@@ -440,12 +430,11 @@ def salad_stswa_mask_build(grid, head_flags, windows, device="cuda", stream=None
     win = (ctypes.c_int32 * H)(*[int(w) for w in windows])
     row_ptr = torch.empty(H * rows + 1, dtype=torch.int32, device=device)
     nnz = ctypes.c_int64(-1)
-    with torch.cuda.device(row_ptr.device):
-        _check(_lib.salad_stswa_mask_build(T, Hs, Ws, H, flags, win, _ptr(row_ptr), None, 0, ctypes.byref(nnz),
-                                           _stream(stream)), "salad_stswa_mask_build")
-        col_idx = torch.empty(max(1, nnz.value), dtype=torch.int32, device=device)
-        _check(_lib.salad_stswa_mask_build(T, Hs, Ws, H, flags, win, _ptr(row_ptr), _ptr(col_idx), col_idx.numel(),
-                                           ctypes.byref(nnz), _stream(stream)), "salad_stswa_mask_build")
+    _call("salad_stswa_mask_build", row_ptr, stream, T, Hs, Ws, H, flags, win, _ptr(row_ptr), None, 0,
+          ctypes.byref(nnz))
+    col_idx = torch.empty(max(1, nnz.value), dtype=torch.int32, device=device)
+    _call("salad_stswa_mask_build", row_ptr, stream, T, Hs, Ws, H, flags, win, _ptr(row_ptr), _ptr(col_idx),
+          col_idx.numel(), ctypes.byref(nnz))
     return row_ptr, col_idx[:nnz.value]
 
 
@@ -475,11 +464,9 @@ def salad_fused_stswa_fwd(q, k, v, grid, head_flags, row_ptr, col_idx, static_sc
     if out is None:
         out = torch.empty_like(q)
     tau = float("-inf") if drop_tau is None else float(drop_tau)
-    with torch.cuda.device(q.device):
-        _check(_lib.salad_fused_stswa_fwd(_ptr(q), _ptr(k), _ptr(v), _ptr(out), B, H, N, d, T, Hs, Ws, flags,
-                                          _ptr(row_ptr), _ptr(col_idx), _ptr(static_scale), _ptr(dyn_scale), tau,
-                                          float(softmax_scale), float(eps), _ptr(workspace), workspace.numel(),
-                                          _ptr(status), _stream(stream)), "salad_fused_stswa_fwd")
+    _call("salad_fused_stswa_fwd", q, stream, _ptr(q), _ptr(k), _ptr(v), _ptr(out), B, H, N, d, T, Hs, Ws, flags,
+          _ptr(row_ptr), _ptr(col_idx), _ptr(static_scale), _ptr(dyn_scale), tau, float(softmax_scale), float(eps),
+          _ptr(workspace), workspace.numel(), _ptr(status))
     return out
 
 
@@ -497,9 +484,8 @@ def salad_proj_combine_fwd(o_s, o_l, w, dyn_scale=None, bias=None, out=None, sta
             raise ValueError(f"{name} must be a contiguous CUDA fp32 tensor with {n} elements")
     if out is None:
         out = torch.empty_like(o_s)
-    with torch.cuda.device(o_s.device):
-        _check(_lib.salad_proj_combine_fwd(_ptr(o_s), _ptr(o_l), _ptr(w), _ptr(bias), _ptr(dyn_scale), _ptr(out),
-                                           B, H, N, d, _ptr(status), _stream(stream)), "salad_proj_combine_fwd")
+    _call("salad_proj_combine_fwd", o_s, stream, _ptr(o_s), _ptr(o_l), _ptr(w), _ptr(bias), _ptr(dyn_scale), _ptr(out),
+          B, H, N, d, _ptr(status))
     return out
 
 
@@ -507,7 +493,7 @@ def salad_selftest_bounded_wait(stream=None):
     """Runs the bounded-wait self-test kernel; returns (status, waited_ns) device tensors."""
     status = torch.zeros(1, dtype=torch.int32, device="cuda")
     waited = torch.zeros(1, dtype=torch.int64, device="cuda")
-    _check(_lib.salad_selftest_bounded_wait(_ptr(status), _ptr(waited), _stream(stream)), "salad_selftest_bounded_wait")
+    _call("salad_selftest_bounded_wait", status, stream, _ptr(status), _ptr(waited))
     return status, waited
 
 
@@ -525,9 +511,8 @@ def salad_dynamic_scale(x, w, bias: float = 0.0, out=None, workspace=None, strea
         out = torch.empty(B, dtype=torch.float32, device=x.device)
     if workspace is None:
         workspace = torch.empty(DYN_SCALE_WS_BYTES, dtype=torch.uint8, device=x.device)
-    with torch.cuda.device(x.device):
-        _check(_lib.salad_dynamic_scale(_ptr(x), _ptr(w), float(bias), B, N, D, _ptr(out), _ptr(workspace),
-                                        workspace.numel(), _stream(stream)), "salad_dynamic_scale")
+    _call("salad_dynamic_scale", x, stream, _ptr(x), _ptr(w), float(bias), B, N, D, _ptr(out), _ptr(workspace),
+          workspace.numel())
     return out
 
 
@@ -543,16 +528,12 @@ def salad_fused_fwd(q, k, v, row_ptr, col_idx, Hm: int, static_scale, dyn_scale,
             raise ValueError(f"{name} must be a contiguous CUDA fp32 tensor with {n} elements")
     if out is None:
         out = torch.empty_like(q)
-    with torch.cuda.device(q.device):
-        if drop_tau is None:
-            _check(_lib.salad_fused_fwd(_ptr(q), _ptr(k), _ptr(v), _ptr(out), B, H, N, d, Bq, Bk,
-                                        _ptr(row_ptr), _ptr(col_idx), Hm, _ptr(static_scale), _ptr(dyn_scale),
-                                        float(softmax_scale), float(eps), _ptr(workspace), workspace.numel(),
-                                        _ptr(status), _stream(stream)), "salad_fused_fwd")
-        else:
-            _check(_lib.salad_fused_drop_fwd(_ptr(q), _ptr(k), _ptr(v), _ptr(out), B, H, N, d, Bq, Bk,
-                                             _ptr(row_ptr), _ptr(col_idx), Hm, _ptr(static_scale), _ptr(dyn_scale),
-                                             float(drop_tau), float(softmax_scale), float(eps), _ptr(workspace),
-                                             workspace.numel(), _ptr(status), _stream(stream)),
-                   "salad_fused_drop_fwd")
+    if drop_tau is None:
+        _call("salad_fused_fwd", q, stream, _ptr(q), _ptr(k), _ptr(v), _ptr(out), B, H, N, d, Bq, Bk, _ptr(row_ptr),
+              _ptr(col_idx), Hm, _ptr(static_scale), _ptr(dyn_scale), float(softmax_scale), float(eps), _ptr(workspace),
+              workspace.numel(), _ptr(status))
+    else:
+        _call("salad_fused_drop_fwd", q, stream, _ptr(q), _ptr(k), _ptr(v), _ptr(out), B, H, N, d, Bq, Bk,
+              _ptr(row_ptr), _ptr(col_idx), Hm, _ptr(static_scale), _ptr(dyn_scale), float(drop_tau),
+              float(softmax_scale), float(eps), _ptr(workspace), workspace.numel(), _ptr(status))
     return out
