@@ -11,9 +11,12 @@
 //   warps 2-5   apply ReLU to the K tile in place in shared memory (16-byte vectors), and at
 //               the end move the fp32 accumulator from TMEM to this chunk's partial in global
 //               memory
-// A second, tiny kernel adds the partials of a head in a fixed order (deterministic), and
+// Long sequences: a second, tiny kernel adds the partials of a head in a fixed order (deterministic), and
 // emits the fp32 state plus the bf16, transposed copy that the fused attention kernel
 // multiplies with ReLU(Q).
+// Up to eight chunks per head: the CTAs of a head are one cluster; every CTA leaves its partial in its own shared memory
+// and adds a slice of the rows over the cluster (distributed shared memory), also in chunk order.  No second launch and
+// no round trip of the partials: 10.2 -> 8.4 us for the state pass of 12 heads of 900 tokens, 41.7 -> 37.7 us at 32760.
 //
 // ROPE variant (linear branch with a rotary position embedding, Sec. 4.1): the ReLU warps rotate the
 // channel pairs of ReLU(K) before the MMA reads them, with the fp16 rotation rows (cosine, sine per
@@ -42,6 +45,9 @@ struct StateCfg {
     static constexpr int STAGES = ROPE ? ((D == 128) ? 4 : 8) : (OVERLAP ? 3 : ((D == 128) ? 6 : 8));
     static constexpr int OFF_ONES = STAGES * STAGE_BYTES;
     static constexpr int SMEM_BYTES = OFF_ONES + 2048 + 1024;
+    // this CTA's partial for the reduction of a cluster, over the stages (all of them idle by then): rows of D + 4 floats, then Z
+    static constexpr int KS = D + 4, OFF_ZP = D * KS * 4, OFF_ZS = OFF_ZP + D * 4;
+    static_assert(OFF_ZS + (ROPE ? 256 * CH * 32 : 0) <= OFF_ONES, "the partial fits over the stages");
     static constexpr int RELU_THREADS = ROPE ? 256 : 128;   // the rotation doubles the work per element
     static constexpr int THREADS = 64 + RELU_THREADS;
     static constexpr int TMEM_COLS = 256;
@@ -54,10 +60,14 @@ struct StateParams {
     int32_t* ws_status;
     int32_t* user_status;
     int clear_status;         // 1: this call's status words are cleared here (by the first state CTA, or with the ordering)
-    // calls with a sparse branch: the first order_ctas CTAs (one per mask head) order the kept lists
+    // calls with a sparse branch: the first order_ctas CTAs (one per mask head, in whole clusters) order the kept lists
     const int32_t* row_ptr;
     int32_t* order;
-    int order_ctas, nQb;
+    int order_ctas, Hm, nQb;
+    // reduce: the CTAs of a head are one cluster, add their partials through shared memory and write the state themselves
+    int reduce;
+    float *kv_out, *z_ws, *z_out;
+    __nv_bfloat16* kvt;
     const float* dyn_scale;   // [B] or null: with drop_tau, batch items whose scale is below it are skipped
     float drop_tau;
     int H;
@@ -86,11 +96,13 @@ salad_linear_state_kernel(const __grid_constant__ CUtensorMap map_k, const __gri
     if (int(blockIdx.x) < p.order_ctas) {
         // Ordering CTA.  Its results are written, and pushed to the L2, before it lets the kernels after this one go:
         // the attention kernel reads them (from the L2) without a wait of its own.
-        grid_dependency_wait();        // (the list validator, if there is one)
-        order_lists<C::THREADS>(p.row_ptr, p.nQb, p.order_ctas, blockIdx.x, p.order, p.ws_status, p.user_status,
-                                p.clear_status, reinterpret_cast<int*>(smem));
-        __threadfence();
-        __syncthreads();
+        if (int(blockIdx.x) < p.Hm) {
+            grid_dependency_wait();    // (the list validator, if there is one)
+            order_lists<C::THREADS>(p.row_ptr, p.nQb, p.Hm, blockIdx.x, p.order, p.ws_status, p.user_status,
+                                    p.clear_status, reinterpret_cast<int*>(smem));
+            __threadfence();
+            __syncthreads();
+        }
         grid_launch_dependents();
         return;
     }
@@ -229,11 +241,13 @@ salad_linear_state_kernel(const __grid_constant__ CUtensorMap map_k, const __gri
         // accumulator -> this chunk's partial.  TMEM lane = key channel a; columns [0,D) = KV
         // row a, column D = Z[a].
         if (ok) ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&acc_done), 0, abortp));
+        float* z_out_ptr = p.reduce ? reinterpret_cast<float*>(smem + C::OFF_ZP) : p.z_part + (size_t(bh) * p.chunks + chunk) * D;
         if (ok) {
             tc_fence_after_sync();
             const int a = (warp & 3) * 32 + lane;       // lanes this warp may access
             const uint32_t t_row = tmem + (uint32_t((warp & 3) * 32) << 16);
-            float* kv_row = p.kv_part + ((size_t(bh) * p.chunks + chunk) * D + a) * D;
+            float* kv_row = p.reduce ? reinterpret_cast<float*>(smem) + (a < D ? a : 0) * C::KS
+                                     : p.kv_part + ((size_t(bh) * p.chunks + chunk) * D + a) * D;
             // (ROPE: eight warps, two per group of 32 lanes: each takes half of the columns)
             constexpr int NCC = (D / 32) / (RW / 128);
             const int cc0 = ((warp - 2) / 4) * NCC;
@@ -254,14 +268,13 @@ salad_linear_state_kernel(const __grid_constant__ CUtensorMap map_k, const __gri
             if (!ROPE) {
                 uint32_t zr[32];
                 if (nblk > 0) { tmem_ld32(t_row + D, zr); tmem_wait_ld(); }   // reads 32 columns, uses the first
-                if (a < D)
-                    p.z_part[(size_t(bh) * p.chunks + chunk) * D + a] = nblk > 0 ? __uint_as_float(zr[0]) : 0.f;
+                if (a < D) z_out_ptr[a] = nblk > 0 ? __uint_as_float(zr[0]) : 0.f;
             }
         }
         if (ROPE && ok) {
-            // Z of this chunk: the threads' register sums, staged in the (now idle) first stage and added
+            // Z of this chunk: the threads' register sums, staged over the (now idle) stages and added
             // per channel over the RW / 8 threads that met it, in a fixed order
-            float* zs = reinterpret_cast<float*>(smem);
+            float* zs = reinterpret_cast<float*>(smem + C::OFF_ZS);
 #pragma unroll
             for (int ch = 0; ch < C::CH; ++ch)
 #pragma unroll
@@ -274,10 +287,53 @@ salad_linear_state_kernel(const __grid_constant__ CUtensorMap map_k, const __gri
 #pragma unroll
                 for (int r8 = 0; r8 < RW / 8; ++r8)
                     sum += zs[(r8 * 8 + (grp ^ (r8 & 7))) * (C::CH * 8) + ch * 8 + e];
-                p.z_part[(size_t(bh) * p.chunks + chunk) * D + wt] = sum;
+                z_out_ptr[wt] = sum;
             }
         }
     }
+    }
+
+    if (p.reduce) {
+        // The partials of the head's CTAs are in their shared memories.  Every CTA adds the rows of its slice (whole
+        // groups of eight key channels) in chunk order, in place: nobody else reads those rows of its own copy.  After
+        // an expired wait the numbers are rubbish and the status says so; the barriers are met all the same.
+        __syncthreads();
+        cluster_sync_all();
+        constexpr int G = D / 8;
+        const int a0 = G * chunk / p.chunks * 8, a1 = G * (chunk + 1) / p.chunks * 8;
+        float* mine = reinterpret_cast<float*>(smem);
+        for (int i = tid; i < (a1 - a0) * (D / 4); i += C::THREADS) {
+            const int a = a0 + i / (D / 4), c = (i % (D / 4)) * 4;
+            const uint32_t off = s_base + (a * C::KS + c) * 4;
+            float4 v[8], s = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+            for (int r = 0; r < 8; ++r) if (r < p.chunks) v[r] = ld_cluster_f4(map_to_cta(off, r));
+#pragma unroll
+            for (int r = 0; r < 8; ++r) if (r < p.chunks) { s.x += v[r].x; s.y += v[r].y; s.z += v[r].z; s.w += v[r].w; }
+            *reinterpret_cast<float4*>(mine + a * C::KS + c) = s;
+            if (p.kv_out) *reinterpret_cast<float4*>(p.kv_out + (size_t(bh) * D + a) * D + c) = s;
+        }
+        if (chunk == 0 && tid < D / 4) {
+            float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+            for (int r = 0; r < p.chunks; ++r) {
+                const float4 v = ld_cluster_f4(map_to_cta(s_base + C::OFF_ZP + tid * 16, r));
+                s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w;
+            }
+            *reinterpret_cast<float4*>(p.z_ws + size_t(bh) * D + tid * 4) = s;
+            if (p.z_out) *reinterpret_cast<float4*>(p.z_out + size_t(bh) * D + tid * 4) = s;
+        }
+        __syncthreads();
+        // the transposed bf16 copy: eight key channels of one value channel per thread
+        for (int i = tid; i < (a1 - a0) / 8 * D; i += C::THREADS) {
+            const int c = i % D, a = a0 + i / D * 8;
+            uint4 o;
+            uint32_t* w = reinterpret_cast<uint32_t*>(&o);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) w[e] = pack_bf16x2(mine[(a + 2 * e) * C::KS + c], mine[(a + 2 * e + 1) * C::KS + c]);
+            *reinterpret_cast<uint4*>(p.kvt + (size_t(bh) * D + c) * D + a) = o;
+        }
+        __syncthreads();
+        cluster_sync_all();            // nobody leaves while its partial is being read
     }
 
     tc_fence_before_sync();

@@ -255,6 +255,27 @@ int list_rows_of(const Problem& P) {
     return (P.st_T > 0 && stswa_geometry(P.st_T, P.st_Hs, P.st_Ws, &sg)) ? sg.rows : 0;
 }
 
+// How many clusters of `size` CTAs of a state kernel the device holds at once (asked once per device and size).
+template <auto Kernel>
+int max_clusters(int size, int threads, int smem) {
+    static int cached[64][9] = {};
+    std::lock_guard<std::mutex> lock(g_init_mutex);
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64 || size < 1 || size > 8) { cudaGetLastError(); return 0; }
+    if (cached[dev][size] == 0) {
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(unsigned(size)); cfg.blockDim = dim3(unsigned(threads)); cfg.dynamicSmemBytes = size_t(smem);
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = unsigned(size); attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+        cfg.attrs = attr; cfg.numAttrs = 1;
+        int n = 0;
+        if (cudaOccupancyMaxActiveClusters(&n, Kernel, &cfg) != cudaSuccess) { cudaGetLastError(); n = 0; }
+        cached[dev][size] = n + 1;
+    }
+    return cached[dev][size] - 1;
+}
+
 // The maps of K and V in 64-token boxes, which the state kernel and the attention kernel share.
 struct KvMaps { CUtensorMap k, v; };
 bool make_kv_maps(const Problem& P, KvMaps* m) {
@@ -270,6 +291,29 @@ int launch_state(const Problem& P, const KvMaps& kv, const Workspace& w, const D
     if (chunks < 1) chunks = 1;
     if (chunks > nKb) chunks = nKb;
     if (int64_t(chunks) * BH > w.slots) chunks = w.slots / BH;
+    // Up to eight chunks per head: the CTAs of a head form a cluster and add their partials through shared memory,
+    // which saves the finalize kernel and the partials' way through global memory -- with one CTA per SM only where the
+    // clusters of all heads are resident together (clusters of six leave a third of a GPC idle: 24 heads of 900
+    // tokens, linear-only, 23.5 against 19.4 us; with two CTAs per SM, in the fused call, 24.0 -> 20.3).  More
+    // chunks than eight are cut to eight where that is the faster: sequences of up to D key blocks (12 heads, D = 128,
+    // fused call: 50.9 -> 49.2 us at 8190 tokens, 92.5 against 92.6 at 16380, 164 against 169 at 32760; two heads: 28.3
+    // -> 22.6 and 30.3 against 33.0 at 8190 and 16380; D = 64, 12 heads: 25.2 -> 24.3 and 34.9 against 35.3 at 5000 and
+    // 8190), and at D = 128 linear-only calls whose eight-fold split still fills 60 % of the SMs, enough for the
+    // memory system (12 heads of 32760 tokens: state pass 41.8 -> 37.7 us on 96 CTAs instead of 144; at D = 64,
+    // with half the bytes in flight per CTA, 25.2 against 32.8).
+    const bool sparse = (P.mode & MODE_SPARSE) != 0;
+    const bool overlap = sparse && !P.rope;          // the short-ring variant, two CTAs per SM
+    auto clusters = [&](int size) {
+        if (P.rope) return max_clusters<salad_linear_state_kernel<D, false, true>>(size, StateCfg<D, false, true>::THREADS, StateCfg<D, false, true>::SMEM_BYTES);
+        return max_clusters<salad_linear_state_kernel<D, false, false>>(size, StateCfg<D, false, false>::THREADS, StateCfg<D, false, false>::SMEM_BYTES);
+    };
+    bool reduce = !P.proj_blocks;
+    if (reduce && chunks > 8) {
+        reduce = (nKb <= D || (D == 128 && !sparse && 8 * BH * 5 >= dev.sms * 3)) && (overlap || clusters(8) >= BH);
+        if (reduce) chunks = 8;
+    } else if (reduce) {
+        reduce = chunks == 1 || overlap || clusters(chunks) >= BH;
+    }
     const int bpc = (nKb + chunks - 1) / chunks;
     uint8_t* ws = static_cast<uint8_t*>(P.ws);
     CUtensorMap mr = kv.k;          // unused without a rotation table
@@ -291,31 +335,51 @@ int launch_state(const Problem& P, const KvMaps& kv, const Workspace& w, const D
     sp.clear_status = validated ? 0 : 1;
     sp.row_ptr = P.row_ptr; sp.order = reinterpret_cast<int32_t*>(ws + w.off_order);
     sp.nQb = list_rows;
-    sp.order_ctas = (P.mode & MODE_SPARSE) ? P.Hm : 0;
+    sp.Hm = (P.mode & MODE_SPARSE) ? P.Hm : 0;
+    sp.order_ctas = reduce ? (sp.Hm + chunks - 1) / chunks * chunks : sp.Hm;
+    sp.reduce = reduce ? 1 : 0;
+    float* z_ws = reinterpret_cast<float*>(ws + w.off_z);
+    __nv_bfloat16* kvt = reinterpret_cast<__nv_bfloat16*>(ws + w.off_kvt);
+    sp.kv_out = P.kv_out; sp.z_out = P.z_out; sp.z_ws = z_ws; sp.kvt = kvt;
     auto launch = [&](auto kernel, int threads, int smem) {
         const dim3 grid(unsigned(sp.order_ctas + int64_t(chunks) * BH));
         SALAD_LOGF("salad_linear_state_kernel grid %d + %d x %d%s", sp.order_ctas, chunks, BH,
                    validated ? " after csr_validate_kernel" : "");
-        if (!validated) kernel<<<grid, dim3(threads), size_t(smem), P.stream>>>(kv.k, kv.v, mr, sp);
-        else launch_dependent(kernel, grid, dim3(threads), size_t(smem), P.stream, kv.k, kv.v, mr, sp);
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = grid; cfg.blockDim = dim3(threads); cfg.dynamicSmemBytes = size_t(smem); cfg.stream = P.stream;
+        cudaLaunchAttribute attr[2];
+        if (validated) {
+            attr[cfg.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+            attr[cfg.numAttrs++].val.programmaticStreamSerializationAllowed = 1;
+        }
+        if (reduce) {
+            attr[cfg.numAttrs].id = cudaLaunchAttributeClusterDimension;
+            attr[cfg.numAttrs].val.clusterDim.x = unsigned(chunks);
+            attr[cfg.numAttrs].val.clusterDim.y = 1;
+            attr[cfg.numAttrs++].val.clusterDim.z = 1;
+        }
+        cfg.attrs = attr;
+        cudaLaunchKernelEx(&cfg, kernel, kv.k, kv.v, mr, sp);          // errors are read by check_launch()
     };
     if (P.rope)
         launch(salad_linear_state_kernel<D, false, true>, StateCfg<D, false, true>::THREADS,
                StateCfg<D, false, true>::SMEM_BYTES);
-    else if (P.mode & MODE_SPARSE)
+    else if (overlap)
         launch(salad_linear_state_kernel<D, true, false>, StateCfg<D, true, false>::THREADS,
                StateCfg<D, true, false>::SMEM_BYTES);
     else
         launch(salad_linear_state_kernel<D, false, false>, StateCfg<D, false, false>::THREADS,
                StateCfg<D, false, false>::SMEM_BYTES);
     if (check_launch() != SALAD_OK) return SALAD_ERR_CUDA;
-    float* z_ws = reinterpret_cast<float*>(ws + w.off_z);
-    __nv_bfloat16* kvt = reinterpret_cast<__nv_bfloat16*>(ws + w.off_kvt);
+    if (reduce) {
+        record_profile(1, P.stream);
+        return SALAD_OK;
+    }
     if (P.proj_blocks)      // block-diagonal projection folded into the state: the attention kernel multiplies with KV W_h^T
         launch_dependent(salad_linear_finalize_proj_kernel<D>, dim3(D / 8, BH), dim3(256), 0, P.stream,
                          sp.kv_part, sp.z_part, chunks, static_cast<const __nv_bfloat16*>(P.proj_blocks), P.kv_out, z_ws,
                          P.z_out, kvt, P.dyn_scale, P.drop_tau, P.H);
-    else if ((P.mode & MODE_SPARSE) && !P.rope)
+    else if (overlap)
         launch_dependent(salad_linear_finalize_kernel<D, 8>, dim3(D / 32, D / 32, BH), dim3(32, 8), 0, P.stream,
                          sp.kv_part, sp.z_part, chunks, P.kv_out, z_ws, P.z_out, kvt, P.dyn_scale, P.drop_tau, P.H);
     else

@@ -1124,3 +1124,34 @@ def test_attention_calls_reject_a_broken_mask_without_touching_the_output(salad)
     after = salad.salad_fused_fwd(q, k, v, *dev_csr(rp, ci), 1, lam, s, status=status)
     torch.cuda.synchronize()
     assert int(status.item()) == 0 and torch.equal(after, good)
+
+
+# Splits of a head's tokens over a cluster: 1, 3, 6 and 8 CTAs, chunks of unequal length, empty chunks (nine key blocks on
+# eight CTAs), a rotation table, and a sequence one key block beyond the cut (the finalize kernel).
+@pytest.mark.parametrize("B,H,N,d", [(1, 2, 130, 128), (1, 3, 570, 64), (1, 12, 1000, 128), (1, 24, 700, 128),
+                                     (2, 20, 450, 64), (2, 74, 200, 64), (1, 2, 64 * 64 + 1, 64), (1, 2, 128 * 64 + 1, 128)])
+def test_linear_state_over_a_cluster(salad, B, H, N, d):
+    torch.manual_seed(B * 1000 + H * 10 + N)
+    q, k, v = (torch.randn(B, H, N, d, device="cuda", dtype=torch.bfloat16) for _ in range(3))
+    kv = torch.full((B, H, d, d), float("nan"), device="cuda")
+    z = torch.full((B, H, d), float("nan"), device="cuda")
+    out = salad.salad_linear_attn_fwd(q, k, v, kv_out=kv, z_out=z)
+    kr = k.double().clamp_min(0)
+    want_kv, want_z = kr.transpose(2, 3) @ v.double(), kr.sum(2)
+    # fp32 sums of N products of bf16 values (exact in fp32): N * 2^-24 relative to the sum of magnitudes at worst
+    bound = N * 2.0 ** -24
+    assert ((kv.double() - want_kv).abs() <= bound * (kr.transpose(2, 3) @ v.double().abs()) + 1e-30).all()
+    assert ((z.double() - want_z).abs() <= bound * want_z + 1e-30).all()
+    qr = q.double().clamp_min(0)
+    want = (qr @ want_kv) / ((qr * want_z[:, :, None]).sum(-1, keepdim=True) + 1e-6)
+    assert float((out.double() - want).norm() / want.norm()) <= 1e-2
+    # the same state in a fused call without a kept block (two CTAs per SM), with the rotation table of the identity
+    rp = torch.zeros((N + 127) // 128 + 1, dtype=torch.int32, device="cuda")
+    ci = torch.zeros(1, dtype=torch.int32, device="cuda")
+    one_h, one_b = torch.ones(H, device="cuda"), torch.ones(B, device="cuda")
+    fused = salad.salad_fused_fwd(q, k, v, rp, ci, 1, one_h, one_b)
+    assert float((fused.double() - want).norm() / want.norm()) <= 1e-2
+    rope = torch.zeros((N, d // 2, 2), dtype=torch.float16, device="cuda")
+    rope[..., 0] = 1
+    rotated = salad.salad_linear_attn_rope_fwd(q, k, v, rope)
+    assert float((rotated.double() - want).norm() / want.norm()) <= 1e-2
