@@ -1155,3 +1155,30 @@ def test_linear_state_over_a_cluster(salad, B, H, N, d):
     rope[..., 0] = 1
     rotated = salad.salad_linear_attn_rope_fwd(q, k, v, rope)
     assert float((rotated.double() - want).norm() / want.norm()) <= 1e-2
+
+
+# Row maxima that move in the middle of a list: by more than the kernel lets pass in every block, in some rows of a
+# warp only, in the ragged last block, downwards (the first block holds the maximum), and by hundreds of powers of two.
+@pytest.mark.parametrize("growth", [9.0, 40.0, -9.0, 300.0])
+@pytest.mark.parametrize("N,d,Bq", [(64 * 9 + 17, 128, 128), (64 * 4, 64, 64), (130, 128, 128)])
+def test_running_maximum_moves(salad, N, d, Bq, growth):
+    torch.manual_seed(N + d)
+    q, k, v = (torch.randn(1, 2, N, d, device="cuda") for _ in range(3))
+    # scores grow by `growth` natural-log units from one key block to the next, in three of every four rows
+    direction = torch.ones(d, device="cuda") / d ** 0.5
+    q = 0.3 * q + (torch.arange(N, device="cuda") % 4 != 0).float()[:, None] * direction * 8
+    step = (torch.arange(N, device="cuda") // 64).float() * growth * d ** 0.5 / 8
+    k = k + step[:, None] * direction
+    q, k, v = q.bfloat16(), k.bfloat16(), v.bfloat16()
+    nQb, nKb = -(-N // Bq), -(-N // 64)
+    rp = torch.arange(nQb + 1, dtype=torch.int32, device="cuda") * nKb
+    ci = torch.arange(nKb, dtype=torch.int32, device="cuda").repeat(nQb)
+    lse = torch.empty(1, 2, N, device="cuda")
+    out = salad.salad_sparse_attn_fwd(q, k, v, rp, ci, 1, Bq=Bq, lse=lse)
+    x = q.double() @ k.double().transpose(2, 3) / d ** 0.5
+    want = torch.softmax(x, -1) @ v.double()
+    # bf16 probabilities and output (2^-9 each, relative); scores of up to 2700 in fp32 (products exact, d additions)
+    err = float(x.abs().max()) * d * 2.0 ** -24
+    assert float((out.double() - want).norm() / want.norm()) <= 1e-2 + err
+    want_lse = torch.logsumexp(x, -1)
+    assert float((lse.double() - want_lse).abs().max()) <= 2e-3 + 2 * err
