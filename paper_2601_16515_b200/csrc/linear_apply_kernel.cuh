@@ -80,12 +80,36 @@ salad_linear_apply_kernel(const __grid_constant__ CUtensorMap map_q, const __gri
     const uint32_t s_base = smem_u32(smem);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     // contiguous, balanced range of tiles (head-major, so the state changes rarely)
-    const long long t0 = p.tiles * blockIdx.x / gridDim.x, t1 = p.tiles * (blockIdx.x + 1) / gridDim.x;
+    const long long t0 = p.tiles * blockIdx.x / gridDim.x;
+    const int tiles = int(p.tiles * (blockIdx.x + 1) / gridDim.x - t0);
+    // The tile in hand, as (batch, head) and query block: every role steps through them without a division (two 64-bit
+    // divisions per tile in the one thread that loads were a tenth of the time at D = 64).
+    struct Walk {
+        int bh, qb, nQb;
+        __device__ __forceinline__ void next() { if (++qb == nQb) { qb = 0; ++bh; } }
+    };
+    const Walk first{int(t0 / p.nQb), int(t0 % p.nQb), p.nQb};
 
-    grid_dependency_wait();
+    // Q is an input of the call, not a product of the kernel before this one: everything up to the first Q tiles runs
+    // while the state pass drains, and only what touches the state waits for it (warp 0 and the ReLU warps): 12.8 ->
+    // 12.1 us for a call on two heads of 900 tokens, 53.3 -> 51.6 us on 24 heads of 8190.  At D = 64 the
+    // kernel waits at its top: started early it ran slower afterwards (80 heads of 32760 tokens 371 against 341 us per
+    // call, 12 heads 54.1 against 49.8) and gained nothing on short sequences.
+    auto load_q = [&](int bh, int qb, int j) {
+        const int s = j % C::NQ;
+        const uint32_t bar = smem_u32(&bars.q_full[s]);
+        mbar_arrive_expect_tx(bar, C::STAGE_BYTES);
+        for (int ch = 0; ch < C::CH; ++ch) {
+            tma_load_3d(s_base + C::OFF_Q + s * C::STAGE_BYTES + ch * C::Q_CHUNK, &map_q, bar, ch * 64, qb * 128, bh);
+            if (ROPE)
+                tma_load_3d(s_base + C::OFF_Q + s * C::STAGE_BYTES + C::Q_BYTES + ch * C::Q_CHUNK, &map_r, bar,
+                            ch * 64, qb * 128, 0);
+        }
+    };
+    if (D == 64) grid_dependency_wait();
     grid_launch_dependents();
     if (tid == 0) {
-        abort_flag = (*reinterpret_cast<volatile int32_t*>(p.ws_status) != 0) ? 2 : 0;    // 2: reported by an earlier kernel
+        abort_flag = 0;
         for (int s = 0; s < C::NQ; ++s) {
             mbar_init(smem_u32(&bars.q_full[s]), 1);
             mbar_init(smem_u32(&bars.q_empty[s]), 1);
@@ -101,6 +125,10 @@ salad_linear_apply_kernel(const __grid_constant__ CUtensorMap map_q, const __gri
         mbar_init(smem_u32(&bars.out_staged), 128);
         mbar_init(smem_u32(&bars.out_free), 1);
         fence_mbar_init();
+        prefetch_tmap(&map_q); prefetch_tmap(&map_st); prefetch_tmap(&map_o);
+        if (ROPE) prefetch_tmap(&map_r);
+        Walk w = first;
+        for (int j = 0; j < C::NQ && j < tiles; ++j, w.next()) load_q(w.bh, w.qb, j);
     }
     if (warp == 1) { tmem_alloc(smem_u32(&tmem_base_slot), C::TMEM_COLS); tmem_relinquish(); }
     tc_fence_before_sync();
@@ -113,11 +141,12 @@ salad_linear_apply_kernel(const __grid_constant__ CUtensorMap map_q, const __gri
     if (warp == 0) {
         // ============================================================== TMA producer
         if (lane == 0) {
-            prefetch_tmap(&map_q); prefetch_tmap(&map_st); prefetch_tmap(&map_o);
-            if (ROPE) prefetch_tmap(&map_r);
-            int prev_bh = -1, n_st = 0, j = 0;
-            for (long long t = t0; t < t1; ++t, ++j) {
-                const int bh = int(t / p.nQb), qb = int(t % p.nQb);
+            grid_dependency_wait();
+            if (*reinterpret_cast<volatile int32_t*>(p.ws_status) != 0) abort_flag = 2;    // reported by an earlier kernel
+            int prev_bh = -1, n_st = 0;
+            Walk w = first;
+            for (int j = 0; j < tiles; ++j, w.next()) {
+                const int bh = w.bh;
                 if (bh != prev_bh) {
                     const int sb = n_st % C::NST;
                     if (!mbar_wait(smem_u32(&bars.st_empty[sb]), ((n_st / C::NST) & 1) ^ 1, abortp)) break;
@@ -128,17 +157,9 @@ salad_linear_apply_kernel(const __grid_constant__ CUtensorMap map_q, const __gri
                                     ch * 64, 0, bh);
                     ++n_st; prev_bh = bh;
                 }
-                const int s = j % C::NQ;
-                if (!mbar_wait(smem_u32(&bars.q_empty[s]), ((j / C::NQ) & 1) ^ 1, abortp)) break;
-                const uint32_t bar = smem_u32(&bars.q_full[s]);
-                mbar_arrive_expect_tx(bar, C::STAGE_BYTES);
-                for (int ch = 0; ch < C::CH; ++ch) {
-                    tma_load_3d(s_base + C::OFF_Q + s * C::STAGE_BYTES + ch * C::Q_CHUNK, &map_q, bar,
-                                ch * 64, qb * 128, bh);
-                    if (ROPE)
-                        tma_load_3d(s_base + C::OFF_Q + s * C::STAGE_BYTES + C::Q_BYTES + ch * C::Q_CHUNK, &map_r, bar,
-                                    ch * 64, qb * 128, 0);
-                }
+                if (j < C::NQ) continue;                                   // the first tiles are on their way
+                if (!mbar_wait(smem_u32(&bars.q_empty[j % C::NQ]), ((j / C::NQ) & 1) ^ 1, abortp)) break;
+                load_q(bh, w.qb, j);
             }
         }
     } else if (warp == 1) {
@@ -146,10 +167,11 @@ salad_linear_apply_kernel(const __grid_constant__ CUtensorMap map_q, const __gri
         if (lane == 0) {
             const uint32_t idesc = make_idesc_bf16(128, D, 0, 0);
             constexpr uint32_t HI = sdesc_hi_sw128(1024);
-            int prev_bh = -1, n_st = 0, j = 0, sb = 0;
+            int prev_bh = -1, n_st = 0, sb = 0;
             bool ok = true;
-            for (long long t = t0; t < t1 && ok; ++t, ++j) {
-                const int bh = int(t / p.nQb);
+            Walk w = first;
+            for (int j = 0; j < tiles && ok; ++j, w.next()) {
+                const int bh = w.bh;
                 if (bh != prev_bh) {
                     // the MMAs that read the previous state buffer are all issued: hand it back
                     if (prev_bh >= 0) tc_commit(smem_u32(&bars.st_empty[sb]));
@@ -176,11 +198,13 @@ salad_linear_apply_kernel(const __grid_constant__ CUtensorMap map_q, const __gri
     } else if (warp < 6) {
         // ============================================================== ReLU(Q) in place, denominators
         const int row = tid - 64;
-        int prev_bh = -1, n_z = 0, j = 0, zb = 0;
+        grid_dependency_wait();
+        int prev_bh = -1, n_z = 0, zb = 0;
         float c_scale = 1.f;
         bool ok = true;
-        for (long long t = t0; t < t1 && ok; ++t, ++j) {
-            const int bh = int(t / p.nQb);
+        Walk w = first;
+        for (int j = 0; j < tiles && ok; ++j, w.next()) {
+            const int bh = w.bh;
             if (bh != prev_bh) {
                 // Z of the new head into the other buffer; nobody reads that one any more (each
                 // thread arrives here only after its last read of the head before the previous one)
@@ -234,10 +258,10 @@ salad_linear_apply_kernel(const __grid_constant__ CUtensorMap map_q, const __gri
         // ============================================================== accumulator -> bf16 -> TMA store
         const int row = (warp & 3) * 32 + lane;                     // = TMEM lane this thread may read
         const uint32_t t_row = tmem + (uint32_t((warp & 3) * 32) << 16);
-        int j = 0;
         bool ok = true;
-        for (long long t = t0; t < t1; ++t, ++j) {
-            const int bh = int(t / p.nQb), qb = int(t % p.nQb);
+        Walk walk = first;
+        for (int j = 0; j < tiles; ++j, walk.next()) {
+            const int bh = walk.bh, qb = walk.qb;
             const int ab = j & 1;                                   // accumulator
             ok = __all_sync(0xffffffffu, ok && mbar_wait(smem_u32(&bars.acc_full[ab]), (j >> 1) & 1, abortp));
             if (!ok) break;
