@@ -966,23 +966,36 @@ SALAD_EXPORT int salad_topk_mask_build(const void* q, const void* k, int B, int 
     float* kmeanT = reinterpret_cast<float*>(ws + align_up(size_t(BH) * nQb * d * 4));
     uint32_t* score = reinterpret_cast<uint32_t*>(ws + align_up(size_t(BH) * nQb * d * 4) +
                                                   align_up(size_t(BH) * d * ldk * 4));
-    MeanJob jq{static_cast<const uint4*>(q), qmean, Bq, int(nQb), 0};
-    MeanJob jk{static_cast<const uint4*>(k), kmeanT, Bk, int(nKb), ldk};
-    block_mean_kernel<<<dim3(unsigned(nQb > nKb ? nQb : nKb), unsigned(BH), 2), kMeanThreads, 0, st>>>(jq, jk, N, d);
+    if (Bq == 128 && Bk == 64) {
+        const dim3 grid(unsigned(nQb), static_cast<unsigned>(BH));
+        if (d == 128)
+            block_mean_pair_kernel<16><<<grid, kMeanThreads, 0, st>>>(static_cast<const uint4*>(q), static_cast<const uint4*>(k),
+                                                                      qmean, kmeanT, N, int(nQb), int(nKb), ldk);
+        else
+            block_mean_pair_kernel<8><<<grid, kMeanThreads, 0, st>>>(static_cast<const uint4*>(q), static_cast<const uint4*>(k),
+                                                                     qmean, kmeanT, N, int(nQb), int(nKb), ldk);
+    } else {
+        MeanJob jq{static_cast<const uint4*>(q), qmean, Bq, int(nQb), 0};
+        MeanJob jk{static_cast<const uint4*>(k), kmeanT, Bk, int(nKb), ldk};
+        block_mean_kernel<<<dim3(unsigned(nQb > nKb ? nQb : nKb), unsigned(BH), 2), kMeanThreads, 0, st>>>(jq, jk, N, d);
+    }
     if (check_launch() != SALAD_OK) return SALAD_ERR_CUDA;
     const size_t smem = kScoreSmemBytes;
     launch_dependent(topk_score_kernel, dim3(unsigned(ldk / kScoreTile), unsigned((nQb + kScoreRows - 1) / kScoreRows),
                                              unsigned(BH)),
                      dim3(128), smem, st, qmean, kmeanT, int(nQb), int(nKb), ldk, d, score);
     if (check_launch() != SALAD_OK) return SALAD_ERR_CUDA;
-    const dim3 pgrid(unsigned((rows + 7) / 8));
-    // a CTA per row while the row fits the threads' registers; the warp-per-two-rows kernel beyond that
-    if (nKb <= 512 && rows <= 2147483647ll)
-        launch_dependent(topk_pick_row_kernel<4>, dim3(unsigned(rows)), dim3(128), 0, st, score, int(nKb), int(kk), d_row_ptr, d_col_idx, rows);
-    else if (nKb <= 1024 && rows <= 2147483647ll)
-        launch_dependent(topk_pick_row_kernel<8>, dim3(unsigned(rows)), dim3(128), 0, st, score, int(nKb), int(kk), d_row_ptr, d_col_idx, rows);
-    else
-        launch_dependent(topk_pick_kernel, pgrid, dim3(128), 0, st, score, int(nKb), int(kk), d_row_ptr, d_col_idx, rows);
+    // a warp per row while the row fits its registers; the kernel that re-reads the row beyond that
+    const dim3 wgrid(unsigned((rows + 3) / 4));
+    auto pick = [&](auto kernel) {
+        launch_dependent(kernel, wgrid, dim3(128), 0, st, score, int(nKb), int(kk), d_row_ptr, d_col_idx, (long long)rows);
+    };
+    if (nKb <= 128) pick(topk_pick_warp_kernel<4>);
+    else if (nKb <= 512) pick(topk_pick_warp_kernel<16>);
+    else if (nKb <= 1024) pick(topk_pick_warp_kernel<32>);
+    else if (nKb <= 2048) pick(topk_pick_warp_kernel<64>);
+    else launch_dependent(topk_pick_kernel, dim3(unsigned((rows + 7) / 8)), dim3(128), 0, st, score, int(nKb), int(kk), d_row_ptr,
+                          d_col_idx, (long long)rows);
     return check_launch();
 }
 

@@ -8,13 +8,15 @@
 //                       block; a thread owns one 16-byte channel group of every G-th row, so a warp
 //                       instruction reads 512 contiguous bytes; the row groups are added in a fixed
 //                       order through shared memory (deterministic), fp32.
+//                       (block_mean_pair_kernel: blocks of 128 queries and 64 keys, the 128 tokens of a
+//                       query block and its two key blocks in one CTA with every load in flight at once.)
 //   topk_score_kernel   s for a 32 x 128 tile of (query block, key block) pairs per CTA: register-tiled
-//                       fp32 FMAs in channel order from channel-major shared memory; the scores go
-//                       to the workspace as order-preserving 32-bit images.
-//   topk_pick_row_kernel  per query block (a CTA each): the kk-th largest score by radix selection on
-//                       the bytes of its image, then an ordered compaction into the CSR row.
-//                       (topk_pick_kernel: the same by bisection, a warp per two rows, for rows of more
-//                       than 1024 key blocks.)
+//                       fp32 FMAs, two at a time, in channel order from channel-major shared memory; the scores
+//                       go to the workspace as order-preserving 32-bit images.
+//   topk_pick_warp_kernel  per query block (a warp each, the scores in its registers): the kk-th largest score by
+//                       bisection on the bits of its image, then an ordered compaction into the CSR row.
+//                       (topk_pick_kernel: the same with the scores re-read in every pass, for rows of more
+//                       than 2048 key blocks.)
 #pragma once
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -69,6 +71,63 @@ block_mean_kernel(MeanJob jq, MeanJob jk, int N, int d)
     }
 }
 
+// Blocks of 128 queries and 64 keys: grid (nQb, BH), 256 threads.  The CTA of query block i also takes the key blocks 2i and
+// 2i + 1, so all of its 2 * 128 rows are the same token range, and every thread issues all of its loads (8 or 4 rows of Q and
+// as many of K) ahead of the adds, half as many CTAs as token blocks with twice the bytes each: 44 -> 39 us at 12 heads of
+// 32760 tokens, d = 128 (5.2 TB/s).  The sums run in the same order as in block_mean_kernel.  It lets the score kernel go
+// only by its end: score CTAs placed early took shared memory from this kernel's (63 -> 73 us per call).
+template <int CHUNKS>                                             // 16-byte groups per row: d / 8
+__global__ void __launch_bounds__(kMeanThreads)
+block_mean_pair_kernel(const uint4* __restrict__ q, const uint4* __restrict__ k, float* __restrict__ qmean,
+                       float* __restrict__ kmeanT, int N, int nQb, int nKb, int ldk)
+{
+    constexpr int D = CHUNKS * 8, GROUPS = kMeanThreads / CHUNKS, ROWS = 128 / GROUPS, HALF = ROWS / 2;
+    __shared__ float part[3][GROUPS][D + 4];                     // queries, keys of block 2i, of block 2i + 1
+    const int blk = blockIdx.x, bh = blockIdx.y, tid = threadIdx.x, c = tid % CHUNKS, g = tid / CHUNKS;
+    const int n0 = blk * 128;
+    const size_t base = (size_t(bh) * N) * CHUNKS + c;
+    uint4 vq[ROWS], vk[ROWS];
+#pragma unroll
+    for (int r = 0; r < ROWS; ++r) {
+        const int n = n0 + g + r * GROUPS;
+        vq[r] = n < N ? __ldg(q + base + size_t(n) * CHUNKS) : make_uint4(0, 0, 0, 0);
+        vk[r] = n < N ? __ldg(k + base + size_t(n) * CHUNKS) : make_uint4(0, 0, 0, 0);
+    }
+    float sum[3][8];
+#pragma unroll
+    for (int j = 0; j < 3; ++j)
+#pragma unroll
+        for (int e = 0; e < 8; ++e) sum[j][e] = 0.f;
+#pragma unroll
+    for (int r = 0; r < ROWS; ++r) {
+        const __nv_bfloat162* hq = reinterpret_cast<const __nv_bfloat162*>(&vq[r]);
+        const __nv_bfloat162* hk = reinterpret_cast<const __nv_bfloat162*>(&vk[r]);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const float2 fq = __bfloat1622float2(hq[e]), fk = __bfloat1622float2(hk[e]);
+            sum[0][2 * e] += fq.x; sum[0][2 * e + 1] += fq.y;
+            sum[r < HALF ? 1 : 2][2 * e] += fk.x; sum[r < HALF ? 1 : 2][2 * e + 1] += fk.y;
+        }
+    }
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+        *reinterpret_cast<float4*>(&part[j][g][c * 8]) = make_float4(sum[j][0], sum[j][1], sum[j][2], sum[j][3]);
+        *reinterpret_cast<float4*>(&part[j][g][c * 8 + 4]) = make_float4(sum[j][4], sum[j][5], sum[j][6], sum[j][7]);
+    }
+    __syncthreads();
+    for (int i = tid; i < 3 * D; i += kMeanThreads) {
+        const int j = i / D, ch = i % D;
+        const int first = j == 2 ? n0 + 64 : n0, tokens = min(N, first + (j == 0 ? 128 : 64)) - first;
+        if (tokens <= 0) continue;                               // the second key block may lie past the end
+        float s = 0.f;
+#pragma unroll
+        for (int gg = 0; gg < GROUPS; ++gg) s += part[j][gg][ch];            // fixed order
+        const float m = s / float(tokens);
+        if (j == 0) qmean[(size_t(bh) * nQb + blk) * D + ch] = m;
+        else        kmeanT[(size_t(bh) * D + ch) * ldk + 2 * blk + j - 1] = m;
+    }
+}
+
 constexpr int kScoreRows = 32;        // query blocks per CTA (four warps, eight each)
 constexpr int kScoreTile = 128;       // key blocks per CTA (four per lane)
 
@@ -109,32 +168,47 @@ topk_score_kernel(const float* __restrict__ qmean, const float* __restrict__ kme
     const int r_q = tid % kScoreRows, ii = min(i0 + r_q, nQb - 1);
     const float* qsrc = qmean + (size_t(bh) * nQb + ii) * d;
     auto fetch = [&](int chunk, int stage) {
-        float* As = sc_smem + stage * STAGE;
-        float* Bs = As + kScoreChunk * kScoreRows;
+        float* Bs = sc_smem + stage * STAGE + kScoreChunk * kScoreRows;
         const int c0 = chunk * kScoreChunk;
         // key-block means: rows of 128 contiguous floats per channel
         for (int idx = tid; idx < kScoreChunk * (kScoreTile / 4); idx += 128) {
             const int c = idx / (kScoreTile / 4), f = idx % (kScoreTile / 4);
             cp_async_16(Bs + c * kScoreTile + f * 4, ksrc + size_t(c0 + c) * ldk + f * 4);
         }
-        // query-block means, transposed on the way in: this thread's row, one float4 of channels
-        for (int c4 = tid / kScoreRows; c4 < kScoreChunk / 4; c4 += 128 / kScoreRows) {     // channels 4 c4 .. 4 c4 + 3 of the chunk
-            const float4 v = __ldg(reinterpret_cast<const float4*>(qsrc + c0) + c4);
-            As[(c4 * 4 + 0) * kScoreRows + r_q] = v.x; As[(c4 * 4 + 1) * kScoreRows + r_q] = v.y;
-            As[(c4 * 4 + 2) * kScoreRows + r_q] = v.z; As[(c4 * 4 + 3) * kScoreRows + r_q] = v.w;
-        }
         asm volatile("cp.async.commit_group;" ::: "memory");
     };
-    float acc[8][4];
+    // query-block means, transposed on the way in: this thread's row, two float4 of channels, in registers while the
+    // chunk before them is multiplied (stored at once they left an L2 round trip exposed per chunk)
+    constexpr int QV = kScoreChunk / 4 / (128 / kScoreRows);
+    float4 qnext[QV];
+    auto fetch_q = [&](int chunk) {
 #pragma unroll
-    for (int r = 0; r < 8; ++r)
+        for (int e = 0; e < QV; ++e)
+            qnext[e] = __ldg(reinterpret_cast<const float4*>(qsrc + chunk * kScoreChunk) + tid / kScoreRows + e * (128 / kScoreRows));
+    };
+    auto store_q = [&](int stage) {
+        float* As = sc_smem + stage * STAGE;
 #pragma unroll
-        for (int u = 0; u < 4; ++u) acc[r][u] = 0.f;
+        for (int e = 0; e < QV; ++e) {
+            const int c = (tid / kScoreRows + e * (128 / kScoreRows)) * 4;
+            As[(c + 0) * kScoreRows + r_q] = qnext[e].x; As[(c + 1) * kScoreRows + r_q] = qnext[e].y;
+            As[(c + 2) * kScoreRows + r_q] = qnext[e].z; As[(c + 3) * kScoreRows + r_q] = qnext[e].w;
+        }
+    };
+    // two query rows in one packed accumulator: 16 packed FMAs per channel instead of 32 (the same roundings)
+    uint64_t acc[4][4];
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+#pragma unroll
+        for (int u = 0; u < 4; ++u) acc[r][u] = pack_f32x2(0.f, 0.f);
     const int chunks = d / kScoreChunk;
     fetch(0, 0);
+    fetch_q(0);
+    store_q(0);
     for (int ch = 0; ch < chunks; ++ch) {
         if (ch + 1 < chunks) {
             fetch(ch + 1, (ch + 1) & 1);
+            fetch_q(ch + 1);
             asm volatile("cp.async.wait_group 1;" ::: "memory");
         } else {
             asm volatile("cp.async.wait_group 0;" ::: "memory");
@@ -147,12 +221,14 @@ topk_score_kernel(const float* __restrict__ qmean, const float* __restrict__ kme
             const float4 qa = *reinterpret_cast<const float4*>(As + c * kScoreRows + warp * 8);
             const float4 qb = *reinterpret_cast<const float4*>(As + c * kScoreRows + warp * 8 + 4);
             const float4 k4 = *reinterpret_cast<const float4*>(Bs + c * kScoreTile + lane * 4);
-            const float qv[8] = {qa.x, qa.y, qa.z, qa.w, qb.x, qb.y, qb.z, qb.w}, kv[4] = {k4.x, k4.y, k4.z, k4.w};
+            const uint64_t qv[4] = {pack_f32x2(qa.x, qa.y), pack_f32x2(qa.z, qa.w), pack_f32x2(qb.x, qb.y), pack_f32x2(qb.z, qb.w)};
+            const uint64_t kv[4] = {pack_f32x2(k4.x, k4.x), pack_f32x2(k4.y, k4.y), pack_f32x2(k4.z, k4.z), pack_f32x2(k4.w, k4.w)};
 #pragma unroll
-            for (int r = 0; r < 8; ++r)
+            for (int r = 0; r < 4; ++r)
 #pragma unroll
-                for (int u = 0; u < 4; ++u) acc[r][u] = fmaf(qv[r], kv[u], acc[r][u]);
+                for (int u = 0; u < 4; ++u) acc[r][u] = fma_f32x2(qv[r], kv[u], acc[r][u]);
         }
+        if (ch + 1 < chunks) store_q((ch + 1) & 1);
         __syncthreads();                                           // the stage is fetched into again two chunks on
     }
 #pragma unroll
@@ -161,8 +237,11 @@ topk_score_kernel(const float* __restrict__ qmean, const float* __restrict__ kme
         if (i >= nQb) break;
         uint32_t* out = score + (size_t(bh) * nQb + i) * nKb + j0 + lane * 4;
 #pragma unroll
-        for (int u = 0; u < 4; ++u)
-            if (j0 + lane * 4 + u < nKb) out[u] = ordered_bits(acc[r][u]);
+        for (int u = 0; u < 4; ++u) {
+            float lo, hi;
+            unpack_f32x2(acc[r / 2][u], lo, hi);
+            if (j0 + lane * 4 + u < nKb) out[u] = ordered_bits((r & 1) ? hi : lo);
+        }
     }
 }
 
@@ -171,7 +250,7 @@ topk_score_kernel(const float* __restrict__ qmean, const float* __restrict__ kme
 // whatever kk), everything above it, and of the scores equal to it the lowest block indices -- the
 // same set as kk rounds of "largest remaining, ties to the lower index".
 // The lane's share of a row is re-read (from L1/L2) in every pass: this is the kernel for rows too long for
-// topk_pick_row_kernel below (more than 1024 key blocks).
+// topk_pick_warp_kernel below (more than 2048 key blocks).
 __global__ void __launch_bounds__(128)
 topk_pick_kernel(const uint32_t* __restrict__ score, int nKb, int kk, int32_t* __restrict__ row_ptr,
                  int32_t* __restrict__ col_idx, long long rows_total)
@@ -226,121 +305,72 @@ topk_pick_kernel(const uint32_t* __restrict__ score, int nKb, int kk, int32_t* _
     }
 }
 
-// One CTA (four warps) per row: with a warp per two rows only ten warps ran on an SM and the selection was a
-// chain of dependent steps (measured 18-20 us for 3072 rows of 512 scores); a CTA per row puts sixteen rows on
-// an SM at a time and shortens every step by a factor of four.
-//   1. radix selection of the kk-th largest image from the top byte down: four passes, each a 256-bin
-//      histogram (shared-memory atomics) of the byte among the keys that still share the bytes chosen so far,
-//      then the bin in which the count from the top reaches what is still needed (every warp does that scan
-//      for itself, so a pass needs one barrier; the histograms rotate through three buffers).  Absent
-//      entries are 0 and every real image is > 0, so they are never counted.
-//   2. ties: if more keys equal the threshold than the selection takes, warp 0 finds the index up to which
-//      they belong to it (a tie goes to the lower block index).
-//   3. ordered compaction: per 128-key chunk a ballot per warp, one table of counts, every thread places its keys.
-// KPT keys per thread in registers (key j = tid + 128 i); needs nKb <= 128 KPT and nKb <= 128 * kPickMaxChunks.
-constexpr int kPickMaxChunks = 8;
-
+// One warp per row, the row's keys in its registers (key j = lane + 32 i in register i; absent ones 0, every real image is
+// > 0).  Nothing crosses warps, so there is no barrier; a pass of the bisection is KPT compares and one warp-wide sum.
+//   1. bisection on the bits of the image, from the highest bit in which the row's largest and smallest keys
+//      differ: T grows as long as at least kk keys are >= T.  As soon as exactly kk are, the set is known: with
+//      distinct scores after about half of the passes.
+//      (A CTA per row with radix passes over shared-memory histograms, which this replaces, took 13 us for 3072 rows of
+//      512 scores against 11, and nothing fitted it beyond 1024: 8 heads of 75600 tokens, 259 -> 161 us per call.)
+//   2. ordered compaction with a ballot per 32 keys; of the keys equal to T only as many as are missing, the lowest
+//      indices first (a tie goes to the lower block index).
 template <int KPT>
 __global__ void __launch_bounds__(128)
-topk_pick_row_kernel(const uint32_t* __restrict__ score, int nKb, int kk, int32_t* __restrict__ row_ptr,
-                     int32_t* __restrict__ col_idx, long long rows_total)
+topk_pick_warp_kernel(const uint32_t* __restrict__ score, int nKb, int kk, int32_t* __restrict__ row_ptr,
+                      int32_t* __restrict__ col_idx, long long rows_total)
 {
-    __shared__ int hist[3][256];
-    __shared__ int wcnt[kPickMaxChunks][4];
-    __shared__ int cut_s;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const long long row = blockIdx.x;
-    hist[0][tid] = 0; hist[0][tid + 128] = 0;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const long long row = (long long)blockIdx.x * 4 + warp;
     grid_dependency_wait();
     grid_launch_dependents();
+    if (row >= rows_total) return;
     const uint32_t* kr = score + row * nKb;
-    uint32_t key[KPT];
-#pragma unroll
-    for (int i = 0; i < KPT; ++i) key[i] = (tid + 128 * i < nKb) ? kr[tid + 128 * i] : 0u;
-    __syncthreads();
-    uint32_t T = 0;
-    int need = kk, n_eq = 0;
-    for (int pass = 0; pass < 4; ++pass) {
-        const int shift = 24 - 8 * pass;
-        const uint32_t mask = pass == 0 ? 0u : (0xffffffffu << (shift + 8));
-        int* h = hist[pass % 3];
-        // for the next pass (that buffer was last read two passes ago: every warp is past the barrier since)
-        hist[(pass + 1) % 3][tid] = 0; hist[(pass + 1) % 3][tid + 128] = 0;
-#pragma unroll
-        for (int i = 0; i < KPT; ++i)
-            if (key[i] != 0u && (key[i] & mask) == T) atomicAdd(&h[(key[i] >> shift) & 255u], 1);
-        __syncthreads();
-        // lane l looks at bins [8 l, 8 l + 8); counts from the top: the lanes above first, then the lane's bins downwards
-        int c[8], sum = 0;
-#pragma unroll
-        for (int i = 0; i < 8; ++i) { c[i] = h[8 * lane + i]; sum += c[i]; }
-        int incl = sum;                                     // this lane's bins and all higher ones
-#pragma unroll
-        for (int off = 1; off < 32; off <<= 1) {
-            const int v = __shfl_down_sync(0xffffffffu, incl, off);
-            if (lane + off < 32) incl += v;
-        }
-        const int above = incl - sum;
-        const bool hit = above < need && incl >= need;     // exactly one lane
-        int bin = 0, above_bin = 0, in_bin = 0;
-        if (hit) {
-            int acc = above;
-#pragma unroll
-            for (int i = 7; i >= 0; --i) {
-                if (acc < need && acc + c[i] >= need) { bin = 8 * lane + i; above_bin = acc; in_bin = c[i]; }
-                acc += c[i];
-            }
-        }
-        const int src = __ffs(__ballot_sync(0xffffffffu, hit)) - 1;
-        bin = __shfl_sync(0xffffffffu, bin, src);
-        above_bin = __shfl_sync(0xffffffffu, above_bin, src);
-        n_eq = __shfl_sync(0xffffffffu, in_bin, src);      // after the last pass: keys equal to the threshold
-        T |= uint32_t(bin) << shift;
-        need -= above_bin;
-    }
-    // `need` of the n_eq keys equal to T belong to the selection: those with the lowest indices
-    int cut = nKb;                                          // equal keys with an index below `cut` are taken
-    if (n_eq > need) {                                      // (uniform over the CTA)
-        if (warp == 0) {
-            int seen = 0;
-            for (int j0 = 0; j0 < nKb && cut == nKb; j0 += 32) {
-                const int j = j0 + lane;
-                const bool eq = j < nKb && kr[j] == T;
-                const unsigned m = __ballot_sync(0xffffffffu, eq);
-                if (seen + __popc(m) >= need) {
-                    // the need-th equal key is in this group: find its lane
-                    unsigned mm = m;
-                    for (int r = seen + 1; r < need; ++r) mm &= mm - 1;       // drop the lowest set bits
-                    cut = j0 + (__ffs(mm) - 1) + 1;
-                }
-                seen += __popc(m);
-            }
-            if (lane == 0) cut_s = cut;
-        }
-        __syncthreads();
-        cut = cut_s;
-    }
-    // ordered compaction
-    bool take[KPT];
+    uint32_t key[KPT], lo = 0xffffffffu, hi = 0;
 #pragma unroll
     for (int i = 0; i < KPT; ++i) {
-        const int j = tid + 128 * i;
-        take[i] = key[i] != 0u && (key[i] > T || (key[i] == T && j < cut));
-        const unsigned m = __ballot_sync(0xffffffffu, take[i]);
-        if (lane == 0 && i < kPickMaxChunks) wcnt[i][warp] = __popc(m);
+        const bool in = lane + 32 * i < nKb;
+        key[i] = in ? kr[lane + 32 * i] : 0u;
+        if (in) { lo = min(lo, key[i]); hi = max(hi, key[i]); }
     }
-    __syncthreads();
+    lo = __reduce_min_sync(0xffffffffu, lo);
+    hi = __reduce_max_sync(0xffffffffu, hi);
+    const int top = 31 - __clz(lo ^ hi);                    // -1: all keys are the same
+    uint32_t T = top < 0 ? lo : (lo & ~((2u << top) - 1u)); // what all of them have in common: nKb >= kk keys are >= T
+    int at_least = nKb;
+    for (int bit = top; bit >= 0 && at_least != kk; --bit) {
+        const uint32_t c = T | (1u << bit);
+        int n = 0;
+#pragma unroll
+        for (int i = 0; i < KPT; ++i) n += (key[i] >= c) ? 1 : 0;
+        n = __reduce_add_sync(0xffffffffu, n);
+        if (n >= kk) { T = c; at_least = n; }
+    }
+    // at_least keys are >= T.  More than kk: T is the kk-th largest image itself and the surplus is among the equal ones.
+    int need_eq = nKb;
+    if (at_least > kk) {
+        int n = 0;
+#pragma unroll
+        for (int i = 0; i < KPT; ++i) n += (key[i] > T) ? 1 : 0;
+        need_eq = kk - __reduce_add_sync(0xffffffffu, n);
+    }
     int32_t* out = col_idx + row * kk;
-    int base = 0;
+    const unsigned below = (1u << lane) - 1u;
+    int count = 0, eq_seen = 0;
 #pragma unroll
     for (int i = 0; i < KPT; ++i) {
-        const unsigned m = __ballot_sync(0xffffffffu, take[i]);
-        int pos = base;
-        for (int w = 0; w < warp; ++w) pos += wcnt[i][w];
-        if (take[i]) out[pos + __popc(m & ((1u << lane) - 1u))] = tid + 128 * i;
-        base += wcnt[i][0] + wcnt[i][1] + wcnt[i][2] + wcnt[i][3];
+        const bool in = lane + 32 * i < nKb;
+        bool take = in && key[i] >= T;
+        if (at_least > kk) {
+            const bool eq = in && key[i] == T;
+            const unsigned m_eq = __ballot_sync(0xffffffffu, eq);
+            if (eq && eq_seen + __popc(m_eq & below) >= need_eq) take = false;
+            eq_seen += __popc(m_eq);
+        }
+        const unsigned m = __ballot_sync(0xffffffffu, take);
+        if (take) out[count + __popc(m & below)] = lane + 32 * i;
+        count += __popc(m);
     }
-    if (tid == 0) {
+    if (lane == 0) {
         row_ptr[row] = int32_t(row * kk);
         if (row == rows_total - 1) row_ptr[rows_total] = int32_t(rows_total * kk);
     }

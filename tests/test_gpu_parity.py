@@ -1182,3 +1182,23 @@ def test_running_maximum_moves(salad, N, d, Bq, growth):
     assert float((out.double() - want).norm() / want.norm()) <= 1e-2 + err
     want_lse = torch.logsumexp(x, -1)
     assert float((lse.double() - want_lse).abs().max()) <= 2e-3 + 2 * err
+
+
+# Every selection kernel at the ends of its range (128 | 512 | 1024 | 2048 key blocks per row), keeping one block, all but
+# one and all; key means in {-1, 0, 1} and an all-ones query make the scores small integers, exact in any order and
+# with many ties: the expected set follows from a stable sort.
+@pytest.mark.parametrize("nKb", [1, 31, 128, 129, 512, 513, 1024, 1025, 2048, 2049])
+@pytest.mark.parametrize("Bk", [16, 64])
+def test_topk_selection_ranges(salad, nKb, Bk):
+    d, N = 64, (nKb - 1) * Bk + 1                     # the last key block holds one token
+    g = torch.Generator().manual_seed(nKb)
+    value = torch.randint(-1, 2, (2, nKb, d), generator=g).float()
+    k = value.repeat_interleave(Bk, dim=1)[:, :N].reshape(1, 2, N, d).bfloat16().cuda()
+    q = torch.ones(1, 2, N, d, dtype=torch.bfloat16, device="cuda")
+    score = value.sum(2)
+    for kk in sorted({1, max(1, nKb - 1), nKb, max(1, nKb // 10)}):
+        rp, ci = salad.salad_topk_mask_build(q, k, kk, Bk=Bk)
+        nQb = -(-N // 128)
+        want = score.argsort(dim=1, descending=True, stable=True)[:, :kk].sort(dim=1).values
+        assert torch.equal(rp.cpu(), torch.arange(2 * nQb + 1, dtype=torch.int32) * kk)
+        assert torch.equal(ci.cpu().view(2, nQb, kk), want[:, None].expand(2, nQb, kk).int())
