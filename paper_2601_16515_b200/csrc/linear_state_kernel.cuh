@@ -76,7 +76,7 @@ struct StateParams {
 // Post-tuning branch dropping (Sec. 4.3): the linear branch of a batch item is skipped when its
 // dynamic scale is below the threshold.  Decided on the device, so no host synchronisation.
 __device__ __forceinline__ bool branch_dropped(const float* dyn_scale, float tau, int b) {
-    return dyn_scale != nullptr && __ldg(dyn_scale + b) < tau;
+    return dyn_scale != nullptr && dyn_scale[b] < tau;
 }
 
 template <int D, bool OVERLAP, bool ROPE>
@@ -93,11 +93,12 @@ salad_linear_state_kernel(const __grid_constant__ CUtensorMap map_k, const __gri
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     const uint32_t s_base = smem_u32(smem);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    // First kernel of its call: set up while the kernel before the call drains, and waits for it here.
+    grid_dependency_wait();
     if (int(blockIdx.x) < p.order_ctas) {
         // Ordering CTA.  Its results are written, and pushed to the L2, before it lets the kernels after this one go:
         // the attention kernel reads them (from the L2) without a wait of its own.
         if (int(blockIdx.x) < p.Hm) {
-            grid_dependency_wait();    // (the list validator, if there is one)
             order_lists<C::THREADS>(p.row_ptr, p.nQb, p.Hm, blockIdx.x, p.order, p.ws_status, p.user_status,
                                     p.clear_status, reinterpret_cast<int*>(smem));
             __threadfence();
@@ -107,8 +108,7 @@ salad_linear_state_kernel(const __grid_constant__ CUtensorMap map_k, const __gri
         return;
     }
     const int chunk = (blockIdx.x - p.order_ctas) % p.chunks, bh = (blockIdx.x - p.order_ctas) / p.chunks;
-    // First kernel of a linear-only call (an ordinary launch, so everything before it in the stream is done):
-    // its first CTA, which is in the first wave, clears the status words at once; a CTA sets them only after
+    // First kernel of a linear-only call: its first CTA, which is in the first wave, clears the status words at once; a CTA sets them only after
     // a bounded wait of a second has run out.  No state CTA reads them.
     if (p.order_ctas == 0 && p.clear_status && chunk == 0 && bh == 0 && tid == 0) {
         p.ws_status[0] = 0; p.ws_status[1] = 0;
@@ -119,8 +119,7 @@ salad_linear_state_kernel(const __grid_constant__ CUtensorMap map_k, const __gri
     const int kb1 = min(p.nKb, kb0 + p.blocks_per_chunk);
     const int nblk = max(0, kb1 - kb0);
 
-    // K and V are inputs of the call, not products of the kernel before this one (the list validator, if any): the
-    // producer thread starts the first loads at once, ahead of the set-up below.
+    // the producer thread starts the first loads at once, ahead of the set-up below
     auto load_stage = [&](int g) {
         const int s = g % C::STAGES;
         const uint32_t bar = smem_u32(&full[s]);
@@ -150,7 +149,6 @@ salad_linear_state_kernel(const __grid_constant__ CUtensorMap map_k, const __gri
         reinterpret_cast<uint32_t*>(smem + C::OFF_ONES)[i] = 0x3F803F80u;
     fence_proxy_async_smem();
     if (warp == 1) { tmem_alloc(smem_u32(&tmem_base_slot), C::TMEM_COLS); tmem_relinquish(); }
-    grid_dependency_wait();            // (nothing to wait for in an ordinary launch)
     grid_launch_dependents();
     if (tid == 0) abort_flag = 0;
     tc_fence_before_sync();

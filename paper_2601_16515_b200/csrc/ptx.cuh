@@ -38,7 +38,10 @@ __device__ __forceinline__ bool elect_one() {
 // A kernel launched with the programmatic-stream-serialization attribute may be set up, and its
 // CTAs placed, while the kernel before it in the stream still runs.  grid_dependency_wait() blocks
 // until that kernel has completed and its writes are visible (a no-op for an ordinary launch);
-// everything a kernel here reads or writes comes after it, so the stream order is kept exactly.
+// what that kernel may have written is read, and everything is written, only after it, so the stream order is kept
+// exactly.  The first kernel of a call, which can be on an SM while a foreign kernel still writes the call's inputs,
+// reads them by TMA or ordinary loads through pointers without __restrict__: the read-only path is for data that
+// nobody writes during a kernel's life.
 __device__ __forceinline__ void grid_dependency_wait() {
     asm volatile("griddepcontrol.wait;" ::: "memory");
 }

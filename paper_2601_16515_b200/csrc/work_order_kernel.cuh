@@ -26,9 +26,9 @@ constexpr int kOrderScratchWords = kOrderBins + 32;      // histogram, then one 
 
 // One CTA of THREADS threads (whole warps) for mask head hm; scratch: kOrderScratchWords words of shared memory, 16-byte aligned.
 template <int THREADS>
-__device__ __forceinline__ void order_lists(const int32_t* __restrict__ row_ptr, int nQb, int Hm, int hm,
-                                            int32_t* __restrict__ order, int32_t* __restrict__ ws_status,
-                                            int32_t* __restrict__ user_status, int clear_status, int* scratch) {
+__device__ __forceinline__ void order_lists(const int32_t* row_ptr, int nQb, int Hm, int hm,
+                                            int32_t* order, int32_t* ws_status,
+                                            int32_t* user_status, int clear_status, int* scratch) {
     int* hist = scratch;
     int* total = scratch + kOrderBins;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -43,8 +43,8 @@ __device__ __forceinline__ void order_lists(const int32_t* __restrict__ row_ptr,
 #pragma unroll
             for (int u = 0; u < 8; ++u) {
                 const long long r = r0 + u * THREADS;
-                a[u] = r < rows ? __ldg(row_ptr + r) : 0;
-                b[u] = r < rows ? __ldg(row_ptr + r + 1) : 0;
+                a[u] = r < rows ? row_ptr[r] : 0;
+                b[u] = r < rows ? row_ptr[r + 1] : 0;
             }
 #pragma unroll
             for (int u = 0; u < 8; ++u) bad |= (a[u] < 0 || b[u] < a[u]) ? 1 : 0;
@@ -63,7 +63,7 @@ __device__ __forceinline__ void order_lists(const int32_t* __restrict__ row_ptr,
     const int32_t* rp = row_ptr + size_t(hm) * nQb;
     // the length of a list, clamped to a bin: a corrupted offset must not index outside the histogram
     // (the order written for a rejected mask is never used: the attention kernel of the call returns at once)
-    auto cost_of = [&](int qb) { return max(0, min(kOrderBins - 1, __ldg(rp + qb + 1) - __ldg(rp + qb))); };
+    auto cost_of = [&](int qb) { return max(0, min(kOrderBins - 1, rp[qb + 1] - rp[qb])); };
     for (int qb = tid; qb < nQb; qb += THREADS) atomicAdd(&hist[cost_of(qb)], 1);
     __syncthreads();
     // start position of every cost, largest cost first: an exclusive suffix sum over the bins.  A thread owns PER
@@ -93,10 +93,11 @@ __device__ __forceinline__ void order_lists(const int32_t* __restrict__ row_ptr,
         order[size_t(hm) * nQb + atomicAdd(&hist[cost_of(qb)], 1)] = qb;
 }
 
-__global__ void __launch_bounds__(1024) work_order_kernel(const int32_t* __restrict__ row_ptr, int nQb, int Hm,
-                                                          int32_t* __restrict__ order,
-                                                          int32_t* __restrict__ ws_status,
-                                                          int32_t* __restrict__ user_status, int clear_status) {
+__global__ void __launch_bounds__(1024) work_order_kernel(const int32_t* row_ptr, int nQb, int Hm,
+                                                          int32_t* order,
+                                                          int32_t* ws_status,
+                                                          int32_t* user_status, int clear_status) {
+    grid_dependency_wait();           // the kernel before the call, which may have written the lists
     grid_launch_dependents();         // the attention kernel may be placed now; it waits for this one
     __shared__ alignas(16) int scratch[kOrderScratchWords];
     order_lists<1024>(row_ptr, nQb, Hm, blockIdx.x, order, ws_status, user_status, clear_status, scratch);

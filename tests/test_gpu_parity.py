@@ -1202,3 +1202,76 @@ def test_topk_selection_ranges(salad, nKb, Bk):
         want = score.argsort(dim=1, descending=True, stable=True)[:, :kk].sort(dim=1).values
         assert torch.equal(rp.cpu(), torch.arange(2 * nQb + 1, dtype=torch.int32) * kk)
         assert torch.equal(ci.cpu().view(2, nQb, kk), want[:, None].expand(2, nQb, kk).int())
+
+
+# The first kernel of a call is launched to overlap the kernel before it: whatever writes the call's inputs last (a torch
+# kernel, a device copy, a memset, another stream joined by an event, one of the library's own calls), eagerly and inside
+# a graph, the call must see it; and calls sharing a workspace must not disturb each other, rejected lists and dropped items
+# among them.
+@pytest.mark.parametrize("captured", [False, True])
+def test_calls_see_what_was_written_just_before_them(salad, captured):
+    B, H, N, d = 2, 4, 2000, 128
+    torch.manual_seed(3)
+    src = [[torch.randn(B, H, N, d, device="cuda", dtype=torch.bfloat16) for _ in range(3)] for _ in range(2)]
+    q, k, v = (torch.empty_like(src[0][0]) for _ in range(3))
+    nQb, nKb = -(-N // 128), -(-N // 64)
+    rp = torch.arange(nQb + 1, dtype=torch.int32, device="cuda") * nKb
+    ci = torch.arange(nKb, dtype=torch.int32, device="cuda").repeat(nQb)
+    bad = rp.clone(); bad[1] = -1
+    lam = torch.ones(H, device="cuda")
+    x, w = torch.randn(B, N, 256, device="cuda", dtype=torch.bfloat16), torch.randn(256, device="cuda")
+    w_proj, sb = torch.randn(H * d, H * d, device="cuda", dtype=torch.bfloat16) / 16, torch.ones(B, device="cuda")
+    ws = salad.alloc_workspace(B, H, N, d)
+    side = torch.cuda.Stream()
+
+    def fill(how, new):
+        for dst, t in zip((q, k, v), new):
+            if how == "kernel": torch.mul(t, 1, out=dst)
+            elif how == "copy": dst.copy_(t)
+            else:
+                dst.zero_()
+                dst.add_(t)
+        if how == "stream":                            # the last writer is on another stream
+            side.wait_stream(torch.cuda.current_stream())
+            with torch.cuda.stream(side):
+                for dst, t in zip((q, k, v), new): torch.mul(t, 1, out=dst)
+            torch.cuda.current_stream().wait_stream(side)
+
+    def calls():
+        out = [salad.salad_fused_fwd(q, k, v, rp, ci, 1, lam, salad.salad_dynamic_scale(x, w), workspace=ws)]
+        salad.salad_fused_fwd(q, k, v, bad, ci, 1, lam, sb, workspace=ws)                              # rejected
+        out.append(salad.salad_linear_attn_fwd(q, k, v, workspace=ws))
+        salad.salad_fused_fwd(q, k, v, rp, ci, 1, lam, sb, workspace=ws, drop_tau=2.0)                 # all items dropped
+        out.append(salad.salad_sparse_attn_fwd(q, k, v, rp, ci, 1, workspace=ws))
+        tr, tc = salad.salad_topk_mask_build(q, k, 5)
+        out.append(salad.salad_fused_fwd(q, k, v, tr, tc, B * H, lam, sb, workspace=ws))
+        out.append(salad.salad_proj_combine_fwd(out[2], out[1], w_proj, sb))
+        return out
+
+    want = []
+    for new in src:
+        fill("copy", new)
+        torch.cuda.synchronize()
+        res = []
+        for i in range(5):                             # call by call, the device idle in between
+            torch.cuda.synchronize()
+            res = calls()
+            torch.cuda.synchronize()
+        want.append(res)
+    steps = [(how, i % 2) for i, how in enumerate(["kernel", "copy", "memset", "stream"] * 6)]
+    steps += [(how, 1 - i) for how, i in steps]
+    if captured:
+        graph, got = torch.cuda.CUDAGraph(), []
+        with torch.cuda.graph(graph):
+            for how, i in steps:
+                fill(how, src[i])
+                got.append(calls())
+        for _ in range(3): graph.replay()
+    else:
+        got = []
+        for how, i in steps:
+            fill(how, src[i])
+            got.append(calls())
+    torch.cuda.synchronize()
+    for (how, i), res in zip(steps, got):
+        for a, b in zip(res, want[i]): assert torch.equal(a, b), how
