@@ -1275,3 +1275,10 @@ def test_calls_see_what_was_written_just_before_them(salad, captured):
     torch.cuda.synchronize()
     for (how, i), res in zip(steps, got):
         for a, b in zip(res, want[i]): assert torch.equal(a, b), how
+
+
+# Query tiles of 100, 99, 68 and 40 rows: seven, seven, five and three of the eight softmax warps hold queries, the last of
+# them not all 16 rows.
+@pytest.mark.parametrize("T", [50, 33, 34, 40])
+def test_stswa_partly_filled_tiles(salad, T):
+    test_stswa_through_the_loads(salad, (T, 3, 5), 1, 2, 64, [1, 0], [7 * T, 100])
