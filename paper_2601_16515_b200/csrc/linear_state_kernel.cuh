@@ -92,7 +92,8 @@ salad_linear_state_kernel(const __grid_constant__ CUtensorMap map_k, const __gri
 
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     const uint32_t s_base = smem_u32(smem);
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, lane = tid & 31;
+    const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);   // (known to be the same in every lane: 9.8 -> 9.5 us at 2310 tokens)
     // First kernel of its call: set up while the kernel before the call drains, and waits for it here.
     grid_dependency_wait();
     if (int(blockIdx.x) < p.order_ctas) {
