@@ -295,29 +295,23 @@ int launch_state(const Problem& P, const KvMaps& kv, const Workspace& w, const D
     if (chunks < 1) chunks = 1;
     if (chunks > nKb) chunks = nKb;
     if (int64_t(chunks) * BH > w.slots) chunks = w.slots / BH;
+    // The number of chunks follows from the sizes alone, whatever the call: its sums are then the same bits in
+    // salad_linear_state_fwd and in the fused call that it prepares.  More chunks than eight are cut to eight where
+    // that is the faster: sequences of up to D key blocks (12 heads, D = 128, fused call: 50.9 -> 49.2 us at 8190 tokens,
+    // 92.5 against 92.6 at 16380, 164 against 169 at 32760; two heads: 28.3 -> 22.6 and 30.3 against 33.0 at 8190 and
+    // 16380; D = 64, 12 heads: 25.2 -> 24.3 and 34.9 against 35.3 at 5000 and 8190).
+    if (!P.proj_blocks && chunks > 8 && nKb <= D) chunks = 8;
     // Up to eight chunks per head: the CTAs of a head form a cluster and add their partials through shared memory,
     // which saves the finalize kernel and the partials' way through global memory -- with one CTA per SM only where the
     // clusters of all heads are resident together (clusters of six leave a third of a GPC idle: 24 heads of 900
-    // tokens, linear-only, 23.5 against 19.4 us; with two CTAs per SM, in the fused call, 24.0 -> 20.3).  More
-    // chunks than eight are cut to eight where that is the faster: sequences of up to D key blocks (12 heads, D = 128,
-    // fused call: 50.9 -> 49.2 us at 8190 tokens, 92.5 against 92.6 at 16380, 164 against 169 at 32760; two heads: 28.3
-    // -> 22.6 and 30.3 against 33.0 at 8190 and 16380; D = 64, 12 heads: 25.2 -> 24.3 and 34.9 against 35.3 at 5000 and
-    // 8190), and at D = 128 linear-only calls whose eight-fold split still fills 60 % of the SMs, enough for the
-    // memory system (12 heads of 32760 tokens: state pass 41.8 -> 37.7 us on 96 CTAs instead of 144; at D = 64,
-    // with half the bytes in flight per CTA, 25.2 against 32.8).
+    // tokens, linear-only, 23.5 against 19.4 us; with two CTAs per SM, in the fused call, 24.0 -> 20.3).
     const bool sparse = (P.mode & MODE_SPARSE) != 0;
     const bool overlap = sparse && !P.rope;          // the short-ring variant, two CTAs per SM
     auto clusters = [&](int size) {
         if (P.rope) return max_clusters<salad_linear_state_kernel<D, false, true>>(size, StateCfg<D, false, true>::THREADS, StateCfg<D, false, true>::SMEM_BYTES);
         return max_clusters<salad_linear_state_kernel<D, false, false>>(size, StateCfg<D, false, false>::THREADS, StateCfg<D, false, false>::SMEM_BYTES);
     };
-    bool reduce = !P.proj_blocks;
-    if (reduce && chunks > 8) {
-        reduce = (nKb <= D || (D == 128 && !sparse && 8 * BH * 5 >= dev.sms * 3)) && (overlap || clusters(8) >= BH);
-        if (reduce) chunks = 8;
-    } else if (reduce) {
-        reduce = chunks == 1 || overlap || clusters(chunks) >= BH;
-    }
+    const bool reduce = !P.proj_blocks && chunks <= 8 && (chunks == 1 || overlap || clusters(chunks) >= BH);
     const int bpc = (nKb + chunks - 1) / chunks;
     uint8_t* ws = static_cast<uint8_t*>(P.ws);
     CUtensorMap mr = kv.k;          // unused without a rotation table

@@ -862,6 +862,27 @@ def test_state_pass_as_its_own_call_on_a_side_stream(salad):
     np.testing.assert_allclose(kv.cpu().numpy(), kv_ref, rtol=1e-3, atol=np.abs(kv_ref).max() * 1e-4)
 
 
+# The two-call form gives the bits of the one-call form whatever the split of the sequence: cut to eight chunks, one
+# chunk per key block, more than eight chunks (the finalize kernel), at lengths on both sides of the cut.
+@pytest.mark.parametrize("B,H,N,d", [(1, 12, 900, 128), (1, 12, 8191, 128), (1, 12, 8193, 128), (1, 12, 21 * 30 * 52, 128),
+                                     (1, 16, 8300, 128), (1, 12, 4097, 64), (2, 6, 21 * 30 * 52, 64), (1, 2, 330, 64)])
+def test_prepared_pair_equals_the_one_call(salad, B, H, N, d):
+    torch.manual_seed(B * 1000 + H * 10 + N)
+    q, k, v = (torch.randn(B, H, N, d, device="cuda", dtype=torch.bfloat16) for _ in range(3))
+    nQb = -(-N // 128)
+    rp, ci = torch.arange(nQb + 1, dtype=torch.int32, device="cuda"), torch.arange(nQb, dtype=torch.int32, device="cuda")
+    lam, s = torch.rand(H, device="cuda"), torch.ones(B, device="cuda")
+    whole = salad.salad_fused_fwd(q, k, v, rp, ci, 1, lam, s, drop_tau=0.5)
+    ws = salad.alloc_workspace(B, H, N, d)
+    kv = [torch.full((B, H, d, d), float("nan"), device="cuda") for _ in range(2)]
+    z = [torch.full((B, H, d), float("nan"), device="cuda") for _ in range(2)]
+    salad.salad_linear_state_fwd(k, v, ws, kv_out=kv[0], z_out=z[0])
+    assert torch.equal(salad.salad_fused_prepared_fwd(q, k, v, rp, ci, 1, lam, s, ws, drop_tau=0.5), whole)
+    # ... and so does the linear branch alone
+    salad.salad_linear_attn_fwd(q, k, v, kv_out=kv[1], z_out=z[1])
+    assert torch.equal(kv[0], kv[1]) and torch.equal(z[0], z[1])
+
+
 # ------------------------------------------------------------------------------ degenerate sizes
 
 @pytest.mark.parametrize("B,H,N,d,Bq", [
