@@ -50,7 +50,11 @@ struct StateCfg {
     static_assert(OFF_ZS + (ROPE ? 256 * CH * 32 : 0) <= OFF_ONES, "the partial fits over the stages");
     static constexpr int RELU_THREADS = ROPE ? 256 : 128;   // the rotation doubles the work per element
     static constexpr int THREADS = 64 + RELU_THREADS;
-    static constexpr int TMEM_COLS = 256;
+    // D columns of KV, then the 32 that the read of Z touches.  Tensor memory has 512 columns, and an allocation that finds
+    // too few left waits for another CTA to free its own: as many CTAs as the shared memory admits have theirs at once.
+    static constexpr int TMEM_COLS = (D == 128) ? 256 : 128;
+    static_assert(TMEM_COLS >= D + 32, "KV and Z fit");
+    static_assert(228 * 1024 / (SMEM_BYTES + 1024) * TMEM_COLS <= 512, "every resident CTA gets its tensor memory");
 };
 
 struct StateParams {
@@ -150,11 +154,12 @@ salad_linear_state_kernel(const __grid_constant__ CUtensorMap map_k, const __gri
         reinterpret_cast<uint32_t*>(smem + C::OFF_ONES)[i] = 0x3F803F80u;
     fence_proxy_async_smem();
     if (warp == 1) { tmem_alloc(smem_u32(&tmem_base_slot), C::TMEM_COLS); tmem_relinquish(); }
-    grid_launch_dependents();
     if (tid == 0) abort_flag = 0;
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
+    // Only now, with this CTA's tensor memory at hand: the CTAs of the next kernel hold theirs while they wait for this grid.
+    grid_launch_dependents();
     const uint32_t tmem = tmem_base_slot;
     volatile int* abortp = &abort_flag;
 
@@ -292,11 +297,24 @@ salad_linear_state_kernel(const __grid_constant__ CUtensorMap map_k, const __gri
     }
     }
 
+    tc_fence_before_sync();
+    __syncthreads();
+    if (abort_flag != 0) {
+        if (tid == 0 && abort_flag == 1) {            // a bounded wait of this CTA ran out
+            atomicExch(p.ws_status, SALAD_ERR_TIMEOUT);
+            if (p.user_status) atomicExch(p.user_status, SALAD_ERR_TIMEOUT);
+        }
+        const uint64_t t0 = global_timer_ns();
+        while (global_timer_ns() - t0 < 200000ull) { __nanosleep(1000); }
+        __syncthreads();
+    }
+    if (warp == 1) tmem_dealloc(tmem, C::TMEM_COLS);
+
     if (p.reduce) {
+        // No CTA holds tensor memory here, so one that waits for its peers keeps none of them from getting theirs.
         // The partials of the head's CTAs are in their shared memories.  Every CTA adds the rows of its slice (whole
         // groups of eight key channels) in chunk order, in place: nobody else reads those rows of its own copy.  After
         // an expired wait the numbers are rubbish and the status says so; the barriers are met all the same.
-        __syncthreads();
         cluster_sync_all();
         constexpr int G = D / 8;
         const int a0 = G * chunk / p.chunks * 8, a1 = G * (chunk + 1) / p.chunks * 8;
@@ -334,19 +352,6 @@ salad_linear_state_kernel(const __grid_constant__ CUtensorMap map_k, const __gri
         __syncthreads();
         cluster_sync_all();            // nobody leaves while its partial is being read
     }
-
-    tc_fence_before_sync();
-    __syncthreads();
-    if (abort_flag != 0) {
-        if (tid == 0 && abort_flag == 1) {            // a bounded wait of this CTA ran out
-            atomicExch(p.ws_status, SALAD_ERR_TIMEOUT);
-            if (p.user_status) atomicExch(p.user_status, SALAD_ERR_TIMEOUT);
-        }
-        const uint64_t t0 = global_timer_ns();
-        while (global_timer_ns() - t0 < 200000ull) { __nanosleep(1000); }
-        __syncthreads();
-    }
-    if (warp == 1) tmem_dealloc(tmem, C::TMEM_COLS);
 }
 
 // Sum the partials of each head in chunk order; emit

@@ -1303,3 +1303,42 @@ def test_calls_see_what_was_written_just_before_them(salad, captured):
 @pytest.mark.parametrize("T", [50, 33, 34, 40])
 def test_stswa_partly_filled_tiles(salad, T):
     test_stswa_through_the_loads(salad, (T, 3, 5), 1, 2, 64, [1, 0], [7 * T, 100])
+
+
+# Calls at d = 64 in a chain: state clusters of two, six and eight CTAs are placed while the grid before them, which fills the
+# chip, drains, beside its CTAs and beside those of a second chain on another stream.
+@pytest.mark.parametrize("H", [18, 24, 74])
+def test_state_clusters_on_a_full_chip(salad, H):
+    grid, d = (4, 15, 25), 64
+    N = 4 * 15 * 25
+    torch.manual_seed(H)
+    nQb, nKb = -(-N // 128), -(-N // 64)
+    rp = torch.arange(nQb + 1, dtype=torch.int32, device="cuda") * nKb
+    ci = torch.arange(nKb, dtype=torch.int32, device="cuda").repeat(nQb)
+    flags = [h % 2 for h in range(H)]
+    srp, sci = salad.salad_stswa_mask_build(grid, flags, [N] * H)
+    lam, one = torch.rand(H, device="cuda"), torch.ones(1, device="cuda")
+    sets = [[torch.randn(1, H, N, d, device="cuda", dtype=torch.bfloat16) for _ in range(3)] for _ in range(2)]
+    streams = [torch.cuda.Stream() for _ in range(2)]
+    ws = [salad.alloc_workspace(1, H, N, d) for _ in streams]
+    sws = [torch.empty(int(salad._lib.salad_stswa_workspace_bytes(1, H, *grid, d)), dtype=torch.uint8, device="cuda") for _ in streams]
+    out = torch.empty((2, 12, 2, 1, H, N, d), dtype=torch.bfloat16, device="cuda")
+    torch.cuda.synchronize()
+    for n_streams in (1, 2):
+        out.fill_(float("nan"))
+        torch.cuda.synchronize()
+        for i in range(out.shape[1]):
+            for j in range(n_streams):
+                qkv = sets[(i + j) % 2]
+                salad.salad_fused_fwd(*qkv, rp, ci, 1, lam, one, out=out[j, i, 0], workspace=ws[j], stream=streams[j])
+                salad.salad_fused_stswa_fwd(*qkv, grid, flags, srp, sci, lam, one, out=out[j, i, 1], workspace=sws[j],
+                                            stream=streams[j])
+        torch.cuda.synchronize()
+        for which, (q, k, v) in enumerate(sets):
+            x = (q.double() @ k.double().transpose(2, 3) / d ** 0.5).softmax(-1) @ v.double()
+            qr, kr = q.double().clamp_min(0), k.double().clamp_min(0)
+            x += lam.double()[:, None, None] * (qr @ (kr.transpose(2, 3) @ v.double())) / (qr @ kr.sum(2)[..., None] + 1e-6)
+            for kind in range(2):                      # fused_fwd, fused_stswa_fwd
+                got = [out[j, i, kind] for j in range(n_streams) for i in range(out.shape[1]) if (i + j) % 2 == which]
+                assert float((got[0].double() - x).norm() / x.norm()) <= REL_L2
+                for g in got[1:]: assert torch.equal(g, got[0])
