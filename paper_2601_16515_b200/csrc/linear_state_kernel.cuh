@@ -83,6 +83,13 @@ __device__ __forceinline__ bool branch_dropped(const float* dyn_scale, float tau
     return dyn_scale != nullptr && dyn_scale[b] < tau;
 }
 
+// Four floats of a caller's optional output, whose base need not be aligned to more than a float.
+__device__ __forceinline__ void store_user_f4(float* base, size_t index, const float4& v) {
+    float* dst = base + index;                       // index is a multiple of four
+    if ((reinterpret_cast<uintptr_t>(base) & 15u) == 0) *reinterpret_cast<float4*>(dst) = v;
+    else { dst[0] = v.x; dst[1] = v.y; dst[2] = v.z; dst[3] = v.w; }
+}
+
 template <int D, bool OVERLAP, bool ROPE>
 __global__ void __launch_bounds__(64 + (ROPE ? 256 : 128))
 salad_linear_state_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v,
@@ -328,7 +335,7 @@ salad_linear_state_kernel(const __grid_constant__ CUtensorMap map_k, const __gri
 #pragma unroll
             for (int r = 0; r < 8; ++r) if (r < p.chunks) { s.x += v[r].x; s.y += v[r].y; s.z += v[r].z; s.w += v[r].w; }
             *reinterpret_cast<float4*>(mine + a * C::KS + c) = s;
-            if (p.kv_out) *reinterpret_cast<float4*>(p.kv_out + (size_t(bh) * D + a) * D + c) = s;
+            if (p.kv_out) store_user_f4(p.kv_out, (size_t(bh) * D + a) * D + c, s);
         }
         if (chunk == 0 && tid < D / 4) {
             float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -337,7 +344,7 @@ salad_linear_state_kernel(const __grid_constant__ CUtensorMap map_k, const __gri
                 s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w;
             }
             *reinterpret_cast<float4*>(p.z_ws + size_t(bh) * D + tid * 4) = s;
-            if (p.z_out) *reinterpret_cast<float4*>(p.z_out + size_t(bh) * D + tid * 4) = s;
+            if (p.z_out) store_user_f4(p.z_out, size_t(bh) * D + tid * 4, s);
         }
         __syncthreads();
         // the transposed bf16 copy: eight key channels of one value channel per thread

@@ -1342,3 +1342,30 @@ def test_state_clusters_on_a_full_chip(salad, H):
                 got = [out[j, i, kind] for j in range(n_streams) for i in range(out.shape[1]) if (i + j) % 2 == which]
                 assert float((got[0].double() - x).norm() / x.norm()) <= REL_L2
                 for g in got[1:]: assert torch.equal(g, got[0])
+
+
+# The optional fp32 outputs at any float's address: every entry point that has them, state added over a cluster and by the
+# finalize kernel.
+@pytest.mark.parametrize("B,H,N,d", [(1, 2, 700, 64), (1, 3, 1000, 128), (1, 2, 64 * 64 + 1, 64), (1, 2, 128 * 64 + 1, 128)])
+@pytest.mark.parametrize("offset", [1, 2, 3])
+def test_state_outputs_at_any_float(salad, B, H, N, d, offset):
+    torch.manual_seed(N)
+    q, k, v = (torch.randn(B, H, N, d, device="cuda", dtype=torch.bfloat16) for _ in range(3))
+    rope = torch.zeros((N, d // 2, 2), dtype=torch.float16, device="cuda")
+    rope[..., 0] = 1
+    ws = salad.alloc_workspace(B, H, N, d)
+    calls = (lambda **kw: salad.salad_linear_attn_fwd(q, k, v, workspace=ws, **kw),
+             lambda **kw: salad.salad_linear_attn_rope_fwd(q, k, v, rope, workspace=ws, **kw),
+             lambda **kw: salad.salad_linear_attn_fwd_noalloc(q, k, v, **kw),
+             lambda **kw: salad.salad_linear_state_fwd(k, v, ws, **kw))
+    for call in calls:
+        got = []
+        for off in (0, offset):
+            kv = torch.full((B * H * d * d + 8,), -7.0, device="cuda")
+            z = torch.full((B * H * d + 8,), -7.0, device="cuda")
+            call(kv_out=kv[off:off + B * H * d * d], z_out=z[off:off + B * H * d])
+            for t, n in ((kv, B * H * d * d), (z, B * H * d)):
+                got.append(t[off:off + n])
+                assert bool((t[:off] == -7.0).all()) and bool((t[off + n:] == -7.0).all())
+        assert torch.equal(got[0], got[2]) and torch.equal(got[1], got[3])
+        assert not bool((got[0] == -7.0).any()) and not bool((got[1] == -7.0).any())
