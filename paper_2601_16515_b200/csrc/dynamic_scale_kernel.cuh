@@ -79,12 +79,12 @@ dynamic_scale_partial_kernel(const uint4* __restrict__ x, const float* __restric
 }
 
 __global__ void __launch_bounds__(32)
-dynamic_scale_finalize_kernel(const float* __restrict__ partial, int G, int N, float* __restrict__ s_out)
+dynamic_scale_finalize_kernel(const float* partial, int G, int N, float* __restrict__ s_out)
 {
     const int b = blockIdx.x, lane = threadIdx.x;
     grid_dependency_wait();
     float s = 0.f;
-    for (int g = lane; g < G; g += 32) s += partial[size_t(b) * G + g];     // fixed assignment and order
+    for (int g = lane; g < G; g += 32) s += __ldcg(partial + size_t(b) * G + g);     // fixed assignment and order
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
     if (lane == 0) s_out[b] = s / float(N);

@@ -212,7 +212,8 @@ salad_linear_apply_kernel(const __grid_constant__ CUtensorMap map_q, const __gri
                 // Z of the new head into the other buffer; nobody reads that one any more (each
                 // thread arrives here only after its last read of the head before the previous one)
                 zb = n_z & 1;
-                for (int a = row; a < D; a += 128) z_s[zb][a] = __ldg(p.z + size_t(bh) * D + a);
+                // (an ordinary load: not __ldg, the kernel before wrote it during this one's life; __ldcg costs 2 us of 86)
+                for (int a = row; a < D; a += 128) z_s[zb][a] = p.z[size_t(bh) * D + a];
                 mbar_arrive(smem_u32(&bars.z_ready[zb]));
                 ok = mbar_wait(smem_u32(&bars.z_ready[zb]), (n_z >> 1) & 1, abortp);
                 if (!ok) break;

@@ -361,13 +361,26 @@ salad_linear_state_kernel(const __grid_constant__ CUtensorMap map_k, const __gri
     }
 }
 
+// The partials of one channel of Z, in chunk order; sixteen loads are issued before the first add.
+__device__ __forceinline__ float sum_z(const float* src, int chunks, int stride) {
+    float s = 0.f;
+    for (int ch0 = 0; ch0 < chunks; ch0 += 16) {
+        float v[16];
+#pragma unroll
+        for (int u = 0; u < 16; ++u) v[u] = (ch0 + u < chunks) ? __ldcg(src + size_t(ch0 + u) * stride) : 0.f;
+#pragma unroll
+        for (int u = 0; u < 16; ++u) s += v[u];
+    }
+    return s;
+}
+
 // Sum the partials of each head in chunk order; emit
 //   kv_out  fp32 [BH][D][D]  (optional)      z fp32 [BH][D]  (+ optional user copy)
 //   kvt     bf16 [BH][D][D]  transposed: kvt[c][a] = KV[a][c], the K-major B operand of
 //           num = ReLU(Q) KV in the fused kernel.
 template <int D, int ROWS>
 __global__ void __launch_bounds__(32 * ROWS)
-salad_linear_finalize_kernel(const float* __restrict__ kv_part, const float* __restrict__ z_part, int chunks,
+salad_linear_finalize_kernel(const float* kv_part, const float* z_part, int chunks,
                              float* __restrict__ kv_out, float* __restrict__ z_ws, float* __restrict__ z_out,
                              __nv_bfloat16* __restrict__ kvt, const float* __restrict__ dyn_scale, float drop_tau, int H)
 {
@@ -396,7 +409,7 @@ salad_linear_finalize_kernel(const float* __restrict__ kv_part, const float* __r
         for (int ch0 = 0; ch0 < chunks; ch0 += 16) {
             float v[16];
 #pragma unroll
-            for (int u = 0; u < 16; ++u) v[u] = (ch0 + u < chunks) ? src[size_t(ch0 + u) * D * D] : 0.f;
+            for (int u = 0; u < 16; ++u) v[u] = (ch0 + u < chunks) ? __ldcg(src + size_t(ch0 + u) * D * D) : 0.f;
 #pragma unroll
             for (int u = 0; u < 16; u += 4) {
                 if (ch0 + u + 4 <= full) { s0 += v[u]; s1 += v[u + 1]; s2 += v[u + 2]; s3 += v[u + 3]; }
@@ -414,8 +427,7 @@ salad_linear_finalize_kernel(const float* __restrict__ kv_part, const float* __r
     if (blockIdx.x == 0 && blockIdx.y == 0) {
         for (int a = ty * 32 + tx; a < D; a += 32 * ROWS) {
             const float* src = z_part + size_t(bh) * chunks * D + a;
-            float s = 0.f;
-            for (int ch = 0; ch < chunks; ++ch) s += src[size_t(ch) * D];
+            const float s = sum_z(src, chunks, D);
             z_ws[size_t(bh) * D + a] = s;
             if (z_out) z_out[size_t(bh) * D + a] = s;
         }
@@ -439,7 +451,7 @@ salad_linear_finalize_kernel(const float* __restrict__ kv_part, const float* __r
 // that has started early: 4 KB of shared memory and few registers, so that all three fit.
 template <int D>
 __global__ void __launch_bounds__(256)
-salad_linear_finalize_proj_kernel(const float* __restrict__ kv_part, const float* __restrict__ z_part, int chunks,
+salad_linear_finalize_proj_kernel(const float* kv_part, const float* z_part, int chunks,
                                   const __nv_bfloat16* __restrict__ w, float* __restrict__ kv_out,
                                   float* __restrict__ z_ws, float* __restrict__ z_out, __nv_bfloat16* __restrict__ kvt,
                                   const float* __restrict__ dyn_scale, float drop_tau, int H)
@@ -460,7 +472,7 @@ salad_linear_finalize_proj_kernel(const float* __restrict__ kv_part, const float
             for (int ch0 = 0; ch0 < chunks; ch0 += 16) {
                 float pv[16];
 #pragma unroll
-                for (int j = 0; j < 16; ++j) pv[j] = (ch0 + j < chunks) ? src[size_t(ch0 + j) * D * D] : 0.f;
+                for (int j = 0; j < 16; ++j) pv[j] = (ch0 + j < chunks) ? __ldcg(src + size_t(ch0 + j) * D * D) : 0.f;
 #pragma unroll
                 for (int j = 0; j < 16; j += 2) { s0 += pv[j]; s1 += pv[j + 1]; }
             }
@@ -508,8 +520,7 @@ salad_linear_finalize_proj_kernel(const float* __restrict__ kv_part, const float
     if (blockIdx.x == 0) {
         for (int a = tid; a < D; a += 256) {
             const float* src = z_part + size_t(bh) * chunks * D + a;
-            float sum = 0.f;
-            for (int ch = 0; ch < chunks; ++ch) sum += src[size_t(ch) * D];
+            const float sum = sum_z(src, chunks, D);
             z_ws[size_t(bh) * D + a] = sum;
             if (z_out) z_out[size_t(bh) * D + a] = sum;
         }

@@ -39,9 +39,11 @@ __device__ __forceinline__ bool elect_one() {
 // CTAs placed, while the kernel before it in the stream still runs.  grid_dependency_wait() blocks
 // until that kernel has completed and its writes are visible (a no-op for an ordinary launch);
 // what that kernel may have written is read, and everything is written, only after it, so the stream order is kept
-// exactly.  The first kernel of a call, which can be on an SM while a foreign kernel still writes the call's inputs,
-// reads them by TMA or ordinary loads through pointers without __restrict__: the read-only path is for data that
-// nobody writes during a kernel's life.
+// exactly.  Such a kernel can be on an SM while the one before it still writes what it is going to read, so it reads
+// that by TMA, cp.async, __ldcg or ordinary loads, all of it through pointers without const __restrict__: the
+// read-only path (__ldg and what the compiler turns into it) is for data that nobody writes during a kernel's life.  This
+// holds for the products of the kernel before (partial states, Z, block means, scores, partial sums) and, in the first
+// kernel of a call, for the call's inputs.
 __device__ __forceinline__ void grid_dependency_wait() {
     asm volatile("griddepcontrol.wait;" ::: "memory");
 }

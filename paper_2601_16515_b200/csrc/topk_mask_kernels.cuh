@@ -155,7 +155,7 @@ constexpr int kScoreSmemBytes = 2 * kScoreChunk * (kScoreRows + kScoreTile) * 4;
 //   qmean  [BH][nQb][d]      kmeanT [BH][d][ldk] (ldk a multiple of 128: whole tiles are readable)
 //   score  [BH][nQb][nKb]    images of s[i][j] = sum_c qmean[i][c] * kmean[j][c], c ascending
 __global__ void __launch_bounds__(128)
-topk_score_kernel(const float* __restrict__ qmean, const float* __restrict__ kmeanT, int nQb, int nKb, int ldk,
+topk_score_kernel(const float* qmean, const float* kmeanT, int nQb, int nKb, int ldk,
                   int d, uint32_t* __restrict__ score)
 {
     extern __shared__ __align__(16) float sc_smem[];
@@ -184,7 +184,7 @@ topk_score_kernel(const float* __restrict__ qmean, const float* __restrict__ kme
     auto fetch_q = [&](int chunk) {
 #pragma unroll
         for (int e = 0; e < QV; ++e)
-            qnext[e] = __ldg(reinterpret_cast<const float4*>(qsrc + chunk * kScoreChunk) + tid / kScoreRows + e * (128 / kScoreRows));
+            qnext[e] = __ldcg(reinterpret_cast<const float4*>(qsrc + chunk * kScoreChunk) + tid / kScoreRows + e * (128 / kScoreRows));
     };
     auto store_q = [&](int stage) {
         float* As = sc_smem + stage * STAGE;
@@ -252,7 +252,7 @@ topk_score_kernel(const float* __restrict__ qmean, const float* __restrict__ kme
 // The lane's share of a row is re-read (from L1/L2) in every pass: this is the kernel for rows too long for
 // topk_pick_warp_kernel below (more than 2048 key blocks).
 __global__ void __launch_bounds__(128)
-topk_pick_kernel(const uint32_t* __restrict__ score, int nKb, int kk, int32_t* __restrict__ row_ptr,
+topk_pick_kernel(const uint32_t* score, int nKb, int kk, int32_t* __restrict__ row_ptr,
                  int32_t* __restrict__ col_idx, long long rows_total)
 {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -316,7 +316,7 @@ topk_pick_kernel(const uint32_t* __restrict__ score, int nKb, int kk, int32_t* _
 //      indices first (a tie goes to the lower block index).
 template <int KPT>
 __global__ void __launch_bounds__(128)
-topk_pick_warp_kernel(const uint32_t* __restrict__ score, int nKb, int kk, int32_t* __restrict__ row_ptr,
+topk_pick_warp_kernel(const uint32_t* score, int nKb, int kk, int32_t* __restrict__ row_ptr,
                       int32_t* __restrict__ col_idx, long long rows_total)
 {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -329,7 +329,7 @@ topk_pick_warp_kernel(const uint32_t* __restrict__ score, int nKb, int kk, int32
 #pragma unroll
     for (int i = 0; i < KPT; ++i) {
         const bool in = lane + 32 * i < nKb;
-        key[i] = in ? kr[lane + 32 * i] : 0u;
+        key[i] = in ? __ldcg(kr + lane + 32 * i) : 0u;
         if (in) { lo = min(lo, key[i]); hi = max(hi, key[i]); }
     }
     lo = __reduce_min_sync(0xffffffffu, lo);

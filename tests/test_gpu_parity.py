@@ -1369,3 +1369,47 @@ def test_state_outputs_at_any_float(salad, B, H, N, d, offset):
                 assert bool((t[:off] == -7.0).all()) and bool((t[off + n:] == -7.0).all())
         assert torch.equal(got[0], got[2]) and torch.equal(got[1], got[3])
         assert not bool((got[0] == -7.0).any()) and not bool((got[1] == -7.0).any())
+
+
+# Calls of each kind in a chain on one workspace, two sets of inputs in alternation and no other launch in between: every
+# kernel starts while the one before it writes what it reads, over the same addresses as the call before.
+@pytest.mark.parametrize("d", [64, 128])
+def test_products_of_the_kernel_before_are_fresh(salad, d):
+    B, H = 1, 4
+    torch.manual_seed(d)
+    N_max = 64 * 128 + 100                                # linear state by the finalize kernel; 700 tokens: over a cluster
+    ws = salad.alloc_workspace(B, H, N_max, d)
+    lam, s = torch.rand(H, device="cuda"), torch.rand(B, device="cuda")
+    dws = torch.empty(salad.DYN_SCALE_WS_BYTES, dtype=torch.uint8, device="cuda")
+    tws = torch.empty(1 << 24, dtype=torch.uint8, device="cuda")
+    blocks = torch.randn(H, d, d, device="cuda", dtype=torch.bfloat16) / d ** 0.5
+    for N in (700, N_max):
+        sets = [[torch.randn(B, H, N, d, device="cuda", dtype=torch.bfloat16) * (1 + i) for _ in range(3)] for i in range(2)]
+        xs = [torch.randn(B, N, 256, device="cuda", dtype=torch.bfloat16) * (1 + i) for i in range(2)]
+        w = torch.randn(256, device="cuda")
+        rope = salad.salad_rope3d_table_build(1, 1, N, d)
+        nQb, nKb = -(-N // 128), -(-N // 64)
+        rp, ci = torch.arange(nQb + 1, dtype=torch.int32, device="cuda"), torch.arange(nQb, dtype=torch.int32, device="cuda")
+        trp = torch.empty(H * nQb + 1, dtype=torch.int32, device="cuda")
+        tci = torch.empty(H * nQb * 3, dtype=torch.int32, device="cuda")
+        tail = (rp, ci, 1, lam, s)
+        for call in (lambda i, o: salad.salad_linear_attn_fwd(*sets[i], out=o, workspace=ws),
+                     lambda i, o: salad.salad_linear_attn_rope_fwd(*sets[i], rope, out=o, workspace=ws),
+                     lambda i, o: salad.salad_fused_fwd(*sets[i], *tail, out=o, workspace=ws),
+                     lambda i, o: salad.salad_fused_rope_fwd(*sets[i], *tail, rope, out=o, workspace=ws),
+                     lambda i, o: salad.salad_fused_proj_fwd(*sets[i], rp, ci, 1, blocks, s, out=o, workspace=ws),
+                     lambda i, o: salad.salad_fused_fwd(*sets[i], rp, ci, 1, lam, salad.salad_dynamic_scale(
+                         xs[i], w, out=s_out, workspace=dws), out=o, workspace=ws),
+                     lambda i, o: salad.salad_fused_fwd(*sets[i], *salad.salad_topk_mask_build(
+                         sets[i][0], sets[i][1], 3, row_ptr=trp, col_idx=tci, workspace=tws), H, lam, s, out=o, workspace=ws)):
+            s_out = torch.empty(B, device="cuda")
+            want = [torch.empty_like(sets[0][0]) for _ in range(2)]
+            got = torch.empty((16, *sets[0][0].shape), dtype=torch.bfloat16, device="cuda")
+            for i in range(2):
+                torch.cuda.synchronize()
+                call(i, want[i])
+                torch.cuda.synchronize()
+            for n in range(16): call(n % 2, got[n])
+            torch.cuda.synchronize()
+            for n in range(16): assert torch.equal(got[n], want[n % 2])
+            assert not torch.equal(want[0], want[1])
