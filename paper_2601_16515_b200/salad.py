@@ -131,6 +131,8 @@ _current_raw_stream = torch._C._cuda_getCurrentRawStream
 def _call(name: str, anchor: torch.Tensor, stream, *args):
     """One library call whose last argument is the stream, on the device of `anchor`."""
     index = anchor.get_device()
+    if index < 0:
+        raise ValueError(f"Expected a cuda device, but got: {anchor.device}")
     if stream is None:
         stream = _current_raw_stream(index)
     else:

@@ -117,3 +117,11 @@ def test_no_gpu_means_error_not_fallback(lib):
     rc = L.salad_sparse_attn_fwd(fake, fake, fake, fake, None, 1, 2, 1024, 64, 64, 64, fake, fake, 1, 0.0,
                                  fake, ws_bytes, None, None)
     assert rc == lib.SALAD_ERR_CUDA
+
+
+def test_a_cpu_device_is_refused(lib):
+    # the builders allocate their outputs on the device they are given: host memory must not reach a kernel
+    for call in (lambda: lib.salad_mask_build(2, 4, 4, 64, 64, [(1, 1, 1)], device="cpu"),
+                 lambda: lib.salad_stswa_mask_build((2, 4, 4), [0, 1], [3, 3], device="cpu")):
+        with pytest.raises(ValueError, match="Expected a cuda device"):
+            call()
