@@ -123,9 +123,8 @@ def _ptr(t: Optional[torch.Tensor]):
 
 # A call is issued on the device of its tensors, on that device's current stream unless the caller names one.  The
 # handles come straight from torch's C layer: the Python device context and Stream objects cost 6 us a call, more than
-# the launches of the smallest calls.
-_current_device = torch._C._cuda_getDevice
-_current_raw_stream = torch._C._cuda_getCurrentRawStream
+# the launches of the smallest calls.  (Looked up in the call: a torch built without CUDA has no such functions, and the
+# host-only entry points work there.)
 
 
 def _call(name: str, anchor: torch.Tensor, stream, *args):
@@ -134,10 +133,10 @@ def _call(name: str, anchor: torch.Tensor, stream, *args):
     if index < 0:
         raise ValueError(f"Expected a cuda device, but got: {anchor.device}")
     if stream is None:
-        stream = _current_raw_stream(index)
+        stream = torch._C._cuda_getCurrentRawStream(index)
     else:
         stream = stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
-    if _current_device() == index:
+    if torch._C._cuda_getDevice() == index:
         rc = getattr(_lib, name)(*args, stream)
     else:
         with torch.cuda.device(index):

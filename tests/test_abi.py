@@ -3,6 +3,8 @@ header declares, and rejects bad arguments on the host before anything could be 
 import ctypes
 import os
 import re
+import subprocess
+import sys
 
 import pytest
 
@@ -125,3 +127,11 @@ def test_a_cpu_device_is_refused(lib):
                  lambda: lib.salad_stswa_mask_build((2, 4, 4), [0, 1], [3, 3], device="cpu")):
         with pytest.raises(ValueError, match="Expected a cuda device"):
             call()
+
+
+def test_host_only_entry_points_need_no_cuda_torch(lib):
+    code = ("import torch\n"
+            "for name in ('_cuda_getDevice', '_cuda_getCurrentRawStream'): delattr(torch._C, name)\n"
+            "from paper_2601_16515_b200 import salad\n"
+            "assert salad.salad_workspace_bytes(1, 2, 1024, 64, 64, 64) > 0 and salad.status_string(0) == 'SALAD_OK'\n")
+    subprocess.run([sys.executable, "-c", code], cwd=ROOT, check=True)
