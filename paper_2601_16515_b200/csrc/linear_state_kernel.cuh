@@ -15,7 +15,7 @@
 // emits the fp32 state plus the bf16, transposed copy that the fused attention kernel
 // multiplies with ReLU(Q).
 // Up to eight chunks per head: the CTAs of a head are one cluster; every CTA leaves its partial in its own shared memory
-// and adds a slice of the rows over the cluster (distributed shared memory), also in chunk order.  No second launch and
+// and adds a slice of the rows over the cluster (distributed shared memory), in the same order.  No second launch and
 // no round trip of the partials: 10.2 -> 8.4 us for the state pass of 12 heads of 900 tokens, 41.7 -> 37.7 us at 32760.
 //
 // ROPE variant (linear branch with a rotary position embedding, Sec. 4.1): the ReLU warps rotate the
@@ -82,6 +82,18 @@ struct StateParams {
 __device__ __forceinline__ bool branch_dropped(const float* dyn_scale, float tau, int b) {
     return dyn_scale != nullptr && dyn_scale[b] < tau;
 }
+
+// The sum of a head's partials of KV, the same bits wherever it is formed (over the cluster or by the finalize kernel):
+// ((p0+p4+..)+(p1+p5+..))+((p2+..)+(p3+..)), the chunks % 4 last partials into the first sum.
+struct PartialSum {
+    float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
+    // partials first .. first + 3 (first a multiple of four) of `chunks`; absent ones are zero
+    __device__ __forceinline__ void add(int first, int chunks, float a, float b, float c, float d) {
+        if (first + 4 <= chunks) { s0 += a; s1 += b; s2 += c; s3 += d; }
+        else if (first < chunks) { s0 += a; s0 += b; s0 += c; }
+    }
+    __device__ __forceinline__ float total() const { return (s0 + s1) + (s2 + s3); }
+};
 
 // Four floats of a caller's optional output, whose base need not be aligned to more than a float.
 __device__ __forceinline__ void store_user_f4(float* base, size_t index, const float4& v) {
@@ -320,7 +332,7 @@ salad_linear_state_kernel(const __grid_constant__ CUtensorMap map_k, const __gri
     if (p.reduce) {
         // No CTA holds tensor memory here, so one that waits for its peers keeps none of them from getting theirs.
         // The partials of the head's CTAs are in their shared memories.  Every CTA adds the rows of its slice (whole
-        // groups of eight key channels) in chunk order, in place: nobody else reads those rows of its own copy.  After
+        // groups of eight key channels), in place: nobody else reads those rows of its own copy.  After
         // an expired wait the numbers are rubbish and the status says so; the barriers are met all the same.
         cluster_sync_all();
         constexpr int G = D / 8;
@@ -329,11 +341,18 @@ salad_linear_state_kernel(const __grid_constant__ CUtensorMap map_k, const __gri
         for (int i = tid; i < (a1 - a0) * (D / 4); i += C::THREADS) {
             const int a = a0 + i / (D / 4), c = (i % (D / 4)) * 4;
             const uint32_t off = s_base + (a * C::KS + c) * 4;
-            float4 v[8], s = make_float4(0.f, 0.f, 0.f, 0.f);
+            float4 v[8];
 #pragma unroll
-            for (int r = 0; r < 8; ++r) if (r < p.chunks) v[r] = ld_cluster_f4(map_to_cta(off, r));
+            for (int r = 0; r < 8; ++r) v[r] = r < p.chunks ? ld_cluster_f4(map_to_cta(off, r)) : make_float4(0.f, 0.f, 0.f, 0.f);
+            PartialSum sx, sy, sz, sw;
 #pragma unroll
-            for (int r = 0; r < 8; ++r) if (r < p.chunks) { s.x += v[r].x; s.y += v[r].y; s.z += v[r].z; s.w += v[r].w; }
+            for (int r = 0; r < 8; r += 4) {
+                sx.add(r, p.chunks, v[r].x, v[r + 1].x, v[r + 2].x, v[r + 3].x);
+                sy.add(r, p.chunks, v[r].y, v[r + 1].y, v[r + 2].y, v[r + 3].y);
+                sz.add(r, p.chunks, v[r].z, v[r + 1].z, v[r + 2].z, v[r + 3].z);
+                sw.add(r, p.chunks, v[r].w, v[r + 1].w, v[r + 2].w, v[r + 3].w);
+            }
+            const float4 s = make_float4(sx.total(), sy.total(), sz.total(), sw.total());
             *reinterpret_cast<float4*>(mine + a * C::KS + c) = s;
             if (p.kv_out) store_user_f4(p.kv_out, (size_t(bh) * D + a) * D + c, s);
         }
@@ -374,7 +393,7 @@ __device__ __forceinline__ float sum_z(const float* src, int chunks, int stride)
     return s;
 }
 
-// Sum the partials of each head in chunk order; emit
+// Sum the partials of each head in a fixed order; emit
 //   kv_out  fp32 [BH][D][D]  (optional)      z fp32 [BH][D]  (+ optional user copy)
 //   kvt     bf16 [BH][D][D]  transposed: kvt[c][a] = KV[a][c], the K-major B operand of
 //           num = ReLU(Q) KV in the fused kernel.
@@ -402,21 +421,16 @@ salad_linear_finalize_kernel(const float* kv_part, const float* z_part, int chun
     for (int r = 0; r < 32 / ROWS; ++r) {
         const int a = a0 + ty + ROWS * r;
         const float* src = kv_part + size_t(bh) * chunks * D * D + size_t(a) * D + c0 + tx;
-        // fixed order: ((p0+p4+..)+(p1+p5+..))+((p2+..)+(p3+..)), the chunks % 4 last partials into the first
-        // sum; sixteen loads are issued before the first add (the kernel is a chain of L2 round trips otherwise)
-        float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
-        const int full = chunks & ~3;
+        // sixteen loads are issued before the first add (the kernel is a chain of L2 round trips otherwise)
+        PartialSum sum;
         for (int ch0 = 0; ch0 < chunks; ch0 += 16) {
             float v[16];
 #pragma unroll
             for (int u = 0; u < 16; ++u) v[u] = (ch0 + u < chunks) ? __ldcg(src + size_t(ch0 + u) * D * D) : 0.f;
 #pragma unroll
-            for (int u = 0; u < 16; u += 4) {
-                if (ch0 + u + 4 <= full) { s0 += v[u]; s1 += v[u + 1]; s2 += v[u + 2]; s3 += v[u + 3]; }
-                else if (ch0 + u < chunks) { s0 += v[u]; s0 += v[u + 1]; s0 += v[u + 2]; }    // absent ones are zero
-            }
+            for (int u = 0; u < 16; u += 4) sum.add(ch0 + u, chunks, v[u], v[u + 1], v[u + 2], v[u + 3]);
         }
-        const float s = (s0 + s1) + (s2 + s3);
+        const float s = sum.total();
         if (kv_out) kv_out[size_t(bh) * D * D + size_t(a) * D + c0 + tx] = s;
         tile[ty + ROWS * r][tx] = s;
     }

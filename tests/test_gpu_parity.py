@@ -865,7 +865,10 @@ def test_state_pass_as_its_own_call_on_a_side_stream(salad):
 # The two-call form gives the bits of the one-call form whatever the split of the sequence: cut to eight chunks, one
 # chunk per key block, more than eight chunks (the finalize kernel), at lengths on both sides of the cut.
 @pytest.mark.parametrize("B,H,N,d", [(1, 12, 900, 128), (1, 12, 8191, 128), (1, 12, 8193, 128), (1, 12, 21 * 30 * 52, 128),
-                                     (1, 16, 8300, 128), (1, 12, 4097, 64), (2, 6, 21 * 30 * 52, 64), (1, 2, 330, 64)])
+                                     (1, 16, 8300, 128), (1, 12, 4097, 64), (2, 6, 21 * 30 * 52, 64), (1, 2, 330, 64),
+                                     # three to eight chunks, where the two calls may add them in different kernels
+                                     (1, 24, 900, 128), (2, 12, 21 * 30 * 52, 128), (1, 24, 5000, 64), (1, 18, 700, 128),
+                                     (1, 40, 3000, 128), (1, 21, 2000, 128), (1, 29, 2000, 64), (1, 74, 300, 128)])
 def test_prepared_pair_equals_the_one_call(salad, B, H, N, d):
     torch.manual_seed(B * 1000 + H * 10 + N)
     q, k, v = (torch.randn(B, H, N, d, device="cuda", dtype=torch.bfloat16) for _ in range(3))
