@@ -32,8 +32,10 @@
  *   - d_status (optional, device int32): set to 0 by a successful launch and to a non-zero
  *     code by a kernel whose bounded internal wait expired (SALAD_ERR_TIMEOUT; the kernel then
  *     returns early instead of hanging) or by the mask checks (SALAD_ERR_BAD_MASK, below); the
- *     remaining kernels of the call then return at once and the outputs are undefined.  Read it
- *     after synchronising the stream.
+ *     kernel of the call that writes the output then returns early and the outputs are undefined.
+ *     (The state pass of a fused call needs nothing of the lists and is not stopped by them: it
+ *     runs, and leaves its state in the workspace, beside the check.)  Read d_status after
+ *     synchronising the stream.
  *   - Mask checks.  The lists are device data, so the host cannot check them before the launch.
  *     Every call with a sparse branch checks, in its first kernel, that the row offsets are
  *     non-negative and non-decreasing (it reads them anyway).  The full contract (offsets

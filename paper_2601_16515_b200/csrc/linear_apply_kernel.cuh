@@ -140,15 +140,17 @@ salad_linear_apply_kernel(const __grid_constant__ CUtensorMap map_q, const __gri
     const uint32_t tmem = tmem_base_slot;
     volatile int* abortp = &abort_flag;
 
-    if (abort_flag == 0) {
     if (warp == 0) {
         // ============================================================== TMA producer
         if (lane == 0) {
             grid_dependency_wait();
-            if (*reinterpret_cast<volatile int32_t*>(p.ws_status) != 0) abort_flag = 2;    // reported by an earlier kernel
+            // A failure reported by an earlier kernel: nothing more is loaded.  Without a state no product is issued and nothing is
+            // stored; the other roles leave at the first wait that this flag ends.
+            const bool failed = *reinterpret_cast<volatile int32_t*>(p.ws_status) != 0;
+            if (failed) *abortp = 2;
             int prev_bh = -1, n_st = 0;
             Walk w = first;
-            for (int j = 0; j < tiles; ++j, w.next()) {
+            for (int j = 0; j < tiles && !failed; ++j, w.next()) {
                 const int bh = w.bh;
                 if (bh != prev_bh) {
                     const int sb = n_st % C::NST;
@@ -314,7 +316,6 @@ salad_linear_apply_kernel(const __grid_constant__ CUtensorMap map_q, const __gri
         }
         if (row == 0) tma_store_wait_read_all();      // the staging tile must outlive the last store's read
     }
-    }  // abort_flag == 0
 
     // ------------------------------------------------------------------ tear-down
     tc_fence_before_sync();

@@ -1416,3 +1416,28 @@ def test_products_of_the_kernel_before_are_fresh(salad, d):
             torch.cuda.synchronize()
             for n in range(16): assert torch.equal(got[n], want[n % 2])
             assert not torch.equal(want[0], want[1])
+
+
+# A failure reported while the state pass runs (the word that an expired wait of it would set, written here from another
+# stream, over and over): the apply kernel stores nothing.  The next call on the workspace is right.
+@pytest.mark.parametrize("d", [64, 128])
+def test_linear_call_stops_on_a_reported_failure(salad, d):
+    B, H, N = 1, 12, 75600
+    torch.manual_seed(d)
+    q, k, v = (torch.randn(B, H, N, d, device="cuda", dtype=torch.bfloat16) for _ in range(3))
+    ws = salad.alloc_workspace(B, H, N, d)
+    want = salad.salad_linear_attn_fwd(q, k, v, workspace=ws)
+    out = torch.full_like(q, -7.0)
+    word = ws[:4].view(torch.int32)
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        for _ in range(1000): word.fill_(salad.SALAD_ERR_TIMEOUT)
+    side = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    with torch.cuda.stream(side):
+        graph.replay()
+    salad.salad_linear_attn_fwd(q, k, v, out=out, workspace=ws)
+    torch.cuda.synchronize()
+    assert int(word.item()) == salad.SALAD_ERR_TIMEOUT
+    assert bool((out == -7.0).all())
+    assert torch.equal(salad.salad_linear_attn_fwd(q, k, v, workspace=ws), want)
