@@ -1151,9 +1151,10 @@ def test_attention_calls_reject_a_broken_mask_without_touching_the_output(salad)
 
 
 # Splits of a head's tokens over a cluster: 1, 3, 6 and 8 CTAs, chunks of unequal length, empty chunks (nine key blocks on
-# eight CTAs), a rotation table, and a sequence one key block beyond the cut (the finalize kernel).
+# eight CTAs), a rotation table, and sequences beyond the cut (9 to 74 chunks, the finalize kernel).
 @pytest.mark.parametrize("B,H,N,d", [(1, 2, 130, 128), (1, 3, 570, 64), (1, 12, 1000, 128), (1, 24, 700, 128),
-                                     (2, 20, 450, 64), (2, 74, 200, 64), (1, 2, 64 * 64 + 1, 64), (1, 2, 128 * 64 + 1, 128)])
+                                     (2, 20, 450, 64), (2, 74, 200, 64), (1, 2, 64 * 64 + 1, 64), (1, 2, 128 * 64 + 1, 128),
+                                     (1, 12, 128 * 64 + 65, 128), (1, 13, 9001, 128), (1, 16, 9100, 128)])
 def test_linear_state_over_a_cluster(salad, B, H, N, d):
     torch.manual_seed(B * 1000 + H * 10 + N)
     q, k, v = (torch.randn(B, H, N, d, device="cuda", dtype=torch.bfloat16) for _ in range(3))
@@ -1183,7 +1184,8 @@ def test_linear_state_over_a_cluster(salad, B, H, N, d):
 
 # Row maxima that move in the middle of a list: by more than the kernel lets pass in every block, in some rows of a
 # warp only, in the ragged last block, downwards (the first block holds the maximum), and by hundreds of powers of two.
-@pytest.mark.parametrize("growth", [9.0, 40.0, -9.0, 300.0])
+# Growing by 1.5 to 5 per block, several blocks stay under the limit, on the old maximum, before one crosses it.
+@pytest.mark.parametrize("growth", [9.0, 40.0, -9.0, 300.0, 1.5, 2.5, 5.0])
 @pytest.mark.parametrize("N,d,Bq", [(64 * 9 + 17, 128, 128), (64 * 4, 64, 64), (130, 128, 128)])
 def test_running_maximum_moves(salad, N, d, Bq, growth):
     torch.manual_seed(N + d)
@@ -1206,6 +1208,33 @@ def test_running_maximum_moves(salad, N, d, Bq, growth):
     assert float((out.double() - want).norm() / want.norm()) <= 1e-2 + err
     want_lse = torch.logsumexp(x, -1)
     assert float((lse.double() - want_lse).abs().max()) <= 2e-3 + 2 * err
+
+
+# One key whose probability against the standing maximum is just under and just over the limit of a thread's sum (2^12, with
+# fifteen others of 1): ln 4081 = 8.314, and 8.3125 and 8.375 are bf16 numbers.  Rows of the same warp without it (zero
+# scores) and with its negative; twice under the limit in a row, over it after that, and far below the maximum once it has moved.
+@pytest.mark.parametrize("peaks", [(8.3125,), (8.375,), (8.3125, 8.3125, 8.375, 8.3125), (0.0, 8.375, 16.625, 16.75, -8.0)])
+@pytest.mark.parametrize("d", [64, 128])
+def test_running_maximum_at_its_limit(salad, d, peaks):
+    torch.manual_seed(d + len(peaks))
+    N = 64 * (len(peaks) + 1)
+    q, k = torch.zeros(1, 1, N, d, device="cuda"), torch.zeros(1, 1, N, d, device="cuda")
+    q[..., 0] = torch.tensor([8.0, 0.0, -8.0, 8.0], device="cuda").repeat(N // 4)
+    for i, x in enumerate(peaks): k[0, 0, 64 * (i + 1) + (26 * i + 5) % 64, 0] = x
+    q, k, v = q.bfloat16(), k.bfloat16(), torch.randn(1, 1, N, d, device="cuda", dtype=torch.bfloat16)
+    nQb, nKb = -(-N // 128), N // 64
+    rp = torch.arange(nQb + 1, dtype=torch.int32, device="cuda") * nKb
+    ci = torch.arange(nKb, dtype=torch.int32, device="cuda").repeat(nQb)
+    lse = torch.empty(1, 1, N, device="cuda")
+    out = salad.salad_sparse_attn_fwd(q, k, v, rp, ci, 1, softmax_scale=0.125, lse=lse)
+    x = q.double() @ k.double().transpose(2, 3) * 0.125
+    want = torch.softmax(x, -1) @ v.double()
+    # bf16 has 8 significant bits: each probability is off by up to 2^-8 of itself, which weighs on |v|, and so is the rounded
+    # output; scores are exact, row sums are fp32 over 64 * 6 keys
+    bound = 2.0 ** -8 * (torch.softmax(x, -1) @ v.double().abs())
+    assert ((out.double() - want).abs() <= bound + 2.0 ** -8 * (want.abs() + bound) + 1e-6).all()
+    assert float((lse.double() - torch.logsumexp(x, -1)).abs().max()) <= 1e-4
+    assert float((out.double() - want).norm() / want.norm()) <= REL_L2
 
 
 # Every selection kernel at the ends of its range (128 | 512 | 1024 | 2048 key blocks per row), keeping one block, all but
@@ -1247,6 +1276,7 @@ def test_calls_see_what_was_written_just_before_them(salad, captured):
     w_proj, sb = torch.randn(H * d, H * d, device="cuda", dtype=torch.bfloat16) / 16, torch.ones(B, device="cuda")
     ws = salad.alloc_workspace(B, H, N, d)
     side = torch.cuda.Stream()
+    untouched = torch.full_like(q, -7.0)               # where the rejected calls would write
 
     def fill(how, new):
         for dst, t in zip((q, k, v), new):
@@ -1261,26 +1291,38 @@ def test_calls_see_what_was_written_just_before_them(salad, captured):
                 for dst, t in zip((q, k, v), new): torch.mul(t, 1, out=dst)
             torch.cuda.current_stream().wait_stream(side)
 
-    def calls():
-        out = [salad.salad_fused_fwd(q, k, v, rp, ci, 1, lam, salad.salad_dynamic_scale(x, w), workspace=ws)]
-        salad.salad_fused_fwd(q, k, v, bad, ci, 1, lam, sb, workspace=ws)                              # rejected
-        out.append(salad.salad_linear_attn_fwd(q, k, v, workspace=ws))
-        salad.salad_fused_fwd(q, k, v, rp, ci, 1, lam, sb, workspace=ws, drop_tau=2.0)                 # all items dropped
-        out.append(salad.salad_sparse_attn_fwd(q, k, v, rp, ci, 1, workspace=ws))
-        tr, tc = salad.salad_topk_mask_build(q, k, 5)
-        out.append(salad.salad_fused_fwd(q, k, v, tr, tc, B * H, lam, sb, workspace=ws))
-        out.append(salad.salad_proj_combine_fwd(out[2], out[1], w_proj, sb))
-        return out
+    def calls(alone):
+        # alone: the device idle before every call, a workspace for each; otherwise one behind the other on one workspace
+        res = []
+
+        def call(f, *args, **kw):
+            if alone: torch.cuda.synchronize()
+            if f in (salad.salad_fused_fwd, salad.salad_linear_attn_fwd, salad.salad_sparse_attn_fwd):
+                kw.update(workspace=salad.alloc_workspace(B, H, N, d) if alone else ws,
+                          status=torch.empty(1, dtype=torch.int32, device="cuda"))
+                res.append(kw["status"])
+            res.append(f(*args, **kw))
+            return res[-1]
+
+        s = call(salad.salad_dynamic_scale, x, w)
+        call(salad.salad_fused_fwd, q, k, v, rp, ci, 1, lam, s)
+        call(salad.salad_fused_fwd, q, k, v, bad, ci, 1, lam, sb, out=untouched)                       # rejected
+        o_l = call(salad.salad_linear_attn_fwd, q, k, v)
+        dropped = call(salad.salad_fused_fwd, q, k, v, rp, ci, 1, lam, sb, drop_tau=2.0)               # all items dropped
+        o_s = call(salad.salad_sparse_attn_fwd, q, k, v, rp, ci, 1)
+        tr, tc = call(salad.salad_topk_mask_build, q, k, 5)
+        res[-1:] = [tr, tc]
+        call(salad.salad_fused_fwd, q, k, v, tr, tc, B * H, lam, sb)
+        call(salad.salad_proj_combine_fwd, o_s, o_l, w_proj, sb)
+        return res, dropped, o_s
 
     want = []
     for new in src:
         fill("copy", new)
+        res, dropped, o_s = calls(alone=True)
         torch.cuda.synchronize()
-        res = []
-        for i in range(5):                             # call by call, the device idle in between
-            torch.cuda.synchronize()
-            res = calls()
-            torch.cuda.synchronize()
+        assert torch.equal(dropped, o_s)
+        assert [int(t.item()) for t in res if t.numel() == 1] == [0, salad.SALAD_ERR_BAD_MASK, 0, 0, 0, 0]
         want.append(res)
     steps = [(how, i % 2) for i, how in enumerate(["kernel", "copy", "memset", "stream"] * 6)]
     steps += [(how, 1 - i) for how, i in steps]
@@ -1289,15 +1331,17 @@ def test_calls_see_what_was_written_just_before_them(salad, captured):
         with torch.cuda.graph(graph):
             for how, i in steps:
                 fill(how, src[i])
-                got.append(calls())
+                got.append(calls(alone=False)[0])
         for _ in range(3): graph.replay()
     else:
         got = []
         for how, i in steps:
             fill(how, src[i])
-            got.append(calls())
+            got.append(calls(alone=False)[0])
     torch.cuda.synchronize()
+    assert bool((untouched == -7.0).all())
     for (how, i), res in zip(steps, got):
+        assert len(res) == len(want[i])
         for a, b in zip(res, want[i]): assert torch.equal(a, b), how
 
 
