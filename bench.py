@@ -441,7 +441,7 @@ def main():
             return {"kernel": kernel, "bound": "hbm", "ms": ms, "algorithmic_bytes": nbytes, "achieved": gbs,
                     "unit": "GB/s", "peak": peaks["hbm_gbs"], "peak_source": peaks["source"] + " copy bandwidth",
                     "frac": gbs / peaks["hbm_gbs"], "frac_of_nominal_8tbs": gbs / 8000.0}
-        extras["linear_branch"] = hbm_record("salad_linear_attn_fwd: state and apply kernels (K, V, Q read, O written)",
+        extras["linear_branch"] = hbm_record("salad_linear_attn_fwd: state (+ finalize beyond eight chunks per head) and apply kernels (K, V, Q read, O written)",
                                              extras["linear_only_ms"], lin_bytes)
         drp, dci = wlmod.dense_csr(wl.nQb, wl.nKb, 1)
         drp_d, dci_d = torch.from_numpy(drp).to(dev), torch.from_numpy(dci).to(dev)

@@ -36,7 +36,7 @@
 // that announces the completion of P V the V-ring stage.
 // The four producer / issuer warps (one warpgroup) hand registers to the eight softmax warps
 // (setmaxnreg: 48 against 96 per thread, all that the block was launched with), which keeps the softmax loop free of
-// spills.
+// spills at D = 128 (at D = 64 the kernel keeps one word on the stack).
 // After the last block the softmax warps apply ReLU to the Q rows in shared memory and compute the
 // linear denominator with plain FMAs; the linear state (bf16, transposed) is loaded over the K
 // ring, which is idle by then; the issuing thread multiplies ReLU(Q) with it, and the epilogue
@@ -139,7 +139,7 @@ salad_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
     const uint32_t s_base = smem_u32(smem);
     const int tid = threadIdx.x, lane = tid & 31;
     // The same as tid >> 5, but known to be the same in every lane, which keeps the roles' branches free of
-    // reconvergence code: with the spill-free 48 registers of the producer warps 638 -> 629 us at 12 heads of 32760 tokens (90 %
+    // reconvergence code: together with 48 registers instead of 40 for the producer warps 638 -> 629 us at 12 heads of 32760 tokens (90 %
     // sparsity, attention alone, at the power limit), 470 -> 451 at d = 64, 35.6 -> 34.7 for 2310 tokens.
     const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
     // The work order (and the verdict on the lists) comes from the first kernel of the call.  Without a linear

@@ -79,8 +79,8 @@ salad_linear_apply_kernel(const __grid_constant__ CUtensorMap map_q, const __gri
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     const uint32_t s_base = smem_u32(smem);
     const int tid = threadIdx.x, lane = tid & 31;
-    // (known to be the same in every lane: no reconvergence code around the roles; 82.3 -> 79.4 us for a linear-only call on
-    // 12 heads of 32760 tokens, most of it here)
+    // (known to be the same in every lane: no reconvergence code around the roles; 87.8 -> 85.7 us for a linear-only call on
+    // 12 heads of 32760 tokens)
     const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
     // contiguous, balanced range of tiles (head-major, so the state changes rarely)
     const long long t0 = p.tiles * blockIdx.x / gridDim.x;

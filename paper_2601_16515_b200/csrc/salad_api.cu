@@ -169,7 +169,7 @@ int prepare_device(DeviceInfo* info) {
 // placed while the kernel before it in the stream drains.  Every kernel launched this way calls
 // grid_dependency_wait() before it touches what that kernel may have written, so stream order is kept; only the launch
 // latency goes away, between the kernels of a call and, for the first of an attention call, behind whatever kernel
-// came before it (12 heads of 2310 tokens, calls back to back: 34.8 -> 32.0 us).  A grid launched this way never ends
+// came before it (12 heads of 2310 tokens, calls back to back: 34.8 -> 32.1 us).  A grid launched this way never ends
 // before the one it waits for, so waiting for the kernel just before covers everything earlier in the stream.  The
 // first kernels of the Top-K, dynamic-scale and projection calls stay ordinary launches: on them it cost more than it
 // gave (63 -> 66 us, 119 -> 127 at 75600 x 5120, 140 -> 147 at the 1.3B width).

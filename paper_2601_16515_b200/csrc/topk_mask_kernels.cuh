@@ -141,9 +141,6 @@ __device__ __forceinline__ void cp_async_16(void* smem_dst, const void* gmem_src
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;"
                  ::"r"(static_cast<uint32_t>(__cvta_generic_to_shared(smem_dst))), "l"(gmem_src) : "memory");
 }
-__device__ __forceinline__ void cp_async_wait_all() {
-    asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
-}
 
 constexpr int kScoreChunk = 32;       // channels per shared-memory stage
 constexpr int kScoreSmemBytes = 2 * kScoreChunk * (kScoreRows + kScoreTile) * 4;      // two stages: 40 KB
