@@ -26,6 +26,10 @@
  *     not be shared by calls that may overlap on the GPU.
  *   - `stream` is a cudaStream_t passed as void* (NULL = default stream).  Work is enqueued
  *     asynchronously on it; only salad_mask_build synchronises (to return nnz).
+ *     Kernels are launched with programmatic stream serialization and wait for the kernel in
+ *     front of them with griddepcontrol.wait.  A caller's own kernel that is launched that way,
+ *     just before a call, must wait for its predecessor too before it ends (as such kernels do),
+ *     or the call does not wait for that predecessor either.
  *   - Return value: SALAD_OK or a negative code.  Argument errors are detected on the host
  *     before anything is launched.  There is no CPU fallback: without a usable CUDA device
  *     the compute entry points return SALAD_ERR_CUDA.
