@@ -10,10 +10,12 @@ from __future__ import annotations
 import os
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libsalad.so")
+FASTCALL = os.path.join(HERE, "_fastcall.so")            # CPython module, see csrc/fastcall.cpp
 SOURCES = ["salad_api.cu"]
 HEADERS = ["ptx.cuh", "tmap.cuh", "mask_kernels.cuh", "linear_state_kernel.cuh", "fused_kernel.cuh",
            "dynamic_scale_kernel.cuh", "linear_apply_kernel.cuh", "topk_mask_kernels.cuh", "permute_kernel.cuh", "proj_gemm_kernel.cuh",
@@ -38,11 +40,25 @@ def needs_build() -> bool:
     return any(os.path.getmtime(d) > t for d in deps)
 
 
+def fastcall_command(out: str):
+    return ["g++", "-O2", "-std=c++17", "-shared", "-fPIC", "-fvisibility=hidden", "-I" + sysconfig.get_paths()["include"],
+            "-o", out, os.path.join(CSRC, "fastcall.cpp")]
+
+
+def _fastcall_needs_build() -> bool:
+    deps = [os.path.join(CSRC, s) for s in ("fastcall.cpp", os.path.join("..", "..", "include", "salad.h"))]
+    return not os.path.exists(FASTCALL) or any(os.path.getmtime(d) > os.path.getmtime(FASTCALL) for d in deps)
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
     if force or needs_build():
         tmp = LIB + f".{os.getpid()}.tmp"
         subprocess.check_call(nvcc_command(tmp, verbose))
         os.replace(tmp, LIB)
+    if force or _fastcall_needs_build():
+        tmp = FASTCALL + f".{os.getpid()}.tmp"
+        subprocess.check_call(fastcall_command(tmp))
+        os.replace(tmp, FASTCALL)
     return LIB
 
 

@@ -108,6 +108,19 @@ def _load() -> ctypes.CDLL:
 _lib = _load()
 
 
+def _load_fast():
+    """{name: function} of the calls that do not go through ctypes (csrc/fastcall.cpp); empty where that module was not built."""
+    try:
+        from . import _fastcall
+    except ImportError:
+        return {}
+    return {name: getattr(_fastcall, name) for name in EXPORTS
+            if _fastcall.bind(name, ctypes.cast(getattr(_lib, name), ctypes.c_void_p).value)}
+
+
+_fast = _load_fast()
+
+
 def status_string(code: int) -> str:
     return _lib.salad_status_string(int(code)).decode()
 
@@ -137,12 +150,18 @@ def _call(name: str, anchor: torch.Tensor, stream, *args):
     else:
         stream = stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
     if torch._C._cuda_getDevice() == index:
-        rc = getattr(_lib, name)(*args, stream)
+        rc = _enter(name, *args, stream)
     else:
         with torch.cuda.device(index):
-            rc = getattr(_lib, name)(*args, stream)
+            rc = _enter(name, *args, stream)
     if rc != SALAD_OK:
         raise SaladError(rc, name)
+
+
+def _enter(name: str, *args) -> int:
+    fast = _fast.get(name)
+    rc = None if fast is None else fast(*args)
+    return getattr(_lib, name)(*args) if rc is None else rc
 
 
 def _bf16_4d(name: str, t: torch.Tensor):

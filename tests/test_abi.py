@@ -135,3 +135,22 @@ def test_host_only_entry_points_need_no_cuda_torch(lib):
             "from paper_2601_16515_b200 import salad\n"
             "assert salad.salad_workspace_bytes(1, 2, 1024, 64, 64, 64) > 0 and salad.status_string(0) == 'SALAD_OK'\n")
     subprocess.run([sys.executable, "-c", code], cwd=ROOT, check=True)
+
+
+def test_native_calls_answer_like_ctypes(lib):
+    """The calls that bypass ctypes (csrc/fastcall.cpp): the same answers on the host-side checks, and whatever they do not
+    convert is left to ctypes, with its errors."""
+    assert set(lib._fast) <= set(lib.EXPORTS) and "salad_fused_fwd" in lib._fast
+    p, ws_bytes = 1 << 20, lib.salad_workspace_bytes(1, 2, 1024, 64, 64, 64)      # never dereferenced
+    good = [p, p, p, p, 1, 2, 1024, 64, 64, 64, p, p, 2, p, p, 0.0, 1e-6, p, ws_bytes, None, None]
+    for change in ({0: None}, {3: p + 8}, {7: 96}, {9: 32}, {12: 5}, {15: -1.0}, {15: float("nan")}, {16: float("inf")}, {17: p + 1},
+                   {18: ws_bytes - 1}, {4: -1}, {6: 0}, {4: 2**32}):
+        args = [change.get(i, a) for i, a in enumerate(good)]
+        rc = lib._fast["salad_fused_fwd"](*args)
+        assert isinstance(rc, int) and rc == lib._lib.salad_fused_fwd(*args) and rc < 0, change
+    for change in ({0: 1.0}, {6: 1024.0}, {15: "0"}, {4: None}):
+        args = [change.get(i, a) for i, a in enumerate(good)]
+        assert lib._fast["salad_fused_fwd"](*args) is None
+        with pytest.raises(ctypes.ArgumentError):
+            lib._enter("salad_fused_fwd", *args)
+    assert lib._fast["salad_fused_fwd"](*good[:-1]) is None
