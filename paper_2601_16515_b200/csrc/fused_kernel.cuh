@@ -1,13 +1,18 @@
 // Block-sparse softmax attention (Eq. 2) fused with the apply step of ReLU linear attention
 // (Eq. 3) and the scaled residual sum of Algorithm 1, for sm_100a.
 //
-// One CTA owns one query block of one (batch, head): a 128-row MMA tile.  Two CTAs share an SM
+// A work item is one query block of one (batch, head): a 128-row MMA tile.  Two CTAs share an SM
 // (each takes half of its shared memory, registers and tensor memory), so the set-up, the first
 // loads and the epilogue of one overlap the main loop of the other, and the two tiles of an SM run
-// independently of each other.
-//   warp 0        TMA producer of the Q tile, the K ring and (at the end) the linear-state tile
+// independently of each other.  The grid has a CTA per item; a CTA that comes to the end of its item takes over the next
+// CTA that has not started (cluster launch control), so that the next item's Q, K and first scores are under way during
+// the epilogue and the set-up of a CTA is paid once per slot (fused calls back to back, a CTA per item -> now: a pair of 12 heads
+// of 32760 tokens at 95 % sparsity 816 -> 797 us, 12 heads at 90 % 668 -> 665, 12 heads of 16464 tokens 252 -> 246, 40 heads of
+// 2310 tokens 78.6 -> 76.2; with all blocks kept, where items have no ends to speak of, 11.31 and 11.33 ms).
+//   warp 0        TMA producer of the Q tile, the K ring and (at the end) the linear-state tile; it also fetches
+//                 the next item for all roles
 //   warp 1        TMA producer of the V ring (independent of the K ring, so neither ring can
-//                 stall the other)
+//                 stall the other); stores the output tile, which is staged over that ring
 //   warp 2        tcgen05 issuer of S = Q K^T; owns the TMEM allocation
 //   warp 3        tcgen05 issuer of O += P V and of the linear numerator
 //                 (an issuing warp walks its loop as a whole, every lane polling the barriers, and one
@@ -36,7 +41,7 @@
 // that announces the completion of P V the V-ring stage.
 // The four producer / issuer warps (one warpgroup) hand registers to the eight softmax warps
 // (setmaxnreg: 48 against 96 per thread, all that the block was launched with), which keeps the softmax loop free of
-// spills at D = 128 (at D = 64 the kernel keeps one word on the stack).
+// spills (one or two words of the epilogue are on the stack).
 // After the last block the softmax warps apply ReLU to the Q rows in shared memory and compute the
 // linear denominator with plain FMAs; the linear state (bf16, transposed) is loaded over the K
 // ring, which is idle by then; the issuing thread multiplies ReLU(Q) with it, and the epilogue
@@ -51,6 +56,8 @@
 // t & 1; its probabilities, packed bf16, overwrite the first 32 columns of the same buffer);
 // [128,128+D) O.  The linear numerator reuses [0,D).
 #pragma once
+#include <type_traits>
+
 #include "ptx.cuh"
 
 namespace salad {
@@ -85,6 +92,7 @@ struct FusedParams {
     float eps;
     float drop_tau;              // linear branch of batch item b skipped when dyn_scale[b] < drop_tau
     const __half* rope;          // [N][D] fp16: (cos, sin) per token and channel pair of the rotary linear branch, or null
+    int take_over;               // 1: a CTA that has finished its item takes over the next CTA of the grid
     int wait_at_top;             // 1: wait for the kernel before this one at once (calls without state kernels)
     int32_t* ws_status;          // library status word (never null)
     int32_t* user_status;        // optional
@@ -117,7 +125,15 @@ static_assert(FusedCfg<64>::ST_BYTES <= FusedCfg<64>::NK * FusedCfg<64>::KV_BYTE
 
 struct FusedBarriers {
     uint64_t q_full, st_full, k_full[2], v_full[2];
-    uint64_t s_full[2], p_ready[2], pv_done[2], o_final, lin_ready, lin_done, out_staged, z_full;
+    uint64_t s_full[2], p_ready[2], pv_done[2], o_final, lin_ready, lin_done, num_free, out_staged, v_free, z_full;
+    uint64_t item_full[2], item_empty[2], taken;
+};
+
+// A work item: a query block of a (batch, head) with its kept list.
+struct FusedItem {
+    int qb, bh, ls, len;               // qb < 0: no item
+    int linear;                        // it has a linear branch,
+    float scale;                       // scaled by this
 };
 
 template <int D>
@@ -131,9 +147,11 @@ salad_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
     using C = FusedCfg<D>;
     extern __shared__ uint8_t smem_raw[];
     __shared__ FusedBarriers bars;
+    __shared__ alignas(16) uint32_t taken_answer[4];
+    __shared__ FusedItem item_slot[2];
     __shared__ uint32_t tmem_base_slot;
-    __shared__ int abort_flag;
-    __shared__ float z_s[D];          // linear normaliser state of this head
+    __shared__ int abort_flag, state_waited;
+    __shared__ alignas(16) float z_s[D];          // linear normaliser state of this head
 
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     const uint32_t s_base = smem_u32(smem);
@@ -153,25 +171,37 @@ salad_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
     // heads last instead was measured to shorten the launch by 0.3 % and to raise its DRAM traffic by
     // half), within a head the query blocks from the most to the least expensive, so that the
     // kernel ends on short items
-    const int rank = blockIdx.x % p.nQb, bh = blockIdx.x / p.nQb;
-    const int h = bh % p.H, b = bh / p.H;
-    const int hm = (p.Hm == 1) ? 0 : (p.Hm == p.H ? h : bh);   // one mask, one per head, or one per (batch, head)
-    const int qb = p.order ? __ldcg(p.order + size_t(hm) * p.nQb + rank) : rank;
-    // temporal head: blocks of spatial positions, fetched through the 4-D maps
-    const bool perm = p.th.T > 0 && ((p.th.flags[h >> 5] >> (h & 31)) & 1u);
+    auto item_of = [&](int block) {
+        FusedItem it;
+        const int rank = block % p.nQb;
+        it.bh = block / p.nQb;
+        const int h = it.bh % p.H, b = it.bh / p.H;
+        const int hm = (p.Hm == 1) ? 0 : (p.Hm == p.H ? h : it.bh);   // one mask, one per head, or one per (batch, head)
+        it.qb = p.order ? __ldcg(p.order + size_t(hm) * p.nQb + rank) : rank;
+        it.linear = (p.mode & MODE_LINEAR) != 0;
+        it.scale = 1.f;
+        if (it.linear) {
+            if (p.static_scale) it.scale *= __ldg(p.static_scale + h);
+            if (p.dyn_scale) {
+                const float dyn = __ldg(p.dyn_scale + b);
+                it.scale *= dyn;
+                if (dyn < p.drop_tau) it.linear = 0;       // post-tuning branch dropping (Sec. 4.3): no linear work at all for a dropped batch item
+            }
+        }
+        it.ls = 0; it.len = 0;
+        if ((p.mode & MODE_SPARSE) != 0) {                               // kept list of the query block
+            it.ls = __ldg(p.row_ptr + size_t(hm) * p.nQb + it.qb);
+            it.len = __ldg(p.row_ptr + size_t(hm) * p.nQb + it.qb + 1) - it.ls;
+        }
+        return it;
+    };
+    const FusedItem first = item_of(blockIdx.x);
+    // temporal head: blocks of spatial positions, fetched through the 4-D maps (a CTA of such a call has one item)
+    const int h0 = first.bh % p.H;
+    const bool perm = p.th.T > 0 && ((p.th.flags[h0 >> 5] >> (h0 & 31)) & 1u);
     const int q_rows = perm ? p.th.kq * p.th.T : p.Bq;          // rows of the 128-row tile that hold queries
     const int k_rows = perm ? p.th.ks * p.th.T : C::BK;         // rows of a 64-row tile that hold keys
-    if (qb >= (perm ? p.th.nQb : p.nQb_tok)) return;            // (a list row beyond this head's blocks: whole CTA)
-    const bool sparse = (p.mode & MODE_SPARSE) != 0;
-    // post-tuning branch dropping (Sec. 4.3): no linear work at all for a dropped batch item
-    const bool linear = (p.mode & MODE_LINEAR) != 0 &&
-                        !(p.dyn_scale != nullptr && __ldg(p.dyn_scale + b) < p.drop_tau);
-    // kept list of the query block
-    int ls = 0, le = 0;
-    if (sparse) {
-        ls = __ldg(p.row_ptr + size_t(hm) * p.nQb + qb);
-        le = __ldg(p.row_ptr + size_t(hm) * p.nQb + qb + 1);
-    }
+    if (first.qb >= (perm ? p.th.nQb : p.nQb_tok)) return;       // (a list row beyond this head's blocks: whole CTA)
 
     // softmax warps whose 16 rows hold queries (64-row query blocks: four of the eight); the others do nothing
     const int row_warps = (q_rows + 15) >> 4;
@@ -181,19 +211,26 @@ salad_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
         // 2: an earlier kernel of this call has already reported a failure (a rejected mask, an expired wait):
         // this CTA starts nothing and reports nothing; 1 (set by a bounded wait of this CTA): a time-out
         abort_flag = (*reinterpret_cast<volatile int32_t*>(p.ws_status) != 0) ? 2 : 0;
+        state_waited = 0;
+        item_slot[0] = first;
         mbar_init(smem_u32(&bars.q_full), 1);
         mbar_init(smem_u32(&bars.st_full), 1);
         mbar_init(smem_u32(&bars.o_final), 1);
-        mbar_init(smem_u32(&bars.lin_ready), 32 * row_warps);
+        mbar_init(smem_u32(&bars.lin_ready), row_warps);
         mbar_init(smem_u32(&bars.lin_done), 1);
-        mbar_init(smem_u32(&bars.out_staged), 32 * row_warps);
+        mbar_init(smem_u32(&bars.num_free), row_warps);
+        mbar_init(smem_u32(&bars.out_staged), row_warps);
+        mbar_init(smem_u32(&bars.v_free), 1);
         mbar_init(smem_u32(&bars.z_full), 32);
+        mbar_init(smem_u32(&bars.taken), 1);
         for (int j = 0; j < 2; ++j) {
             mbar_init(smem_u32(&bars.s_full[j]), 1);
             mbar_init(smem_u32(&bars.p_ready[j]), row_warps);  // one arrival per softmax warp
             mbar_init(smem_u32(&bars.pv_done[j]), 1);
             mbar_init(smem_u32(&bars.k_full[j]), 1);
             mbar_init(smem_u32(&bars.v_full[j]), 1);
+            mbar_init(smem_u32(&bars.item_full[j]), 1);
+            mbar_init(smem_u32(&bars.item_empty[j]), 3 + row_warps);
         }
         fence_mbar_init();
     }
@@ -219,13 +256,23 @@ salad_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
     tc_fence_after_sync();
     const uint32_t tmem = tmem_base_slot;
     volatile int* abortp = &abort_flag;
-    const int len = le - ls;
     const bool inherited_abort = abort_flag != 0;      // uniform: read after the barrier above, before any wait
 
     // a bounded wait taken by a whole warp: warp-uniform outcome
     auto wait_warp = [&](uint64_t* bar, uint32_t parity) -> bool {
         return __all_sync(0xffffffffu, mbar_wait(smem_u32(bar), parity, abortp));
     };
+    // The items of this CTA: item k in slot k & 1, left there by warp 0 (the first one above).  false: there is none.
+    auto get_item = [&](int k) -> bool {
+        if (k > 0 && !wait_warp(&bars.item_full[k & 1], ((k - 1) >> 1) & 1)) return false;
+        return item_slot[k & 1].qb >= 0;
+    };
+    auto release_item = [&](int k) {
+        __syncwarp();
+        if (lane == 0) mbar_arrive(smem_u32(&bars.item_empty[k & 1]));
+    };
+    // Every role counts what it needs for the phases of the barriers: the blocks before the item at hand (g: block t of it is
+    // block g + t of the CTA, which decides its buffers), the items that loaded Q, and those with a linear branch.
 
     if (!inherited_abort) {
     if (warp < 4) {
@@ -233,72 +280,137 @@ salad_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
     asm volatile("setmaxnreg.dec.sync.aligned.u32 48;");
     if (warp == 0) {
         // ============================================================== TMA producer: Q, the K ring, the state tile
-        bool ok = true;
+        auto load_q = [&](const FusedItem& it) {
+            const uint32_t bar = smem_u32(&bars.q_full);
+            mbar_arrive_expect_tx(bar, uint32_t(q_rows) * D * 2);
+            for (int ch = 0; ch < C::CH; ++ch) {
+                if (perm) tma_load_4d(s_base + C::OFF_Q + ch * C::Q_CHUNK, &map_q4, bar, ch * 64, 0, it.qb * p.th.kq, it.bh);
+                else tma_load_3d(s_base + C::OFF_Q + ch * C::Q_CHUNK, &map_q, bar, ch * 64, it.qb * p.Bq, it.bh);
+            }
+        };
         if (lane == 0) {
-            prefetch_tmap(&map_q); prefetch_tmap(&map_k);
-            // A block with no kept key block and no linear branch never reads Q: its epilogue
-            // stages zeros in the Q tile without waiting for q_full, so nothing may land there.
-            if (len > 0 || linear) {
-                const uint32_t bar = smem_u32(&bars.q_full);
-                mbar_arrive_expect_tx(bar, uint32_t(q_rows) * D * 2);
-                for (int ch = 0; ch < C::CH; ++ch) {
-                    if (perm) tma_load_4d(s_base + C::OFF_Q + ch * C::Q_CHUNK, &map_q4, bar, ch * 64, 0, qb * p.th.kq, bh);
-                    else tma_load_3d(s_base + C::OFF_Q + ch * C::Q_CHUNK, &map_q, bar, ch * 64, qb * p.Bq, bh);
-                }
-            }
-            for (int t = 0; t < len; ++t) {
-                const int s = t % C::NK;
-                // stage s = t & 1 is free once Q K^T of block t - 2 has completed: the barrier that hands its
-                // scores to the softmax warps says so (one commit serves both)
-                if (t >= C::NK) ok = mbar_wait(smem_u32(&bars.s_full[s]), ((t >> 1) - 1) & 1, abortp);
-                if (!ok) break;
-                const int col = __ldg(p.col_idx + ls + t);
-                const uint32_t bar = smem_u32(&bars.k_full[s]);
-                mbar_arrive_expect_tx(bar, uint32_t(k_rows) * D * 2);
-                for (int ch = 0; ch < C::CH; ++ch) {     // chunk-major: the two stages of a chunk are adjacent
-                    const uint32_t dst = s_base + C::OFF_K + ch * (C::NK * C::KV_CHUNK) + s * C::KV_CHUNK;
-                    if (perm) tma_load_4d(dst, &map_k4, bar, ch * 64, 0, col * p.th.ks, bh);
-                    else tma_load_3d(dst, &map_k, bar, ch * 64, col * C::BK, bh);
-                }
-            }
+            if (first.len > 0 || first.linear) load_q(first);
+            prefetch_tmap(&map_k);
         }
-        if (linear) {
-            // From here on the linear state is needed: wait for the kernels that make it (whole warp: the
-            // other lanes fetch the normaliser Z of this head for the softmax warps meanwhile).
-            __syncwarp();
-            grid_dependency_wait();
-            if (*reinterpret_cast<volatile int32_t*>(p.ws_status) != 0 && *abortp == 0) *abortp = 2;   // the state kernel gave up (and said so)
-            for (int a = lane; a < D; a += 32) z_s[a] = __ldcg(p.z + size_t(bh) * D + a);
-            mbar_arrive(smem_u32(&bars.z_full));
-            if (lane == 0 && ok) {
-                // the state tile goes over the K ring: every Q K^T must have read its K block.  The products
-                // complete in order, so the last one (signalled on its score buffer's barrier) covers all.
-                if (len > 0) ok = mbar_wait(smem_u32(&bars.s_full[(len - 1) & 1]), ((len - 1) >> 1) & 1, abortp);
+        int g = 0, n_lin = 0;
+        bool ok = true;
+        FusedItem item = first;
+        for (int k = 0; ; ++k) {
+            const int len = item.len, bh = item.bh;
+            if (lane == 0) {
+                // A block with no kept key block and no linear branch never reads Q.
+                if (k > 0 && (len > 0 || item.linear)) {
+                    // the products that read the Q tile and the K ring of the items before (the state tile lies over it)
+                    if (n_lin > 0) ok = mbar_wait(smem_u32(&bars.lin_done), (n_lin - 1) & 1, abortp);
+                    if (ok && g > 0) ok = mbar_wait(smem_u32(&bars.s_full[(g - 1) & 1]), ((g - 1) >> 1) & 1, abortp);
+                    if (ok) load_q(item);
+                }
+                int col = len > 0 ? __ldg(p.col_idx + item.ls) : 0;
+                for (int t = 0; t < len && ok; ++t) {
+                    const int gt = g + t, s = gt & 1;
+                    // stage s is free once Q K^T of the block before the last has completed: the barrier that hands its
+                    // scores to the softmax warps says so (one commit serves both)
+                    if (gt >= C::NK) ok = mbar_wait(smem_u32(&bars.s_full[s]), ((gt >> 1) - 1) & 1, abortp);
+                    if (!ok) break;
+                    const uint32_t bar = smem_u32(&bars.k_full[s]);
+                    mbar_arrive_expect_tx(bar, uint32_t(k_rows) * D * 2);
+                    for (int ch = 0; ch < C::CH; ++ch) {     // chunk-major: the two stages of a chunk are adjacent
+                        const uint32_t dst = s_base + C::OFF_K + ch * (C::NK * C::KV_CHUNK) + s * C::KV_CHUNK;
+                        if (perm) tma_load_4d(dst, &map_k4, bar, ch * 64, 0, col * p.th.ks, bh);
+                        else tma_load_3d(dst, &map_k, bar, ch * 64, col * C::BK, bh);
+                    }
+                    if (t + 1 < len) col = __ldg(p.col_idx + item.ls + t + 1);
+                }
+                // The next item: that of the next CTA of the grid that has not started, which this one takes over.  Asked
+                // for only now, a few blocks before the end, so that at the end of the grid no CTA sits on an item while
+                // another has none.
+                FusedItem next;
+                next.qb = -1; next.bh = 0; next.ls = 0; next.len = 0; next.linear = 0; next.scale = 0.f;
+                if (ok && p.take_over) {
+                    mbar_arrive_expect_tx(smem_u32(&bars.taken), 16);
+                    clc_try_cancel(smem_u32(taken_answer), smem_u32(&bars.taken));
+                    ok = mbar_wait(smem_u32(&bars.taken), k & 1, abortp);
+                    if (ok) {
+                        const int block = clc_answer(smem_u32(taken_answer));
+                        fence_proxy_async_smem();            // (read, before the next answer is written over it)
+                        if (block >= 0 && *reinterpret_cast<volatile int32_t*>(p.ws_status) == 0) next = item_of(block);
+                    }
+                }
+                if (ok && k >= 1) ok = mbar_wait(smem_u32(&bars.item_empty[(k + 1) & 1]), ((k - 1) >> 1) & 1, abortp);
                 if (ok) {
-                    prefetch_tmap(&map_st);
-                    const uint32_t bar = smem_u32(&bars.st_full);
-                    mbar_arrive_expect_tx(bar, C::ST_BYTES);
-                    for (int ch = 0; ch < C::CH; ++ch)
-                        tma_load_3d(s_base + C::OFF_ST + ch * C::ST_CHUNK, &map_st, bar, ch * 64, 0, bh);
+                    item_slot[(k + 1) & 1] = next;
+                    mbar_arrive(smem_u32(&bars.item_full[(k + 1) & 1]));
                 }
             }
+            g += len;
+            if (item.linear) {
+                // From here on the linear state is needed: wait for the kernels that make it (whole warp: the
+                // other lanes fetch the normaliser Z of this head for the softmax warps meanwhile).
+                __syncwarp();
+                if (n_lin == 0) {
+                    grid_dependency_wait();
+                    if (lane == 0) state_waited = 1;
+                    if (*reinterpret_cast<volatile int32_t*>(p.ws_status) != 0 && *abortp == 0) *abortp = 2;   // the state kernel gave up (and said so)
+                }
+                for (int a = lane; a < D; a += 32) z_s[a] = __ldcg(p.z + size_t(bh) * D + a);
+                mbar_arrive(smem_u32(&bars.z_full));
+                if (lane == 0 && ok) {
+                    // the state tile goes over the K ring: every Q K^T must have read its K block.  The products
+                    // complete in order, so the last one (signalled on its score buffer's barrier) covers all.
+                    if (g > 0) ok = mbar_wait(smem_u32(&bars.s_full[(g - 1) & 1]), ((g - 1) >> 1) & 1, abortp);
+                    if (ok) {
+                        prefetch_tmap(&map_st);
+                        const uint32_t bar = smem_u32(&bars.st_full);
+                        mbar_arrive_expect_tx(bar, C::ST_BYTES);
+                        for (int ch = 0; ch < C::CH; ++ch)
+                            tma_load_3d(s_base + C::OFF_ST + ch * C::ST_CHUNK, &map_st, bar, ch * 64, 0, bh);
+                    }
+                }
+                ++n_lin;
+            }
+            if (!__all_sync(0xffffffffu, ok) || !get_item(k + 1)) break;
+            item = item_slot[(k + 1) & 1];
         }
     } else if (warp == 1) {
-        // ============================================================== TMA producer of the V ring
+        // ============================================================== TMA producer of the V ring, output store
         if (lane == 0) {
             prefetch_tmap(&map_v);
-            for (int t = 0; t < len; ++t) {
-                const int s = t % C::NV;
-                // stage s = t & 1 is free once P V of block t - 2 has completed
-                if (t >= C::NV && !mbar_wait(smem_u32(&bars.pv_done[s]), ((t >> 1) - 1) & 1, abortp)) break;
-                const int col = __ldg(p.col_idx + ls + t);
-                const uint32_t bar = smem_u32(&bars.v_full[s]);
-                mbar_arrive_expect_tx(bar, uint32_t(k_rows) * D * 2);
-                for (int ch = 0; ch < C::CH; ++ch) {
-                    const uint32_t dst = s_base + C::OFF_V + s * C::KV_BYTES + ch * C::KV_CHUNK;
-                    if (perm) tma_load_4d(dst, &map_v4, bar, ch * 64, 0, col * p.th.ks, bh);
-                    else tma_load_3d(dst, &map_v, bar, ch * 64, col * C::BK, bh);
+            int g = 0;
+            bool ok = true;
+            for (int k = 0; ok; ++k) {
+                if (k > 0 && !mbar_wait(smem_u32(&bars.item_full[k & 1]), ((k - 1) >> 1) & 1, abortp)) break;
+                const FusedItem item = item_slot[k & 1];
+                if (item.qb < 0) break;
+                mbar_arrive(smem_u32(&bars.item_empty[k & 1]));
+                const int len = item.len, bh = item.bh;
+                for (int t = 0; t < len; ++t) {
+                    const int gt = g + t, s = gt & 1;
+                    // stage s is free once P V of the block before the last has completed
+                    if (gt >= C::NV) ok = mbar_wait(smem_u32(&bars.pv_done[s]), ((gt >> 1) - 1) & 1, abortp);
+                    if (!ok) break;
+                    const int col = __ldg(p.col_idx + item.ls + t);
+                    const uint32_t bar = smem_u32(&bars.v_full[s]);
+                    mbar_arrive_expect_tx(bar, uint32_t(k_rows) * D * 2);
+                    for (int ch = 0; ch < C::CH; ++ch) {
+                        const uint32_t dst = s_base + C::OFF_V + s * C::KV_BYTES + ch * C::KV_CHUNK;
+                        if (perm) tma_load_4d(dst, &map_v4, bar, ch * 64, 0, col * p.th.ks, bh);
+                        else tma_load_3d(dst, &map_v, bar, ch * 64, col * C::BK, bh);
+                    }
                 }
+                if (!ok) break;
+                g += len;
+                // the output tile, staged over the V ring
+                ok = mbar_wait(smem_u32(&bars.out_staged), k & 1, abortp);
+                if (!ok) break;
+                for (int ch = 0; ch < C::CH; ++ch) {
+                    if (perm) tma_store_4d(&map_o4, s_base + C::OFF_V + ch * C::Q_CHUNK, ch * 64, 0, item.qb * p.th.kq, bh);
+                    else tma_store_3d(&map_o, s_base + C::OFF_V + ch * C::Q_CHUNK, ch * 64, item.qb * p.Bq, bh);
+                }
+                tma_store_commit();
+                // only the shared-memory source must have been read before it is written again or the CTA exits; the
+                // writes are complete, like all of the kernel's, when the grid is
+                tma_store_wait_read_all();
+                mbar_arrive(smem_u32(&bars.v_free));
             }
         }
     } else if (warp == 2) {
@@ -310,27 +422,39 @@ salad_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
         constexpr uint32_t HI = sdesc_hi_sw128(1024);   // the high descriptor word is one constant here
         const uint32_t q_lo = sdesc_lo(s_base + C::OFF_Q, 16);
         const uint32_t k_lo0 = sdesc_lo(s_base + C::OFF_K, 16);
-        bool ok = true;
-        {
-            if (len > 0) ok = wait_warp(&bars.q_full, 0);
+        int g = 0, n_q = 0, n_lin = 0;
+        bool ok = true, before_linear = false;
+        for (int k = 0; ok; ++k) {
+            if (!get_item(k)) break;
+            const int len = item_slot[k & 1].len;
+            const bool linear = item_slot[k & 1].linear != 0;
+            release_item(k);
+            // Every phase of these two is waited for, also where this item needs neither: a wait tells a phase from the one
+            // before the last only by that.  First the numerator of the item before, which lies over both score buffers.
+            if (before_linear) ok = wait_warp(&bars.num_free, (n_lin - 1) & 1);
+            if (ok && (len > 0 || linear)) ok = wait_warp(&bars.q_full, n_q & 1);
+            before_linear = linear;
             for (int t = 0; t < len && ok; ++t) {
-                const int s = t % C::NK;
-                ok = wait_warp(&bars.k_full[s], (t / C::NK) & 1);
-                // score buffer t & 1 held P of block t - 2: its P V product must have read it
-                if (ok && t >= 2) ok = wait_warp(&bars.pv_done[t & 1], ((t >> 1) - 1) & 1);
+                const int gt = g + t, s = gt & 1;
+                ok = wait_warp(&bars.k_full[s], (gt >> 1) & 1);
+                // score buffer s held P of the block before the last: its P V product must have read it
+                if (ok && gt >= 2) ok = wait_warp(&bars.pv_done[s], ((gt >> 1) - 1) & 1);
                 if (!ok) break;
                 tc_fence_after_sync();
                 if (elect_one()) {
                     const uint32_t kb_lo = k_lo0 + s * (C::KV_CHUNK >> 4);
 #pragma unroll
-                    for (int k = 0; k < D / 16; ++k)   // 16 channels: 32 bytes of each Q and K row, chunk k/4
-                        mma_ss_lohi(tmem + C::COL_SP + (t & 1) * C::SP_STRIDE,
-                                    q_lo + (((k / 4) * C::Q_CHUNK + (k % 4) * 32) >> 4), HI,
-                                    kb_lo + (((k / 4) * (C::NK * C::KV_CHUNK) + (k % 4) * 32) >> 4), HI, idesc_qk, k > 0);
-                    tc_commit(smem_u32(&bars.s_full[t & 1]));
+                    for (int kk = 0; kk < D / 16; ++kk)   // 16 channels: 32 bytes of each Q and K row, chunk kk/4
+                        mma_ss_lohi(tmem + C::COL_SP + s * C::SP_STRIDE,
+                                    q_lo + (((kk / 4) * C::Q_CHUNK + (kk % 4) * 32) >> 4), HI,
+                                    kb_lo + (((kk / 4) * (C::NK * C::KV_CHUNK) + (kk % 4) * 32) >> 4), HI, idesc_qk, kk > 0);
+                    tc_commit(smem_u32(&bars.s_full[s]));
                 }
                 __syncwarp();
             }
+            g += len;
+            if (len > 0 || linear) ++n_q;
+            if (linear) ++n_lin;
         }
     } else if (warp == 3) {
         // ============================================================== issuer of O += P V and of the linear numerator
@@ -339,39 +463,49 @@ salad_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
         constexpr uint32_t HI = sdesc_hi_sw128(1024);
         const uint32_t q_lo = sdesc_lo(s_base + C::OFF_Q, 16);
         const uint32_t v_lo0 = sdesc_lo(s_base + C::OFF_V, C::KV_CHUNK);
+        int g = 0, n_lin = 0;
         bool ok = true;
-        for (int t = 0; t < len && ok; ++t) {
-            const int s = t % C::NV;
-            ok = wait_warp(&bars.v_full[s], (t / C::NV) & 1);
-            if (ok) ok = wait_warp(&bars.p_ready[t & 1], (t >> 1) & 1);
-            if (!ok) break;
-            tc_fence_after_sync();
-            if (elect_one()) {
-                const uint32_t vb_lo = v_lo0 + s * (C::KV_BYTES >> 4);
-                const uint32_t p_col = tmem + C::COL_SP + (t & 1) * C::SP_STRIDE;
-#pragma unroll
-                for (int k = 0; k < C::BK / 16; ++k)      // 16 keys = 16 rows of 128 bytes
-                    mma_ts_lohi(tmem + C::COL_O, p_col + k * 8, vb_lo + ((k * 2048) >> 4), HI, idesc_pv,
-                                (t > 0 || k > 0) ? 1u : 0u);
-                tc_commit(smem_u32(&bars.pv_done[t & 1]));
-                if (t + 1 == len) tc_commit(smem_u32(&bars.o_final));
-            }
-            __syncwarp();
-        }
-        if (ok && linear) {
-            ok = wait_warp(&bars.st_full, 0);
-            if (ok) ok = wait_warp(&bars.lin_ready, 0);
-            if (ok) {
+        for (int k = 0; ok; ++k) {
+            if (!get_item(k)) break;
+            const int len = item_slot[k & 1].len;
+            const bool linear = item_slot[k & 1].linear != 0;
+            release_item(k);
+            for (int t = 0; t < len && ok; ++t) {
+                const int gt = g + t, s = gt & 1;
+                ok = wait_warp(&bars.v_full[s], (gt >> 1) & 1);
+                // (with the first P of an item all softmax warps have read the accumulator of the item before)
+                if (ok) ok = wait_warp(&bars.p_ready[s], (gt >> 1) & 1);
+                if (!ok) break;
                 tc_fence_after_sync();
                 if (elect_one()) {
-                    const uint32_t st_lo = sdesc_lo(s_base + C::OFF_ST, 16);
+                    const uint32_t vb_lo = v_lo0 + s * (C::KV_BYTES >> 4);
+                    const uint32_t p_col = tmem + C::COL_SP + s * C::SP_STRIDE;
 #pragma unroll
-                    for (int k = 0; k < D / 16; ++k)
-                        mma_ss_lohi(tmem, q_lo + (((k / 4) * C::Q_CHUNK + (k % 4) * 32) >> 4), HI,
-                                    st_lo + (((k / 4) * C::ST_CHUNK + (k % 4) * 32) >> 4), HI, idesc_lin, k > 0);
-                    tc_commit(smem_u32(&bars.lin_done));
+                    for (int kk = 0; kk < C::BK / 16; ++kk)      // 16 keys = 16 rows of 128 bytes
+                        mma_ts_lohi(tmem + C::COL_O, p_col + kk * 8, vb_lo + ((kk * 2048) >> 4), HI, idesc_pv,
+                                    (t > 0 || kk > 0) ? 1u : 0u);
+                    tc_commit(smem_u32(&bars.pv_done[s]));
+                    if (t + 1 == len) tc_commit(smem_u32(&bars.o_final));
                 }
                 __syncwarp();
+            }
+            g += len;
+            if (ok && linear) {
+                ok = wait_warp(&bars.st_full, n_lin & 1);
+                if (ok) ok = wait_warp(&bars.lin_ready, n_lin & 1);
+                if (ok) {
+                    tc_fence_after_sync();
+                    if (elect_one()) {
+                        const uint32_t st_lo = sdesc_lo(s_base + C::OFF_ST, 16);
+#pragma unroll
+                        for (int kk = 0; kk < D / 16; ++kk)
+                            mma_ss_lohi(tmem, q_lo + (((kk / 4) * C::Q_CHUNK + (kk % 4) * 32) >> 4), HI,
+                                        st_lo + (((kk / 4) * C::ST_CHUNK + (kk % 4) * 32) >> 4), HI, idesc_lin, kk > 0);
+                        tc_commit(smem_u32(&bars.lin_done));
+                    }
+                    __syncwarp();
+                }
+                ++n_lin;
             }
         }
     }
@@ -385,17 +519,12 @@ salad_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
         const int sw = warp - 4;
         const int q4 = lane & 3;                                // position in the group of four
         const int lane0 = (warp & 3) * 32 + (sw >> 2) * 16;          // first TMEM lane of this warp
-        const int ra = lane0 + (lane >> 2), rb = ra + 8;        // the thread's two query rows
+        // (the thread's two query rows: lane0 + lane / 4 and eight more)
         // Without queries in its rows a warp leaves its P as it is: whatever it holds meets only accumulator rows that nobody
         // reads.  (64-row query blocks spend half of the exponentials for nothing otherwise: 12 heads of 32760 tokens
         // 1070 -> 932 us per fused call, 2310 tokens 40.1 -> 38.5.)
         if (lane0 < q_rows) {
         const uint32_t t_tile = tmem + (uint32_t(lane0) << 16);
-        const int len = le - ls;
-        uint8_t* qtile = smem + C::OFF_Q;
-        float m_a = -INFINITY, m_b = -INFINITY;                 // running maxima (log2 domain)
-        float l_a = 0.f, l_b = 0.f;                             // this thread's share of the row sums
-        bool ok = true;
         // every lane of a warp must take the same path around the warp-collective tcgen05
         // loads/stores, so the outcome of a bounded wait is made warp-uniform
         auto wait_uniform = [&](uint64_t* bar, uint32_t parity) -> bool {
@@ -410,6 +539,17 @@ salad_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
             return v + __shfl_xor_sync(0xffffffffu, v, 2);
         };
 
+        // the counters of this role, as much of them as the parities need: blocks before this item & 3, then a bit each for
+        // the items with Q, with kept blocks and with a linear branch
+        uint32_t ph = 0;
+        bool ok = true;
+        for (int k = 0; ok; ++k) {
+        if (!get_item(k)) break;
+        const FusedItem& item = item_slot[k & 1];
+        const int len = item.len;
+        const bool linear = item.linear != 0;
+        float m_a = -INFINITY, m_b = -INFINITY;                 // running maxima (log2 domain)
+        float l_a = 0.f, l_b = 0.f;                             // this thread's share of the row sums
         // Only the last key block of the sequence can be short (N not a multiple of 64), and in an ascending
         // list it can only be the last entry: one look at that entry, before the loop, settles which block
         // needs its missing keys masked.
@@ -417,14 +557,17 @@ salad_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
         int valid_last = k_rows;
         if (len > 0) {
             if (perm) {
-                if (__ldg(p.col_idx + le - 1) == p.th.nKb - 1) valid_last = (p.th.S - (p.th.nKb - 1) * p.th.ks) * p.th.T;
-            } else if ((p.N % C::BK) != 0 && __ldg(p.col_idx + le - 1) == p.nKb - 1) {
+                if (__ldg(p.col_idx + item.ls + len - 1) == p.th.nKb - 1) valid_last = (p.th.S - (p.th.nKb - 1) * p.th.ks) * p.th.T;
+            } else if ((p.N % C::BK) != 0 && __ldg(p.col_idx + item.ls + len - 1) == p.nKb - 1) {
                 valid_last = p.N - (p.nKb - 1) * C::BK;
             }
         }
+        const int limits = valid_last | (k_rows << 8);          // (one register instead of two)
         constexpr float SUM_LIMIT = 4096.f;
+        const int g0 = int(ph & 3u);
         for (int t = 0; t < len && ok; ++t) {
-            ok = wait_uniform(&bars.s_full[t & 1], (t >> 1) & 1);
+            const int gt = g0 + t, s = gt & 1;
+            ok = wait_uniform(&bars.s_full[s], (gt >> 1) & 1);
             if (!ok) break;
             tc_fence_after_sync();
             uint32_t pk[16];
@@ -432,10 +575,10 @@ salad_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
             while (true) {                      // once, or twice when the first pass finds that the max has to move
                 // x[4n], x[4n+1] = S(row a, keys 8n + 2 q4, + 1);  x[4n+2], x[4n+3] = the same keys of row b
                 uint32_t xr[32];
-                tmem_ld_16x256b_x8(t_tile + C::COL_SP + (t & 1) * C::SP_STRIDE, xr);
+                tmem_ld_16x256b_x8(t_tile + C::COL_SP + s * C::SP_STRIDE, xr);
                 tmem_wait_ld();
                 float* x = reinterpret_cast<float*>(xr);
-                const int valid = (t + 1 == len) ? valid_last : k_rows;      // keys of this block that exist
+                const int valid = (t + 1 == len) ? (limits & 255) : (limits >> 8);      // keys of this block that exist
                 if (valid < C::BK) {
 #pragma unroll
                     for (int n = 0; n < 8; ++n) {
@@ -459,7 +602,7 @@ salad_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                         // has landed in it.  pv_done[b] completes a phase for every second block; the product of block
                         // t cannot be issued before this warp hands over P of block t, so the barrier is at most one
                         // phase past the one tested here and the parity test is exact.
-                        ok = wait_uniform(&bars.pv_done[(t - 1) & 1], ((t - 1) >> 1) & 1);
+                        ok = wait_uniform(&bars.pv_done[s ^ 1], ((gt - 1) >> 1) & 1);
                         if (!ok) break;
                         tc_fence_after_sync();
                         const float na = fmaxf(m_a, msa), nb = fmaxf(m_b, msb);
@@ -507,12 +650,18 @@ salad_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
             }
             if (!ok) break;
             // P goes over the scores it was computed from (this warp's own lanes, already in registers)
-            tmem_st_16x128b_x8(t_tile + C::COL_SP + (t & 1) * C::SP_STRIDE, pk);
+            tmem_st_16x128b_x8(t_tile + C::COL_SP + s * C::SP_STRIDE, pk);
             tmem_wait_st();
             tc_fence_before_sync();
             __syncwarp();
-            if (lane == 0) mbar_arrive(smem_u32(&bars.p_ready[t & 1]));   // one arrival per warp
+            if (lane == 0) mbar_arrive(smem_u32(&bars.p_ready[s]));   // one arrival per warp
         }
+        // From here on addresses come from copies that the compiler knows nothing of: it would form all of them once, ahead of
+        // the items, and keep them in registers that the loop above needs (1580 cycles per block instead of 1380).
+        int elane = lane;
+        uint32_t sb = s_base;
+        asm volatile("" : "+r"(elane), "+r"(sb));
+        const int q4 = elane & 3, ra = lane0 + (elane >> 2), rb = ra + 8;
         float coef_a = 0.f, coef_b = 0.f;
         if (ok && linear) {
             // ReLU of the Q rows in place, and the denominators ReLU(Q_n) . Z: the four threads of a
@@ -526,70 +675,83 @@ salad_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
             const bool rotary = p.rope != nullptr;
             auto rot_ptr = [&](int it) {
                 const int row = (it & 1) ? rb : ra;
-                const int tok = min(qb * p.Bq + row, p.N - 1);           // rows past the block or N hold zeros
+                const int tok = min(item.qb * p.Bq + row, p.N - 1);           // rows past the block or N hold zeros
                 return reinterpret_cast<const uint4*>(p.rope + size_t(tok) * D + (it >> 2) * 64 +
                                                       (q4 + 4 * ((it >> 1) & 1)) * 8);
             };
-            uint4 tw[2];
-#pragma unroll
-            for (int u = 0; u < 2; ++u) {
-                tw[u] = make_uint4(0, 0, 0, 0);
-                if (rotary) tw[u] = __ldg(rot_ptr(u));
-            }
-            ok = wait_uniform(&bars.q_full, 0);
-            if (ok) ok = wait_uniform(&bars.z_full, 0);
+            ok = wait_uniform(&bars.q_full, (ph >> 2) & 1);
+            if (ok) ok = wait_uniform(&bars.z_full, (ph >> 4) & 1);
             if (ok) {
+                // Four vectors are read before the first is written over (in turn, each load would wait for the store before it,
+                // which may go to the same place for all the compiler knows), Z is read once for both rows, the rotary form
+                // has a loop of its own: the pass takes 2000 cycles instead of 2700 at 12 heads of 32760 tokens.
+                const uint32_t qa = sb + C::OFF_Q + ra * 128, sw_a = ra & 7;      // row b: 8 rows on, the same swizzle
                 float den_a = 0.f, den_b = 0.f;
+                auto pass = [&](auto with_rotation) {
+                    constexpr bool ROT = decltype(with_rotation)::value;
+                    uint4 tw[2];
+                    if (ROT) { tw[0] = __ldg(rot_ptr(0)); tw[1] = __ldg(rot_ptr(1)); }
 #pragma unroll
-                for (int it = 0; it < NIT; ++it) {
-                    const int ch = it >> 2, c16 = q4 + 4 * ((it >> 1) & 1), e2 = it & 1;
-                    const int row = e2 ? rb : ra;
-                    uint4* ptr = reinterpret_cast<uint4*>(qtile + ch * C::Q_CHUNK + row * 128 +
-                                                          ((c16 ^ (row & 7)) << 4));
-                    uint4 v = *ptr;
-                    __nv_bfloat162* hv = reinterpret_cast<__nv_bfloat162*>(&v);
-                    const uint4 tv = tw[it & 1];
-                    if (rotary && it + 2 < NIT) tw[it & 1] = __ldg(rot_ptr(it + 2));
-                    const __half2* th = reinterpret_cast<const __half2*>(&tv);      // (cos, sin) of four pairs
-                    float den = 0.f;
+                    for (int ch = 0; ch < C::CH; ++ch) {
+                        uint4 v[4];
 #pragma unroll
-                    for (int e = 0; e < 4; ++e) {
-                        hv[e] = __hmax2(hv[e], __float2bfloat162_rn(0.f));
-                        const float2 f = __bfloat1622float2(hv[e]);
-                        const int a = ch * 64 + c16 * 8 + e * 2;
-                        den = fmaf(f.x, z_s[a], den);
-                        den = fmaf(f.y, z_s[a + 1], den);
-                        if (rotary) {
-                            const float2 cs = __half22float2(th[e]);
-                            hv[e] = __floats2bfloat162_rn(cs.x * f.x - cs.y * f.y, cs.y * f.x + cs.x * f.y);
+                        for (int u = 0; u < 4; ++u) v[u] = lds_128(qa + ch * C::Q_CHUNK + (u & 1) * 1024 + (((q4 + 4 * (u >> 1)) ^ sw_a) << 4));
+#pragma unroll
+                        for (int u2 = 0; u2 < 2; ++u2) {
+                            const float4* zp = reinterpret_cast<const float4*>(z_s + ch * 64 + (q4 + 4 * u2) * 8);
+                            const float4 z0 = zp[0], z1 = zp[1];                 // for both rows
+                            const float z[8] = {z0.x, z0.y, z0.z, z0.w, z1.x, z1.y, z1.z, z1.w};
+#pragma unroll
+                            for (int e2 = 0; e2 < 2; ++e2) {
+                                const int u = u2 * 2 + e2, it = ch * 4 + u;
+                                __nv_bfloat162* hv = reinterpret_cast<__nv_bfloat162*>(&v[u]);
+                                const uint4 tv = ROT ? tw[u & 1] : make_uint4(0, 0, 0, 0);
+                                if (ROT && it + 2 < NIT) tw[u & 1] = __ldg(rot_ptr(it + 2));
+                                const __half2* th = reinterpret_cast<const __half2*>(&tv);      // (cos, sin) of four pairs
+                                float den = 0.f;
+#pragma unroll
+                                for (int e = 0; e < 4; ++e) {
+                                    hv[e] = __hmax2(hv[e], __float2bfloat162_rn(0.f));
+                                    const float2 f = __bfloat1622float2(hv[e]);
+                                    den = fmaf(f.x, z[2 * e], den);
+                                    den = fmaf(f.y, z[2 * e + 1], den);
+                                    if (ROT) {
+                                        const float2 cs = __half22float2(th[e]);
+                                        hv[e] = __floats2bfloat162_rn(cs.x * f.x - cs.y * f.y, cs.y * f.x + cs.x * f.y);
+                                    }
+                                }
+                                if (e2) den_b += den; else den_a += den;
+                            }
                         }
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) sts_128(qa + ch * C::Q_CHUNK + (u & 1) * 1024 + (((q4 + 4 * (u >> 1)) ^ sw_a) << 4), v[u]);
                     }
-                    *ptr = v;
-                    if (e2) den_b += den; else den_a += den;
-                }
+                };
+                if (rotary) pass(std::true_type{}); else pass(std::false_type{});
+                fence_proxy_async_smem();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(smem_u32(&bars.lin_ready));
                 den_a = quad_sum(den_a); den_b = quad_sum(den_b);
-                float c_scale = 1.f;
-                if (p.static_scale) c_scale *= __ldg(p.static_scale + h);
-                if (p.dyn_scale) c_scale *= __ldg(p.dyn_scale + b);
                 // a row with ReLU(Q_n) = 0 and eps = 0 is 0/0: defined as 0 (the numerator is 0 as well)
                 const float da = den_a + p.eps, db = den_b + p.eps;
-                coef_a = da > 0.f ? c_scale / da : 0.f;
-                coef_b = db > 0.f ? c_scale / db : 0.f;
-                fence_proxy_async_smem();
-                mbar_arrive(smem_u32(&bars.lin_ready));
+                coef_a = da > 0.f ? item.scale / da : 0.f;
+                coef_b = db > 0.f ? item.scale / db : 0.f;
             }
         }
         if (ok && len > 0) {
-            ok = wait_uniform(&bars.o_final, 0);
+            ok = wait_uniform(&bars.o_final, (ph >> 3) & 1);
             tc_fence_after_sync();
+        } else if (ok && k > 0) {
+            // (the store of the item before has read the tile that is written below: said by its V loads otherwise)
+            ok = wait_uniform(&bars.v_free, (k - 1) & 1);
         }
         if (ok && linear) {
-            ok = wait_uniform(&bars.lin_done, 0);
+            ok = wait_uniform(&bars.lin_done, (ph >> 4) & 1);
             tc_fence_after_sync();
         }
 
         if (ok) {
-            // O = O_acc / l + coef * num, rounded once to bf16, staged in the Q tile
+            // O = O_acc / l + coef * num, rounded once to bf16, staged over the V ring
             const float lt_a = quad_sum(l_a), lt_b = quad_sum(l_b);
             const float inv_a = (len > 0) ? 1.0f / lt_a : 0.f, inv_b = (len > 0) ? 1.0f / lt_b : 0.f;
 #pragma unroll
@@ -598,6 +760,7 @@ salad_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                 if (len > 0) tmem_ld_16x256b_x4(t_tile + C::COL_O + cc * 32, orr);
                 if (linear) tmem_ld_16x256b_x4(t_tile + cc * 32, nr);
                 tmem_wait_ld();
+                const uint32_t oa = sb + C::OFF_V + (cc >> 1) * C::Q_CHUNK + ra * 128 + q4 * 4;        // over the V ring
 #pragma unroll
                 for (int n = 0; n < 4; ++n) {
                     float a0 = 0.f, a1 = 0.f, b0 = 0.f, b1 = 0.f;
@@ -609,52 +772,46 @@ salad_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                         a0 = fmaf(coef_a, __uint_as_float(nr[4 * n]), a0);     a1 = fmaf(coef_a, __uint_as_float(nr[4 * n + 1]), a1);
                         b0 = fmaf(coef_b, __uint_as_float(nr[4 * n + 2]), b0); b1 = fmaf(coef_b, __uint_as_float(nr[4 * n + 3]), b1);
                     }
-                    const int col16 = cc * 4 + n;                  // 16-byte group (8 columns) within the row
-                    const int ch = col16 / 8, c16 = col16 % 8;
-                    *reinterpret_cast<uint32_t*>(qtile + ch * C::Q_CHUNK + ra * 128 + ((c16 ^ (ra & 7)) << 4) + q4 * 4) =
-                        pack_bf16x2(a0, a1);
-                    *reinterpret_cast<uint32_t*>(qtile + ch * C::Q_CHUNK + rb * 128 + ((c16 ^ (rb & 7)) << 4) + q4 * 4) =
-                        pack_bf16x2(b0, b1);
+                    const int off = ((((cc & 1) * 4 + n) ^ (ra & 7)) << 4);       // 16-byte group (8 columns) within the row
+                    sts_32(oa + off, pack_bf16x2(a0, a1));
+                    sts_32(oa + 8 * 128 + off, pack_bf16x2(b0, b1));
                 }
             }
+            tc_fence_before_sync();
+            __syncwarp();
+            if (linear && lane == 0) mbar_arrive(smem_u32(&bars.num_free));     // the score buffers are free for the next item
             fence_proxy_async_smem();
-            mbar_arrive(smem_u32(&bars.out_staged));
-            if (ra == 0 && q4 == 0 && mbar_wait(smem_u32(&bars.out_staged), 0, abortp)) {
-                for (int ch = 0; ch < C::CH; ++ch) {
-                    if (perm) tma_store_4d(&map_o4, s_base + C::OFF_Q + ch * C::Q_CHUNK, ch * 64, 0, qb * p.th.kq, bh);
-                    else tma_store_3d(&map_o, s_base + C::OFF_Q + ch * C::Q_CHUNK, ch * 64, qb * p.Bq, bh);
-                }
-                tma_store_commit();
-                // only the shared-memory source must have been read before the CTA may exit; the
-                // writes are complete, like all of the kernel's, when the grid is
-                tma_store_wait_read_all();
-            }
+            __syncwarp();
+            if (lane == 0) mbar_arrive(smem_u32(&bars.out_staged));
             if (p.lse != nullptr && q4 == 0) {
 #pragma unroll
                 for (int e2 = 0; e2 < 2; ++e2) {
                     const int row = e2 ? rb : ra;
-                    int n = qb * p.Bq + row;
+                    int n = item.qb * p.Bq + row;
                     if (perm) {                      // row = position within the block * T + frame
-                        const int sp = qb * p.th.kq + row / p.th.T;
+                        const int sp = item.qb * p.th.kq + row / p.th.T;
                         n = (sp < p.th.S) ? (row % p.th.T) * p.th.S + sp : p.N;
                     }
                     if (row < q_rows && n < p.N)
-                        p.lse[size_t(bh) * p.N + n] =
+                        p.lse[size_t(item.bh) * p.N + n] =
                             (len > 0) ? ((e2 ? m_b : m_a) + log2f(e2 ? lt_b : lt_a)) * 0.6931471805599453f : -INFINITY;
                 }
             }
         }
+        release_item(k);
+        ph = ((ph + uint32_t(len)) & 3u) | ((ph ^ ((len > 0 || linear) ? 4u : 0u) ^ (len > 0 ? 8u : 0u) ^ (linear ? 16u : 0u)) & 28u);
+        }  // items
         }  // rows of queries
     }
     }  // !inherited_abort
 
     // ------------------------------------------------------------------ tear-down
+    tc_fence_before_sync();
+    __syncthreads();
     // The first kernel of the next call waits for this grid and for nothing before it, so this grid must not end ahead of the
     // state kernels of its own call, also where no CTA needed them (rejected lists, dropped items).
     // (Only there: the instruction is not free, 2 us of a 32 us call when every CTA issues it once more.)
-    if ((p.mode & MODE_LINEAR) != 0 && (!linear || inherited_abort)) grid_dependency_wait();
-    tc_fence_before_sync();
-    __syncthreads();
+    if ((p.mode & MODE_LINEAR) != 0 && state_waited == 0) grid_dependency_wait();
     if (abort_flag != 0 && !inherited_abort) {
         // a bounded wait expired somewhere (1: in this CTA, reported here; 2: in the state kernels, which
         // reported it themselves): give copies in flight time to land, leave

@@ -1485,3 +1485,40 @@ def test_linear_call_stops_on_a_reported_failure(salad, d):
     assert int(word.item()) == salad.SALAD_ERR_TIMEOUT
     assert bool((out == -7.0).all())
     assert torch.equal(salad.salad_linear_attn_fwd(q, k, v, workspace=ws), want)
+
+
+# ------------------------------------------------------------------------------ several items per CTA
+
+@pytest.mark.parametrize("d,Bq,longest", [(128, 128, 5), (128, 64, 3), (64, 128, 2), (64, 64, 4)])
+def test_a_cta_with_several_items(salad, d, Bq, longest):
+    # More work items than the chip takes at once, with lists of 0 to `longest` blocks in any order (the parity of the
+    # buffers changes from item to item), half of the items without a linear branch, a ragged end.
+    B, H, N = 2, 40, 1290
+    q, k, v = rand_qkv(B, H, N, d, 5 * d + Bq)
+    nQb, nKb = -(-N // Bq), -(-N // 64)
+    assert B * H * nQb > 4 * torch.cuda.get_device_properties(0).multi_processor_count
+    rp, ci = random_csr(B * H * nQb, nKb, d + Bq, lo=0, hi=longest)
+    rp_d, ci_d = dev_csr(rp, ci)
+    rng = np.random.default_rng(d)
+    lam, s = rng.random(H).astype(np.float32), np.array([0.9, 0.1], np.float32)
+    qd, kd, vd, lam_d, s_d = q.cuda(), k.cuda(), v.cuda(), torch.from_numpy(lam).cuda(), torch.from_numpy(s).cuda()
+    g_out, status = Guarded((B, H, N, d), torch.bfloat16, fill=1.0), torch.ones(1, dtype=torch.int32, device="cuda")
+    out = salad.salad_fused_fwd(qd, kd, vd, rp_d, ci_d, B * H, lam_d, s_d, Bq=Bq, drop_tau=0.5, out=g_out.t, status=status)
+    status_ok(status)
+    g_out.check("several items")
+    ref = orc.salad_fused_drop(f32(q), f32(k), f32(v), Bq, 64, rp, ci, B * H, lam, s, tau=0.5)
+    assert_close(f32(out.cpu()).reshape(-1, d), ref, "several items")
+    lse = torch.full((B, H, N), float("nan"), device="cuda")
+    sparse = salad.salad_sparse_attn_fwd(qd, kd, vd, rp_d, ci_d, B * H, Bq=Bq, lse=lse)
+    ref, ref_lse = orc.sparse_attn(f32(q), f32(k), f32(v), Bq, 64, rp, ci, B * H)
+    assert_close(f32(sparse.cpu()).reshape(-1, d), ref, "several items, sparse")
+    got_lse, empty = lse.cpu().numpy().reshape(-1), np.isneginf(ref_lse)
+    assert np.array_equal(np.isneginf(got_lse), empty)
+    np.testing.assert_allclose(got_lse[~empty], ref_lse[~empty], atol=2e-3, rtol=1e-4)
+    # what one item leaves in shared and tensor memory does not reach the next: infinities in a few heads change nothing else
+    for x in (kd, vd):
+        for h in (0, 7, 23):
+            x[0, h] = float("inf")
+    again = salad.salad_fused_fwd(qd, kd, vd, rp_d, ci_d, B * H, lam_d, s_d, Bq=Bq, drop_tau=0.5)
+    clean = [h for h in range(H) if h not in (0, 7, 23)]
+    assert torch.equal(again[0, clean], out[0, clean]) and torch.equal(again[1], out[1])
