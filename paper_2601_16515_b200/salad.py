@@ -1,4 +1,5 @@
-"""ctypes binding of ``libsalad.so``: the same entry points as ``include/salad.h``.
+"""Binding of ``libsalad.so``: the same entry points as ``include/salad.h``, through ctypes or, for the calls that
+a layer makes on every step, a small CPython module (csrc/fastcall.cpp).
 
 The functions here only marshal arguments (tensor -> device pointer, sizes, the current
 CUDA stream) and allocate outputs / workspace with torch when the caller does not pass
