@@ -84,6 +84,7 @@ struct FusedParams {
     const int32_t* col_idx;
     const int32_t* order;        // [Hm][nQb] launch order of the query blocks, or null (identity)
     int BH;                      // batch * heads
+    int by_rank;                 // order of the work items: 1: by expense over all heads, 0: head by head
     const float* static_scale;   // [H] or null (=1)
     const float* dyn_scale;      // [B] or null (=1)
     const float* z;              // [B*H, D] linear normaliser state
@@ -167,14 +168,14 @@ salad_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
     if ((p.mode & MODE_LINEAR) == 0 || p.wait_at_top) grid_dependency_wait();
     grid_launch_dependents();
 
-    // work item: head by head (K/V of one head stay hot in L2: ordering the cheapest items of all
-    // heads last instead was measured to shorten the launch by 0.3 % and to raise its DRAM traffic by
-    // half), within a head the query blocks from the most to the least expensive, so that the
-    // kernel ends on short items
+    // Work items: head by head, within a head the query blocks from the most to the least expensive, so that the
+    // kernel ends on short items and K/V of one head stay hot in L2; or, where K and V of all heads fit there (by_rank),
+    // the most expensive items of all heads first: the CTAs that wait for a state CTA's place, and the second CTA of an SM where
+    // the items do not fill all, then hold the cheapest items, and the launch ends on the cheapest of all heads.
     auto item_of = [&](int block) {
         FusedItem it;
-        const int rank = block % p.nQb;
-        it.bh = block / p.nQb;
+        const int rank = p.by_rank ? block / p.BH : block % p.nQb;
+        it.bh = p.by_rank ? block % p.BH : block / p.nQb;
         const int h = it.bh % p.H, b = it.bh / p.H;
         const int hm = (p.Hm == 1) ? 0 : (p.Hm == p.H ? h : it.bh);   // one mask, one per head, or one per (batch, head)
         it.qb = p.order ? __ldcg(p.order + size_t(hm) * p.nQb + rank) : rank;
