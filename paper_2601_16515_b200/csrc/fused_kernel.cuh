@@ -40,9 +40,10 @@
 // barrier that announces the scores of block t also frees the K-ring stage for block t + 2, the one
 // that announces the completion of P V the V-ring stage.
 // The four producer / issuer warps (one warpgroup) hand registers to the eight softmax warps
-// (setmaxnreg: 32 against 104 per thread, all that the block was launched with: 128 x 32 + 256 x 104 = 384 x 80), which keeps
-// the softmax loop free of spills (two words of the epilogue are on the stack).  48 against 96: 11.22 instead of 11.11 ms with
-// all blocks kept at 2 x 12 heads of 32760 tokens, attention alone, and 615 instead of 613 us at 12 heads and 90 % sparsity.
+// (setmaxnreg: 48 against 96 per thread, all that the block was launched with: 128 x 48 + 256 x 96 = 384 x 80), which keeps
+// the softmax loop free of spills (two words of the epilogue are on the stack).  The producer side by itself takes 38 registers
+// of its own accord.  Fewer than that are not to be left to it: with 32 (and 104) a form of this kernel for one item per CTA lost the
+// head's index in the storing warp and wrote every tile to the first head, without a word from the compiler; with 48 it is right.
 // After the last block the softmax warps apply ReLU to the Q rows in shared memory and compute the
 // linear denominator with plain FMAs; the linear state (bf16, transposed) is loaded over the K
 // ring, which is idle by then; the issuing thread multiplies ReLU(Q) with it, and the epilogue
@@ -279,7 +280,7 @@ salad_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
     if (!inherited_abort) {
     if (warp < 4) {
     // the four producer / issuer warps (one warpgroup) give registers up, the eight softmax warps take them
-    asm volatile("setmaxnreg.dec.sync.aligned.u32 32;");
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 48;");
     if (warp == 0) {
         // ============================================================== TMA producer: Q, the K ring, the state tile
         auto load_q = [&](const FusedItem& it) {
@@ -512,7 +513,7 @@ salad_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
         }
     }
     } else {
-        asm volatile("setmaxnreg.inc.sync.aligned.u32 104;");
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 96;");
         // ============================================================== softmax + epilogue
         // Eight warps.  A warp works on 16 TMEM lanes (query rows) with the 16-lane
         // load/store shapes: four threads share a row, each holding a quarter of its columns,
