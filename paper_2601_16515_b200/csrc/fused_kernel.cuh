@@ -579,7 +579,6 @@ salad_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                 // x[4n], x[4n+1] = S(row a, keys 8n + 2 q4, + 1);  x[4n+2], x[4n+3] = the same keys of row b
                 uint32_t xr[32];
                 tmem_ld_16x256b_x8(t_tile + C::COL_SP + s * C::SP_STRIDE, xr);
-                tmem_wait_ld();
                 float* x = reinterpret_cast<float*>(xr);
                 const int valid = (t + 1 == len) ? (limits & 255) : (limits >> 8);      // keys of this block that exist
                 if (valid < C::BK) {
@@ -616,7 +615,6 @@ salad_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                         for (int cc = 0; cc < D / 32; ++cc) {
                             uint32_t orr[16];
                             tmem_ld_16x256b_x4(t_tile + C::COL_O + cc * 32, orr);
-                            tmem_wait_ld();
 #pragma unroll
                             for (int n = 0; n < 4; ++n) {
                                 orr[4 * n] = __float_as_uint(__uint_as_float(orr[4 * n]) * al_a);
@@ -761,9 +759,9 @@ salad_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
 #pragma unroll
             for (int cc = 0; cc < D / 32; ++cc) {
                 uint32_t orr[16], nr[16];
-                if (len > 0) tmem_ld_16x256b_x4(t_tile + C::COL_O + cc * 32, orr);
-                if (linear) tmem_ld_16x256b_x4(t_tile + cc * 32, nr);
-                tmem_wait_ld();
+                if (len > 0 && linear) tmem_ld_16x256b_x4(t_tile + C::COL_O + cc * 32, orr, t_tile + cc * 32, nr);
+                else if (len > 0) tmem_ld_16x256b_x4(t_tile + C::COL_O + cc * 32, orr);
+                else if (linear) tmem_ld_16x256b_x4(t_tile + cc * 32, nr);
                 const uint32_t oa = sb + C::OFF_V + (cc >> 1) * C::Q_CHUNK + ra * 128 + q4 * 4;        // over the V ring
 #pragma unroll
                 for (int n = 0; n < 4; ++n) {

@@ -284,7 +284,6 @@ salad_linear_apply_kernel(const __grid_constant__ CUtensorMap map_q, const __gri
             for (int cc = 0; cc < D / 16; ++cc) {
                 uint32_t nr[16];
                 tmem_ld16(t_row + ab * D + cc * 16, nr);
-                tmem_wait_ld();
 #pragma unroll
                 for (int c8 = 0; c8 < 2; ++c8) {
                     uint32_t w[4];

@@ -277,7 +277,7 @@ salad_linear_state_kernel(const __grid_constant__ CUtensorMap map_k, const __gri
 #pragma unroll
             for (int cc = cc0; cc < cc0 + NCC; ++cc) {
                 uint32_t r[32];
-                if (nblk > 0) { tmem_ld32(t_row + cc * 32, r); tmem_wait_ld(); }
+                if (nblk > 0) tmem_ld32(t_row + cc * 32, r);
                 if (a < D) {
 #pragma unroll
                     for (int c = 0; c < 32; c += 4) {
@@ -290,7 +290,7 @@ salad_linear_state_kernel(const __grid_constant__ CUtensorMap map_k, const __gri
             }
             if (!ROPE) {
                 uint32_t zr[32];
-                if (nblk > 0) { tmem_ld32(t_row + D, zr); tmem_wait_ld(); }   // reads 32 columns, uses the first
+                if (nblk > 0) tmem_ld32(t_row + D, zr);   // reads 32 columns, uses the first
                 if (a < D) z_out_ptr[a] = nblk > 0 ? __uint_as_float(zr[0]) : 0.f;
             }
         }

@@ -134,7 +134,6 @@ salad_proj_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
             for (int cc = 0; cc < C::BN / 32; ++cc) {
                 uint32_t acc[32];
                 tmem_ld32(t_row + ab * C::BN + cc * 32, acc);
-                tmem_wait_ld();
                 const int j0 = nt * C::BN + cc * 32;                // first output channel of this chunk
                 if (n < p.N && j0 < p.D) {
                     const size_t idx = ((size_t(b) * p.H + j0 / p.d) * p.N + n) * p.d + j0 % p.d;
@@ -316,7 +315,6 @@ salad_proj_gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __g
                 const int cc = cc0 + u;
                 uint32_t acc[32];
                 tmem_ld32(t_row + ab * 256 + cc * 32, acc);
-                tmem_wait_ld();
                 const int j0 = nt * C::BN + cc * 32;                // first output channel of this chunk
                 if (n < p.N && j0 < p.D) {
                     const size_t idx = ((size_t(b) * p.H + j0 / p.d) * p.N + n) * p.d + j0 % p.d;

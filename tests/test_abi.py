@@ -177,3 +177,17 @@ def test_registers_left_to_the_producer_warps(lib, tmp_path):
     assert done.returncode == 0, done.stderr[-2000:]
     took = [int(n) for n in re.findall(r"Used (\d+) registers", done.stderr)]
     assert len(took) == len(kinds) and max(took) <= dec, (took, dec)
+
+
+def test_tensor_memory_loads_wait_where_they_load():
+    """tcgen05.ld is asynchronous and its wait names no register: one statement issues a load and waits for it, or the compiler
+    may use (or copy) the registers in between."""
+    csrc, loads = os.path.join(ROOT, "paper_2601_16515_b200", "csrc"), 0
+    for name in sorted(os.listdir(csrc)):
+        text = re.sub(r"//[^\n]*", "", open(os.path.join(csrc, name)).read())
+        for statement in re.findall(r"\basm\b[^;]*?\((?:\"(?:[^\"\\]|\\.)*\"|[^\"])*?\)\s*;", text):
+            code = "".join(re.findall(r"\"((?:[^\"\\]|\\.)*)\"", statement))
+            if "tcgen05.ld." in code or "tcgen05.wait::ld" in code:
+                loads += 1
+                assert "tcgen05.ld." in code and "tcgen05.wait::ld" in code[code.rindex("tcgen05.ld."):], (name, statement[:120])
+    assert loads >= 4
