@@ -11,11 +11,13 @@ import os
 import subprocess
 import sys
 import sysconfig
+import warnings
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libsalad.so")
-FASTCALL = os.path.join(HERE, "_fastcall.so")            # CPython module, see csrc/fastcall.cpp
+# CPython module, see csrc/fastcall.cpp; named for the interpreter whose headers it is compiled with
+FASTCALL = os.path.join(HERE, "_fastcall" + sysconfig.get_config_var("EXT_SUFFIX"))
 SOURCES = ["salad_api.cu"]
 HEADERS = ["ptx.cuh", "tmap.cuh", "mask_kernels.cuh", "linear_state_kernel.cuh", "fused_kernel.cuh",
            "dynamic_scale_kernel.cuh", "linear_apply_kernel.cuh", "topk_mask_kernels.cuh", "permute_kernel.cuh", "proj_gemm_kernel.cuh",
@@ -57,8 +59,15 @@ def build(force: bool = False, verbose: bool = False) -> str:
         os.replace(tmp, LIB)
     if force or _fastcall_needs_build():
         tmp = FASTCALL + f".{os.getpid()}.tmp"
-        subprocess.check_call(fastcall_command(tmp))
-        os.replace(tmp, FASTCALL)
+        try:
+            subprocess.check_call(fastcall_command(tmp))
+            os.replace(tmp, FASTCALL)
+        except (OSError, subprocess.CalledProcessError) as e:
+            # The binding does without it (its calls go through ctypes then), but not with one of other sources.
+            for stale in (tmp, FASTCALL):
+                if os.path.exists(stale):
+                    os.remove(stale)
+            warnings.warn(f"{os.path.basename(FASTCALL)} not built, calls go through ctypes: {e}", RuntimeWarning)
     return LIB
 
 

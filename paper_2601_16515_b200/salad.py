@@ -9,10 +9,13 @@ implementation to fall back to: if the library is missing, importing this module
 from __future__ import annotations
 
 import ctypes
+import importlib.util
 import os
 from typing import Optional, Sequence, Tuple
 
 import torch
+
+from . import build
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "libsalad.so")
@@ -110,11 +113,13 @@ _lib = _load()
 
 
 def _load_fast():
-    """{name: function} of the calls that do not go through ctypes (csrc/fastcall.cpp); empty where that module was not built."""
-    try:
-        from . import _fastcall
-    except ImportError:
+    """{name: function} of the calls that do not go through ctypes (csrc/fastcall.cpp); empty where that module was not built
+    for this interpreter."""
+    if not os.path.exists(build.FASTCALL):
         return {}
+    spec = importlib.util.spec_from_file_location(__package__ + "._fastcall", build.FASTCALL)
+    _fastcall = importlib.util.module_from_spec(spec)
+    spec.loader.exec_module(_fastcall)
     return {name: getattr(_fastcall, name) for name in EXPORTS
             if _fastcall.bind(name, ctypes.cast(getattr(_lib, name), ctypes.c_void_p).value)}
 

@@ -5,6 +5,7 @@ import os
 import re
 import subprocess
 import sys
+import sysconfig
 
 import pytest
 
@@ -191,3 +192,28 @@ def test_tensor_memory_loads_wait_where_they_load():
                 loads += 1
                 assert "tcgen05.ld." in code and "tcgen05.wait::ld" in code[code.rindex("tcgen05.ld."):], (name, statement[:120])
     assert loads >= 4
+
+
+def test_without_the_native_module(lib, tmp_path, monkeypatch):
+    """The module that bypasses ctypes is named for its interpreter, the build goes on without it where it cannot be compiled (and
+    leaves none of other sources), and the binding answers the same through ctypes."""
+    from paper_2601_16515_b200 import build
+    assert os.path.basename(build.FASTCALL) == "_fastcall" + sysconfig.get_config_var("EXT_SUFFIX")
+    stale = tmp_path / os.path.basename(build.FASTCALL)
+    monkeypatch.setattr(build, "FASTCALL", str(stale))
+    for command in (["no-such-compiler"], [sys.executable, "-c", "raise SystemExit(1)"]):
+        stale.write_bytes(b"")
+        os.utime(stale, (0, 0))
+        monkeypatch.setattr(build, "fastcall_command", lambda out: command)
+        with pytest.warns(RuntimeWarning, match="not built"):
+            assert build.build() == build.LIB
+        assert not os.listdir(tmp_path)
+    code = ("from paper_2601_16515_b200 import build\n"
+            "build.FASTCALL += '.absent'\n"
+            "from paper_2601_16515_b200 import salad\n"
+            "p, n = 1 << 20, salad.salad_workspace_bytes(1, 2, 1024, 64, 64, 64)\n"
+            "good = [p, p, p, p, 1, 2, 1024, 64, 64, 64, p, p, 2, p, p, 0.0, 1e-6, p, n, None, None]\n"
+            "assert salad._fast == {}\n"
+            "assert salad._enter('salad_fused_fwd', None, *good[1:]) == salad.SALAD_ERR_INVALID_ARG\n"
+            "assert salad._enter('salad_fused_fwd', *good[:18], n - 1, None, None) == salad.SALAD_ERR_WORKSPACE\n")
+    subprocess.run([sys.executable, "-c", code], cwd=ROOT, check=True)
