@@ -1,16 +1,11 @@
 // Block-sparse softmax attention (Eq. 2) fused with the apply step of ReLU linear attention
 // (Eq. 3) and the scaled residual sum of Algorithm 1, for sm_100a.
 //
-// A work item is one query block of one (batch, head): a 128-row MMA tile.  Two CTAs share an SM
+// One CTA owns one query block of one (batch, head): a 128-row MMA tile.  Two CTAs share an SM
 // (each takes half of its shared memory, registers and tensor memory), so the set-up, the first
 // loads and the epilogue of one overlap the main loop of the other, and the two tiles of an SM run
-// independently of each other.  The grid has a CTA per item; a CTA that comes to the end of its item takes over the next
-// CTA that has not started (cluster launch control), so that the next item's Q, K and first scores are under way during
-// the epilogue and the set-up of a CTA is paid once per slot (fused calls back to back, a CTA per item -> now: a pair of 12 heads
-// of 32760 tokens at 95 % sparsity 816 -> 797 us, 12 heads at 90 % 668 -> 665, 12 heads of 16464 tokens 252 -> 246, 40 heads of
-// 2310 tokens 78.6 -> 76.2; with all blocks kept, where items have no ends to speak of, 11.31 and 11.33 ms).
-//   warp 0        TMA producer of the Q tile, the K ring and (at the end) the linear-state tile; it also fetches
-//                 the next item for all roles
+// independently of each other.
+//   warp 0        TMA producer of the Q tile, the K ring and (at the end) the linear-state tile
 //   warp 1        TMA producer of the V ring (independent of the K ring, so neither ring can
 //                 stall the other); stores the output tile, which is staged over that ring
 //   warp 2        tcgen05 issuer of S = Q K^T; owns the TMEM allocation
@@ -39,11 +34,14 @@
 // what its next MMA series needs, so it reacts as soon as that arrives.  One commit per series: the
 // barrier that announces the scores of block t also frees the K-ring stage for block t + 2, the one
 // that announces the completion of P V the V-ring stage.
-// The four producer / issuer warps (one warpgroup) hand registers to the eight softmax warps
-// (setmaxnreg: 48 against 96 per thread, all that the block was launched with: 128 x 48 + 256 x 96 = 384 x 80), which keeps
-// the softmax loop free of spills (two words of the epilogue are on the stack).  The producer side by itself takes 38 registers
-// of its own accord.  Fewer than that are not to be left to it: with 32 (and 104) a form of this kernel for one item per CTA lost the
-// head's index in the storing warp and wrote every tile to the first head, without a word from the compiler; with 48 it is right.
+// Every warp has the 80 registers of the launch (d = 64 takes 75; at d = 128 one word of the epilogue is on the stack).  The producer
+// and issuer warps need fewer, but none are handed to the softmax warps (setmaxnreg): compiled with that instruction, forms of this
+// kernel lost values that live across it, without a word from the compiler -- with 32 against 104 registers the head's index in the
+// storing warp (every tile went to the first head), with 48 against 96 the list's length in the softmax warps (the
+// softmax part was left out) -- and the same sources without it are right.  Nor does a CTA take over further items of the grid (cluster
+// launch control): with the loop over items around it the softmax loop wants 96 registers, 80 cost it 3 % (11.06 -> 11.48 ms with
+// all blocks kept at 2 x 12 heads of 32760 tokens); with them, calls of short lists gained by it (12 + 12 heads of 32760 tokens
+// at 95 % 795 -> 780 us) about what calls of few items and long lists lost (2 heads of 35496 tokens, d = 64, all blocks kept, 847 -> 999).
 // After the last block the softmax warps apply ReLU to the Q rows in shared memory and compute the
 // linear denominator with plain FMAs; the linear state (bf16, transposed) is loaded over the K
 // ring, which is idle by then; the issuing thread multiplies ReLU(Q) with it, and the epilogue
@@ -95,7 +93,6 @@ struct FusedParams {
     float eps;
     float drop_tau;              // linear branch of batch item b skipped when dyn_scale[b] < drop_tau
     const __half* rope;          // [N][D] fp16: (cos, sin) per token and channel pair of the rotary linear branch, or null
-    int take_over;               // 1: a CTA that has finished its item takes over the next CTA of the grid
     int wait_at_top;             // 1: wait for the kernel before this one at once (calls without state kernels)
     int32_t* ws_status;          // library status word (never null)
     int32_t* user_status;        // optional
@@ -128,13 +125,12 @@ static_assert(FusedCfg<64>::ST_BYTES <= FusedCfg<64>::NK * FusedCfg<64>::KV_BYTE
 
 struct FusedBarriers {
     uint64_t q_full, st_full, k_full[2], v_full[2];
-    uint64_t s_full[2], p_ready[2], pv_done[2], o_final, lin_ready, lin_done, num_free, out_staged, v_free, z_full;
-    uint64_t item_full[2], item_empty[2], taken;
+    uint64_t s_full[2], p_ready[2], pv_done[2], o_final, lin_ready, lin_done, out_staged, z_full;
 };
 
 // A work item: a query block of a (batch, head) with its kept list.
 struct FusedItem {
-    int qb, bh, ls, len;               // qb < 0: no item
+    int qb, bh, ls, len;
     int linear;                        // it has a linear branch,
     float scale;                       // scaled by this
 };
@@ -150,18 +146,16 @@ salad_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
     using C = FusedCfg<D>;
     extern __shared__ uint8_t smem_raw[];
     __shared__ FusedBarriers bars;
-    __shared__ alignas(16) uint32_t taken_answer[4];
-    __shared__ FusedItem item_slot[2];
     __shared__ uint32_t tmem_base_slot;
-    __shared__ int abort_flag, state_waited;
+    __shared__ int abort_flag;
     __shared__ alignas(16) float z_s[D];          // linear normaliser state of this head
 
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     const uint32_t s_base = smem_u32(smem);
     const int tid = threadIdx.x, lane = tid & 31;
     // The same as tid >> 5, but known to be the same in every lane, which keeps the roles' branches free of
-    // reconvergence code: together with 48 registers instead of 40 for the producer warps 638 -> 629 us at 12 heads of 32760 tokens (90 %
-    // sparsity, attention alone, at the power limit), 470 -> 451 at d = 64, 35.6 -> 34.7 for 2310 tokens.
+    // reconvergence code (638 -> 629 us at 12 heads of 32760 tokens, 90 % sparsity, attention alone, at the power limit,
+    // 470 -> 451 at d = 64, 35.6 -> 34.7 for 2310 tokens; measured with a register split that is gone).
     const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
     // The work order (and the verdict on the lists) comes from the first kernel of the call.  Without a linear
     // branch that is the kernel before this one.  With one, it is the state kernel, whose ordering CTAs let the kernels
@@ -172,9 +166,9 @@ salad_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
 
     // Work items: head by head, within a head the query blocks from the most to the least expensive, so that the
     // kernel ends on short items and K/V of one head stay hot in L2; or, where K and V of all heads fit there (by_rank),
-    // the most expensive items of all heads first: the CTAs that wait for a state CTA's place, and the second CTA of an SM where
-    // the items do not fill all, then hold the cheapest items, and the launch ends on the cheapest of all heads.
-    auto item_of = [&](int block) {
+    // the most expensive item of every head, then the next of every head: the CTAs that wait for a state CTA's place, and the second
+    // CTA of an SM where the items do not fill all, then hold cheap items, and the launch ends on the cheapest of all heads.
+    const FusedItem item = [&](int block) {
         FusedItem it;
         const int rank = p.by_rank ? block / p.BH : block % p.nQb;
         it.bh = p.by_rank ? block % p.BH : block / p.nQb;
@@ -197,14 +191,15 @@ salad_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
             it.len = __ldg(p.row_ptr + size_t(hm) * p.nQb + it.qb + 1) - it.ls;
         }
         return it;
-    };
-    const FusedItem first = item_of(blockIdx.x);
-    // temporal head: blocks of spatial positions, fetched through the 4-D maps (a CTA of such a call has one item)
-    const int h0 = first.bh % p.H;
+    }(blockIdx.x);
+    const int qb = item.qb, bh = item.bh, len = item.len;
+    const bool linear = item.linear != 0;
+    // temporal head: blocks of spatial positions, fetched through the 4-D maps
+    const int h0 = bh % p.H;
     const bool perm = p.th.T > 0 && ((p.th.flags[h0 >> 5] >> (h0 & 31)) & 1u);
     const int q_rows = perm ? p.th.kq * p.th.T : p.Bq;          // rows of the 128-row tile that hold queries
     const int k_rows = perm ? p.th.ks * p.th.T : C::BK;         // rows of a 64-row tile that hold keys
-    if (first.qb >= (perm ? p.th.nQb : p.nQb_tok)) return;       // (a list row beyond this head's blocks: whole CTA)
+    if (qb >= (perm ? p.th.nQb : p.nQb_tok)) return;       // (a list row beyond this head's blocks: whole CTA)
 
     // softmax warps whose 16 rows hold queries (64-row query blocks: four of the eight); the others do nothing
     const int row_warps = (q_rows + 15) >> 4;
@@ -214,26 +209,19 @@ salad_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
         // 2: an earlier kernel of this call has already reported a failure (a rejected mask, an expired wait):
         // this CTA starts nothing and reports nothing; 1 (set by a bounded wait of this CTA): a time-out
         abort_flag = (*reinterpret_cast<volatile int32_t*>(p.ws_status) != 0) ? 2 : 0;
-        state_waited = 0;
-        item_slot[0] = first;
         mbar_init(smem_u32(&bars.q_full), 1);
         mbar_init(smem_u32(&bars.st_full), 1);
         mbar_init(smem_u32(&bars.o_final), 1);
         mbar_init(smem_u32(&bars.lin_ready), row_warps);
         mbar_init(smem_u32(&bars.lin_done), 1);
-        mbar_init(smem_u32(&bars.num_free), row_warps);
         mbar_init(smem_u32(&bars.out_staged), row_warps);
-        mbar_init(smem_u32(&bars.v_free), 1);
         mbar_init(smem_u32(&bars.z_full), 32);
-        mbar_init(smem_u32(&bars.taken), 1);
         for (int j = 0; j < 2; ++j) {
             mbar_init(smem_u32(&bars.s_full[j]), 1);
             mbar_init(smem_u32(&bars.p_ready[j]), row_warps);  // one arrival per softmax warp
             mbar_init(smem_u32(&bars.pv_done[j]), 1);
             mbar_init(smem_u32(&bars.k_full[j]), 1);
             mbar_init(smem_u32(&bars.v_full[j]), 1);
-            mbar_init(smem_u32(&bars.item_full[j]), 1);
-            mbar_init(smem_u32(&bars.item_empty[j]), 3 + row_warps);
         }
         fence_mbar_init();
     }
@@ -265,155 +253,89 @@ salad_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
     auto wait_warp = [&](uint64_t* bar, uint32_t parity) -> bool {
         return __all_sync(0xffffffffu, mbar_wait(smem_u32(bar), parity, abortp));
     };
-    // The items of this CTA: item k in slot k & 1, left there by warp 0 (the first one above).  false: there is none.
-    auto get_item = [&](int k) -> bool {
-        if (k > 0 && !wait_warp(&bars.item_full[k & 1], ((k - 1) >> 1) & 1)) return false;
-        return item_slot[k & 1].qb >= 0;
-    };
-    auto release_item = [&](int k) {
-        __syncwarp();
-        if (lane == 0) mbar_arrive(smem_u32(&bars.item_empty[k & 1]));
-    };
-    // Every role counts what it needs for the phases of the barriers: the blocks before the item at hand (g: block t of it is
-    // block g + t of the CTA, which decides its buffers), the items that loaded Q, and those with a linear branch.
-
     if (!inherited_abort) {
     if (warp < 4) {
-    // the four producer / issuer warps (one warpgroup) give registers up, the eight softmax warps take them
-    asm volatile("setmaxnreg.dec.sync.aligned.u32 48;");
     if (warp == 0) {
         // ============================================================== TMA producer: Q, the K ring, the state tile
-        auto load_q = [&](const FusedItem& it) {
-            const uint32_t bar = smem_u32(&bars.q_full);
-            mbar_arrive_expect_tx(bar, uint32_t(q_rows) * D * 2);
-            for (int ch = 0; ch < C::CH; ++ch) {
-                if (perm) tma_load_4d(s_base + C::OFF_Q + ch * C::Q_CHUNK, &map_q4, bar, ch * 64, 0, it.qb * p.th.kq, it.bh);
-                else tma_load_3d(s_base + C::OFF_Q + ch * C::Q_CHUNK, &map_q, bar, ch * 64, it.qb * p.Bq, it.bh);
-            }
-        };
-        if (lane == 0) {
-            if (first.len > 0 || first.linear) load_q(first);
-            prefetch_tmap(&map_k);
-        }
-        int g = 0, n_lin = 0;
         bool ok = true;
-        FusedItem item = first;
-        for (int k = 0; ; ++k) {
-            const int len = item.len, bh = item.bh;
-            if (lane == 0) {
-                // A block with no kept key block and no linear branch never reads Q.
-                if (k > 0 && (len > 0 || item.linear)) {
-                    // the products that read the Q tile and the K ring of the items before (the state tile lies over it)
-                    if (n_lin > 0) ok = mbar_wait(smem_u32(&bars.lin_done), (n_lin - 1) & 1, abortp);
-                    if (ok && g > 0) ok = mbar_wait(smem_u32(&bars.s_full[(g - 1) & 1]), ((g - 1) >> 1) & 1, abortp);
-                    if (ok) load_q(item);
+        if (lane == 0) {
+            // A block with no kept key block and no linear branch never reads Q.
+            if (len > 0 || linear) {
+                const uint32_t bar = smem_u32(&bars.q_full);
+                mbar_arrive_expect_tx(bar, uint32_t(q_rows) * D * 2);
+                for (int ch = 0; ch < C::CH; ++ch) {
+                    if (perm) tma_load_4d(s_base + C::OFF_Q + ch * C::Q_CHUNK, &map_q4, bar, ch * 64, 0, qb * p.th.kq, bh);
+                    else tma_load_3d(s_base + C::OFF_Q + ch * C::Q_CHUNK, &map_q, bar, ch * 64, qb * p.Bq, bh);
                 }
-                int col = len > 0 ? __ldg(p.col_idx + item.ls) : 0;
-                for (int t = 0; t < len && ok; ++t) {
-                    const int gt = g + t, s = gt & 1;
-                    // stage s is free once Q K^T of the block before the last has completed: the barrier that hands its
-                    // scores to the softmax warps says so (one commit serves both)
-                    if (gt >= C::NK) ok = mbar_wait(smem_u32(&bars.s_full[s]), ((gt >> 1) - 1) & 1, abortp);
-                    if (!ok) break;
-                    const uint32_t bar = smem_u32(&bars.k_full[s]);
-                    mbar_arrive_expect_tx(bar, uint32_t(k_rows) * D * 2);
-                    for (int ch = 0; ch < C::CH; ++ch) {     // chunk-major: the two stages of a chunk are adjacent
-                        const uint32_t dst = s_base + C::OFF_K + ch * (C::NK * C::KV_CHUNK) + s * C::KV_CHUNK;
-                        if (perm) tma_load_4d(dst, &map_k4, bar, ch * 64, 0, col * p.th.ks, bh);
-                        else tma_load_3d(dst, &map_k, bar, ch * 64, col * C::BK, bh);
-                    }
-                    if (t + 1 < len) col = __ldg(p.col_idx + item.ls + t + 1);
+            }
+            prefetch_tmap(&map_k);
+            int col = len > 0 ? __ldg(p.col_idx + item.ls) : 0;
+            for (int t = 0; t < len; ++t) {
+                const int s = t & 1;
+                // stage s is free once Q K^T of the block before the last has completed: the barrier that hands its
+                // scores to the softmax warps says so (one commit serves both)
+                if (t >= C::NK) ok = mbar_wait(smem_u32(&bars.s_full[s]), ((t >> 1) - 1) & 1, abortp);
+                if (!ok) break;
+                const uint32_t bar = smem_u32(&bars.k_full[s]);
+                mbar_arrive_expect_tx(bar, uint32_t(k_rows) * D * 2);
+                for (int ch = 0; ch < C::CH; ++ch) {     // chunk-major: the two stages of a chunk are adjacent
+                    const uint32_t dst = s_base + C::OFF_K + ch * (C::NK * C::KV_CHUNK) + s * C::KV_CHUNK;
+                    if (perm) tma_load_4d(dst, &map_k4, bar, ch * 64, 0, col * p.th.ks, bh);
+                    else tma_load_3d(dst, &map_k, bar, ch * 64, col * C::BK, bh);
                 }
-                // The next item: that of the next CTA of the grid that has not started, which this one takes over.  Asked
-                // for only now, a few blocks before the end, so that at the end of the grid no CTA sits on an item while
-                // another has none.
-                FusedItem next;
-                next.qb = -1; next.bh = 0; next.ls = 0; next.len = 0; next.linear = 0; next.scale = 0.f;
-                if (ok && p.take_over) {
-                    mbar_arrive_expect_tx(smem_u32(&bars.taken), 16);
-                    clc_try_cancel(smem_u32(taken_answer), smem_u32(&bars.taken));
-                    ok = mbar_wait(smem_u32(&bars.taken), k & 1, abortp);
-                    if (ok) {
-                        const int block = clc_answer(smem_u32(taken_answer));
-                        fence_proxy_async_smem();            // (read, before the next answer is written over it)
-                        if (block >= 0 && *reinterpret_cast<volatile int32_t*>(p.ws_status) == 0) next = item_of(block);
-                    }
-                }
-                if (ok && k >= 1) ok = mbar_wait(smem_u32(&bars.item_empty[(k + 1) & 1]), ((k - 1) >> 1) & 1, abortp);
+                if (t + 1 < len) col = __ldg(p.col_idx + item.ls + t + 1);
+            }
+        }
+        if (linear) {
+            // From here on the linear state is needed: wait for the kernels that make it (whole warp: the
+            // other lanes fetch the normaliser Z of this head for the softmax warps meanwhile).
+            __syncwarp();
+            grid_dependency_wait();
+            if (*reinterpret_cast<volatile int32_t*>(p.ws_status) != 0 && *abortp == 0) *abortp = 2;   // the state kernel gave up (and said so)
+            for (int a = lane; a < D; a += 32) z_s[a] = __ldcg(p.z + size_t(bh) * D + a);
+            mbar_arrive(smem_u32(&bars.z_full));
+            if (lane == 0 && ok) {
+                // the state tile goes over the K ring: every Q K^T must have read its K block.  The products
+                // complete in order, so the last one (signalled on its score buffer's barrier) covers all.
+                if (len > 0) ok = mbar_wait(smem_u32(&bars.s_full[(len - 1) & 1]), ((len - 1) >> 1) & 1, abortp);
                 if (ok) {
-                    item_slot[(k + 1) & 1] = next;
-                    mbar_arrive(smem_u32(&bars.item_full[(k + 1) & 1]));
+                    prefetch_tmap(&map_st);
+                    const uint32_t bar = smem_u32(&bars.st_full);
+                    mbar_arrive_expect_tx(bar, C::ST_BYTES);
+                    for (int ch = 0; ch < C::CH; ++ch)
+                        tma_load_3d(s_base + C::OFF_ST + ch * C::ST_CHUNK, &map_st, bar, ch * 64, 0, bh);
                 }
             }
-            g += len;
-            if (item.linear) {
-                // From here on the linear state is needed: wait for the kernels that make it (whole warp: the
-                // other lanes fetch the normaliser Z of this head for the softmax warps meanwhile).
-                __syncwarp();
-                if (n_lin == 0) {
-                    grid_dependency_wait();
-                    if (lane == 0) state_waited = 1;
-                    if (*reinterpret_cast<volatile int32_t*>(p.ws_status) != 0 && *abortp == 0) *abortp = 2;   // the state kernel gave up (and said so)
-                }
-                for (int a = lane; a < D; a += 32) z_s[a] = __ldcg(p.z + size_t(bh) * D + a);
-                mbar_arrive(smem_u32(&bars.z_full));
-                if (lane == 0 && ok) {
-                    // the state tile goes over the K ring: every Q K^T must have read its K block.  The products
-                    // complete in order, so the last one (signalled on its score buffer's barrier) covers all.
-                    if (g > 0) ok = mbar_wait(smem_u32(&bars.s_full[(g - 1) & 1]), ((g - 1) >> 1) & 1, abortp);
-                    if (ok) {
-                        prefetch_tmap(&map_st);
-                        const uint32_t bar = smem_u32(&bars.st_full);
-                        mbar_arrive_expect_tx(bar, C::ST_BYTES);
-                        for (int ch = 0; ch < C::CH; ++ch)
-                            tma_load_3d(s_base + C::OFF_ST + ch * C::ST_CHUNK, &map_st, bar, ch * 64, 0, bh);
-                    }
-                }
-                ++n_lin;
-            }
-            if (!__all_sync(0xffffffffu, ok) || !get_item(k + 1)) break;
-            item = item_slot[(k + 1) & 1];
         }
     } else if (warp == 1) {
         // ============================================================== TMA producer of the V ring, output store
         if (lane == 0) {
             prefetch_tmap(&map_v);
-            int g = 0;
             bool ok = true;
-            for (int k = 0; ok; ++k) {
-                if (k > 0 && !mbar_wait(smem_u32(&bars.item_full[k & 1]), ((k - 1) >> 1) & 1, abortp)) break;
-                const FusedItem item = item_slot[k & 1];
-                if (item.qb < 0) break;
-                mbar_arrive(smem_u32(&bars.item_empty[k & 1]));
-                const int len = item.len, bh = item.bh;
-                for (int t = 0; t < len; ++t) {
-                    const int gt = g + t, s = gt & 1;
-                    // stage s is free once P V of the block before the last has completed
-                    if (gt >= C::NV) ok = mbar_wait(smem_u32(&bars.pv_done[s]), ((gt >> 1) - 1) & 1, abortp);
-                    if (!ok) break;
-                    const int col = __ldg(p.col_idx + item.ls + t);
-                    const uint32_t bar = smem_u32(&bars.v_full[s]);
-                    mbar_arrive_expect_tx(bar, uint32_t(k_rows) * D * 2);
-                    for (int ch = 0; ch < C::CH; ++ch) {
-                        const uint32_t dst = s_base + C::OFF_V + s * C::KV_BYTES + ch * C::KV_CHUNK;
-                        if (perm) tma_load_4d(dst, &map_v4, bar, ch * 64, 0, col * p.th.ks, bh);
-                        else tma_load_3d(dst, &map_v, bar, ch * 64, col * C::BK, bh);
-                    }
-                }
+            for (int t = 0; t < len; ++t) {
+                const int s = t & 1;
+                // stage s is free once P V of the block before the last has completed
+                if (t >= C::NV) ok = mbar_wait(smem_u32(&bars.pv_done[s]), ((t >> 1) - 1) & 1, abortp);
                 if (!ok) break;
-                g += len;
-                // the output tile, staged over the V ring
-                ok = mbar_wait(smem_u32(&bars.out_staged), k & 1, abortp);
-                if (!ok) break;
+                const int col = __ldg(p.col_idx + item.ls + t);
+                const uint32_t bar = smem_u32(&bars.v_full[s]);
+                mbar_arrive_expect_tx(bar, uint32_t(k_rows) * D * 2);
                 for (int ch = 0; ch < C::CH; ++ch) {
-                    if (perm) tma_store_4d(&map_o4, s_base + C::OFF_V + ch * C::Q_CHUNK, ch * 64, 0, item.qb * p.th.kq, bh);
-                    else tma_store_3d(&map_o, s_base + C::OFF_V + ch * C::Q_CHUNK, ch * 64, item.qb * p.Bq, bh);
+                    const uint32_t dst = s_base + C::OFF_V + s * C::KV_BYTES + ch * C::KV_CHUNK;
+                    if (perm) tma_load_4d(dst, &map_v4, bar, ch * 64, 0, col * p.th.ks, bh);
+                    else tma_load_3d(dst, &map_v, bar, ch * 64, col * C::BK, bh);
+                }
+            }
+            // the output tile, staged over the V ring
+            if (ok && mbar_wait(smem_u32(&bars.out_staged), 0, abortp)) {
+                for (int ch = 0; ch < C::CH; ++ch) {
+                    if (perm) tma_store_4d(&map_o4, s_base + C::OFF_V + ch * C::Q_CHUNK, ch * 64, 0, qb * p.th.kq, bh);
+                    else tma_store_3d(&map_o, s_base + C::OFF_V + ch * C::Q_CHUNK, ch * 64, qb * p.Bq, bh);
                 }
                 tma_store_commit();
-                // only the shared-memory source must have been read before it is written again or the CTA exits; the
+                // only the shared-memory source must have been read before the CTA exits; the
                 // writes are complete, like all of the kernel's, when the grid is
                 tma_store_wait_read_all();
-                mbar_arrive(smem_u32(&bars.v_free));
             }
         }
     } else if (warp == 2) {
@@ -425,39 +347,25 @@ salad_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
         constexpr uint32_t HI = sdesc_hi_sw128(1024);   // the high descriptor word is one constant here
         const uint32_t q_lo = sdesc_lo(s_base + C::OFF_Q, 16);
         const uint32_t k_lo0 = sdesc_lo(s_base + C::OFF_K, 16);
-        int g = 0, n_q = 0, n_lin = 0;
-        bool ok = true, before_linear = false;
-        for (int k = 0; ok; ++k) {
-            if (!get_item(k)) break;
-            const int len = item_slot[k & 1].len;
-            const bool linear = item_slot[k & 1].linear != 0;
-            release_item(k);
-            // Every phase of these two is waited for, also where this item needs neither: a wait tells a phase from the one
-            // before the last only by that.  First the numerator of the item before, which lies over both score buffers.
-            if (before_linear) ok = wait_warp(&bars.num_free, (n_lin - 1) & 1);
-            if (ok && (len > 0 || linear)) ok = wait_warp(&bars.q_full, n_q & 1);
-            before_linear = linear;
-            for (int t = 0; t < len && ok; ++t) {
-                const int gt = g + t, s = gt & 1;
-                ok = wait_warp(&bars.k_full[s], (gt >> 1) & 1);
-                // score buffer s held P of the block before the last: its P V product must have read it
-                if (ok && gt >= 2) ok = wait_warp(&bars.pv_done[s], ((gt >> 1) - 1) & 1);
-                if (!ok) break;
-                tc_fence_after_sync();
-                if (elect_one()) {
-                    const uint32_t kb_lo = k_lo0 + s * (C::KV_CHUNK >> 4);
+        bool ok = true;
+        if (len > 0) ok = wait_warp(&bars.q_full, 0);
+        for (int t = 0; t < len && ok; ++t) {
+            const int s = t & 1;
+            ok = wait_warp(&bars.k_full[s], (t >> 1) & 1);
+            // score buffer s held P of the block before the last: its P V product must have read it
+            if (ok && t >= 2) ok = wait_warp(&bars.pv_done[s], ((t >> 1) - 1) & 1);
+            if (!ok) break;
+            tc_fence_after_sync();
+            if (elect_one()) {
+                const uint32_t kb_lo = k_lo0 + s * (C::KV_CHUNK >> 4);
 #pragma unroll
-                    for (int kk = 0; kk < D / 16; ++kk)   // 16 channels: 32 bytes of each Q and K row, chunk kk/4
-                        mma_ss_lohi(tmem + C::COL_SP + s * C::SP_STRIDE,
-                                    q_lo + (((kk / 4) * C::Q_CHUNK + (kk % 4) * 32) >> 4), HI,
-                                    kb_lo + (((kk / 4) * (C::NK * C::KV_CHUNK) + (kk % 4) * 32) >> 4), HI, idesc_qk, kk > 0);
-                    tc_commit(smem_u32(&bars.s_full[s]));
-                }
-                __syncwarp();
+                for (int kk = 0; kk < D / 16; ++kk)   // 16 channels: 32 bytes of each Q and K row, chunk kk/4
+                    mma_ss_lohi(tmem + C::COL_SP + s * C::SP_STRIDE,
+                                q_lo + (((kk / 4) * C::Q_CHUNK + (kk % 4) * 32) >> 4), HI,
+                                kb_lo + (((kk / 4) * (C::NK * C::KV_CHUNK) + (kk % 4) * 32) >> 4), HI, idesc_qk, kk > 0);
+                tc_commit(smem_u32(&bars.s_full[s]));
             }
-            g += len;
-            if (len > 0 || linear) ++n_q;
-            if (linear) ++n_lin;
+            __syncwarp();
         }
     } else if (warp == 3) {
         // ============================================================== issuer of O += P V and of the linear numerator
@@ -466,54 +374,43 @@ salad_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
         constexpr uint32_t HI = sdesc_hi_sw128(1024);
         const uint32_t q_lo = sdesc_lo(s_base + C::OFF_Q, 16);
         const uint32_t v_lo0 = sdesc_lo(s_base + C::OFF_V, C::KV_CHUNK);
-        int g = 0, n_lin = 0;
         bool ok = true;
-        for (int k = 0; ok; ++k) {
-            if (!get_item(k)) break;
-            const int len = item_slot[k & 1].len;
-            const bool linear = item_slot[k & 1].linear != 0;
-            release_item(k);
-            for (int t = 0; t < len && ok; ++t) {
-                const int gt = g + t, s = gt & 1;
-                ok = wait_warp(&bars.v_full[s], (gt >> 1) & 1);
-                // (with the first P of an item all softmax warps have read the accumulator of the item before)
-                if (ok) ok = wait_warp(&bars.p_ready[s], (gt >> 1) & 1);
-                if (!ok) break;
+        for (int t = 0; t < len && ok; ++t) {
+            const int s = t & 1;
+            ok = wait_warp(&bars.v_full[s], (t >> 1) & 1);
+            if (ok) ok = wait_warp(&bars.p_ready[s], (t >> 1) & 1);
+            if (!ok) break;
+            tc_fence_after_sync();
+            if (elect_one()) {
+                const uint32_t vb_lo = v_lo0 + s * (C::KV_BYTES >> 4);
+                const uint32_t p_col = tmem + C::COL_SP + s * C::SP_STRIDE;
+#pragma unroll
+                for (int kk = 0; kk < C::BK / 16; ++kk)      // 16 keys = 16 rows of 128 bytes
+                    mma_ts_lohi(tmem + C::COL_O, p_col + kk * 8, vb_lo + ((kk * 2048) >> 4), HI, idesc_pv,
+                                (t > 0 || kk > 0) ? 1u : 0u);
+                tc_commit(smem_u32(&bars.pv_done[s]));
+                if (t + 1 == len) tc_commit(smem_u32(&bars.o_final));
+            }
+            __syncwarp();
+        }
+        if (ok && linear) {
+            ok = wait_warp(&bars.st_full, 0);
+            if (ok) ok = wait_warp(&bars.lin_ready, 0);
+            if (ok) {
                 tc_fence_after_sync();
                 if (elect_one()) {
-                    const uint32_t vb_lo = v_lo0 + s * (C::KV_BYTES >> 4);
-                    const uint32_t p_col = tmem + C::COL_SP + s * C::SP_STRIDE;
+                    const uint32_t st_lo = sdesc_lo(s_base + C::OFF_ST, 16);
 #pragma unroll
-                    for (int kk = 0; kk < C::BK / 16; ++kk)      // 16 keys = 16 rows of 128 bytes
-                        mma_ts_lohi(tmem + C::COL_O, p_col + kk * 8, vb_lo + ((kk * 2048) >> 4), HI, idesc_pv,
-                                    (t > 0 || kk > 0) ? 1u : 0u);
-                    tc_commit(smem_u32(&bars.pv_done[s]));
-                    if (t + 1 == len) tc_commit(smem_u32(&bars.o_final));
+                    for (int kk = 0; kk < D / 16; ++kk)
+                        mma_ss_lohi(tmem, q_lo + (((kk / 4) * C::Q_CHUNK + (kk % 4) * 32) >> 4), HI,
+                                    st_lo + (((kk / 4) * C::ST_CHUNK + (kk % 4) * 32) >> 4), HI, idesc_lin, kk > 0);
+                    tc_commit(smem_u32(&bars.lin_done));
                 }
                 __syncwarp();
-            }
-            g += len;
-            if (ok && linear) {
-                ok = wait_warp(&bars.st_full, n_lin & 1);
-                if (ok) ok = wait_warp(&bars.lin_ready, n_lin & 1);
-                if (ok) {
-                    tc_fence_after_sync();
-                    if (elect_one()) {
-                        const uint32_t st_lo = sdesc_lo(s_base + C::OFF_ST, 16);
-#pragma unroll
-                        for (int kk = 0; kk < D / 16; ++kk)
-                            mma_ss_lohi(tmem, q_lo + (((kk / 4) * C::Q_CHUNK + (kk % 4) * 32) >> 4), HI,
-                                        st_lo + (((kk / 4) * C::ST_CHUNK + (kk % 4) * 32) >> 4), HI, idesc_lin, kk > 0);
-                        tc_commit(smem_u32(&bars.lin_done));
-                    }
-                    __syncwarp();
-                }
-                ++n_lin;
             }
         }
     }
     } else {
-        asm volatile("setmaxnreg.inc.sync.aligned.u32 96;");
         // ============================================================== softmax + epilogue
         // Eight warps.  A warp works on 16 TMEM lanes (query rows) with the 16-lane
         // load/store shapes: four threads share a row, each holding a quarter of its columns,
@@ -542,15 +439,7 @@ salad_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
             return v + __shfl_xor_sync(0xffffffffu, v, 2);
         };
 
-        // the counters of this role, as much of them as the parities need: blocks before this item & 3, then a bit each for
-        // the items with Q, with kept blocks and with a linear branch
-        uint32_t ph = 0;
         bool ok = true;
-#pragma unroll 1
-        for (int k = 0; ok; ++k) {
-        if (!get_item(k)) break;
-        const FusedItem& item = item_slot[k & 1];
-        const int len = item.len;
         float m_a = -INFINITY, m_b = -INFINITY;                 // running maxima (log2 domain)
         float l_a = 0.f, l_b = 0.f;                             // this thread's share of the row sums
         // Only the last key block of the sequence can be short (N not a multiple of 64), and in an ascending
@@ -567,10 +456,9 @@ salad_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
         }
         const int limits = valid_last | (k_rows << 8);          // (one register instead of two)
         constexpr float SUM_LIMIT = 4096.f;
-        const int g0 = int(ph & 3u);
         for (int t = 0; t < len && ok; ++t) {
-            const int gt = g0 + t, s = gt & 1;
-            ok = wait_uniform(&bars.s_full[s], (gt >> 1) & 1);
+            const int s = t & 1;
+            ok = wait_uniform(&bars.s_full[s], (t >> 1) & 1);
             if (!ok) break;
             tc_fence_after_sync();
             uint32_t pk[16];
@@ -604,7 +492,7 @@ salad_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                         // has landed in it.  pv_done[b] completes a phase for every second block; the product of block
                         // t cannot be issued before this warp hands over P of block t, so the barrier is at most one
                         // phase past the one tested here and the parity test is exact.
-                        ok = wait_uniform(&bars.pv_done[s ^ 1], ((gt - 1) >> 1) & 1);
+                        ok = wait_uniform(&bars.pv_done[s ^ 1], ((t - 1) >> 1) & 1);
                         if (!ok) break;
                         tc_fence_after_sync();
                         const float na = fmaxf(m_a, msa), nb = fmaxf(m_b, msb);
@@ -657,9 +545,8 @@ salad_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
             __syncwarp();
             if (lane == 0) mbar_arrive(smem_u32(&bars.p_ready[s]));   // one arrival per warp
         }
-        // From here on addresses come from copies that the compiler knows nothing of: it would form all of them once, ahead of
-        // the items, and keep them in registers that the loop above needs (1580 cycles per block instead of 1380).
-        const bool linear = item.linear != 0;
+        // From here on addresses come from copies that the compiler knows nothing of: it would form all of them ahead of
+        // the loop above and keep them in registers that the loop needs.
         int elane = lane;
         uint32_t sb = s_base;
         asm volatile("" : "+r"(elane), "+r"(sb));
@@ -677,12 +564,12 @@ salad_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
             const bool rotary = p.rope != nullptr;
             auto rot_ptr = [&](int it) {
                 const int row = (it & 1) ? rb : ra;
-                const int tok = min(item.qb * p.Bq + row, p.N - 1);           // rows past the block or N hold zeros
+                const int tok = min(qb * p.Bq + row, p.N - 1);           // rows past the block or N hold zeros
                 return reinterpret_cast<const uint4*>(p.rope + size_t(tok) * D + (it >> 2) * 64 +
                                                       (q4 + 4 * ((it >> 1) & 1)) * 8);
             };
-            ok = wait_uniform(&bars.q_full, (ph >> 2) & 1);
-            if (ok) ok = wait_uniform(&bars.z_full, (ph >> 4) & 1);
+            ok = wait_uniform(&bars.q_full, 0);
+            if (ok) ok = wait_uniform(&bars.z_full, 0);
             if (ok) {
                 // Four vectors are read before the first is written over (in turn, each load would wait for the store before it,
                 // which may go to the same place for all the compiler knows), Z is read once for both rows, the rotary form
@@ -741,14 +628,11 @@ salad_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
             }
         }
         if (ok && len > 0) {
-            ok = wait_uniform(&bars.o_final, (ph >> 3) & 1);
+            ok = wait_uniform(&bars.o_final, 0);
             tc_fence_after_sync();
-        } else if (ok && k > 0) {
-            // (the store of the item before has read the tile that is written below: said by its V loads otherwise)
-            ok = wait_uniform(&bars.v_free, (k - 1) & 1);
         }
         if (ok && linear) {
-            ok = wait_uniform(&bars.lin_done, (ph >> 4) & 1);
+            ok = wait_uniform(&bars.lin_done, 0);
             tc_fence_after_sync();
         }
 
@@ -779,9 +663,6 @@ salad_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
                     sts_32(oa + 8 * 128 + off, pack_bf16x2(b0, b1));
                 }
             }
-            tc_fence_before_sync();
-            __syncwarp();
-            if (linear && lane == 0) mbar_arrive(smem_u32(&bars.num_free));     // the score buffers are free for the next item
             fence_proxy_async_smem();
             __syncwarp();
             if (lane == 0) mbar_arrive(smem_u32(&bars.out_staged));
@@ -789,20 +670,17 @@ salad_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
 #pragma unroll
                 for (int e2 = 0; e2 < 2; ++e2) {
                     const int row = e2 ? rb : ra;
-                    int n = item.qb * p.Bq + row;
+                    int n = qb * p.Bq + row;
                     if (perm) {                      // row = position within the block * T + frame
-                        const int sp = item.qb * p.th.kq + row / p.th.T;
+                        const int sp = qb * p.th.kq + row / p.th.T;
                         n = (sp < p.th.S) ? (row % p.th.T) * p.th.S + sp : p.N;
                     }
                     if (row < q_rows && n < p.N)
-                        p.lse[size_t(item.bh) * p.N + n] =
+                        p.lse[size_t(bh) * p.N + n] =
                             (len > 0) ? ((e2 ? m_b : m_a) + log2f(e2 ? lt_b : lt_a)) * 0.6931471805599453f : -INFINITY;
                 }
             }
         }
-        release_item(k);
-        ph = ((ph + uint32_t(len)) & 3u) | ((ph ^ ((len > 0 || linear) ? 4u : 0u) ^ (len > 0 ? 8u : 0u) ^ (linear ? 16u : 0u)) & 28u);
-        }  // items
         }  // rows of queries
     }
     }  // !inherited_abort
@@ -813,7 +691,7 @@ salad_fused_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_const
     // The first kernel of the next call waits for this grid and for nothing before it, so this grid must not end ahead of the
     // state kernels of its own call, also where no CTA needed them (rejected lists, dropped items).
     // (Only there: the instruction is not free, 2 us of a 32 us call when every CTA issues it once more.)
-    if ((p.mode & MODE_LINEAR) != 0 && state_waited == 0) grid_dependency_wait();
+    if ((p.mode & MODE_LINEAR) != 0 && (!linear || inherited_abort)) grid_dependency_wait();
     if (abort_flag != 0 && !inherited_abort) {
         // a bounded wait expired somewhere (1: in this CTA, reported here; 2: in the state kernels, which
         // reported it themselves): give copies in flight time to land, leave

@@ -52,27 +52,6 @@ __device__ __forceinline__ void grid_launch_dependents() {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
-// ---------------------------------------------------------------------------------- cluster launch control
-// A running CTA takes the place of the next CTA of its grid that has not started: the answer (16 bytes, completing as
-// many on the barrier) says whether there was one and which.  No further request after an answer that there was none.
-__device__ __forceinline__ void clc_try_cancel(uint32_t answer, uint32_t bar) {
-    asm volatile("clusterlaunchcontrol.try_cancel.async.shared::cta.mbarrier::complete_tx::bytes.b128 [%0], [%1];"
-                 ::"r"(answer), "r"(bar) : "memory");
-}
-// blockIdx.x of the CTA taken over, or -1
-__device__ __forceinline__ int clc_answer(uint32_t answer) {
-    int x;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t.reg .b128 a;\n\t.reg .b32 cx, cy, cz;\n\t"
-        "ld.shared.b128 a, [%1];\n\t"
-        "clusterlaunchcontrol.query_cancel.is_canceled.pred.b128 p, a;\n\t"
-        "mov.b32 %0, -1;\n\t"
-        "@p clusterlaunchcontrol.query_cancel.get_first_ctaid.v4.b32.b128 {cx, cy, cz, _}, a;\n\t"
-        "@p mov.b32 %0, cx;\n\t}"
-        : "=r"(x) : "r"(answer) : "memory");
-    return x;
-}
-
 // ---------------------------------------------------------------------------------- mbarrier
 __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");

@@ -433,11 +433,6 @@ int launch_fused(const Problem& P, const KvMaps& kv, const Workspace& w, const D
     fp.rope = static_cast<const __half*>(P.rope);
     fp.ws_status = reinterpret_cast<int32_t*>(ws + w.off_status);
     fp.user_status = P.d_status;
-    // More items than the chip takes at once: a CTA that has finished one takes over the next.  (With no more, there is
-    // nothing to take but the few CTAs that wait for a state CTA to leave their SM, and they start sooner by themselves:
-    // 12 heads of 2310 tokens 37.7 against 32.3 us; 396 and 456 items 47.3 -> 46.1 and 49.9 -> 48.2.)  The tiles of ST-SWA's
-    // two kinds of heads differ in their unused rows, which a CTA clears only once.
-    fp.take_over = P.st_T == 0 && int64_t(fp.nQb) * BH > 2 * dev.sms ? 1 : 0;
     fp.wait_at_top = P.prepared ? 1 : 0;      // no state kernels in this call: the kernel before is the first one
     const int64_t grid = int64_t(fp.nQb) * BH;
     if (grid > 2147483647ll) return SALAD_ERR_UNSUPPORTED;

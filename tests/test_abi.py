@@ -157,27 +157,12 @@ def test_native_calls_answer_like_ctypes(lib):
     assert lib._fast["salad_fused_fwd"](*good[:-1]) is None
 
 
-def test_registers_left_to_the_producer_warps(lib, tmp_path):
-    """What setmaxnreg.dec leaves to the producer and issuer warps of the attention kernel is more than they take when nothing limits
-    them, and all that is handed over was there at launch.  Compiled here: the kernel without its softmax warps and without setmaxnreg."""
-    from paper_2601_16515_b200 import build
-    source = open(os.path.join(build.CSRC, "fused_kernel.cuh")).read()
-    dec, inc = (int(re.search(r"setmaxnreg\.%s\.sync\.aligned\.u32 (\d+);" % x, source).group(1)) for x in ("dec", "inc"))
-    at_launch = 65536 // (2 * 384) // 8 * 8
-    assert 128 * dec + 256 * inc <= 384 * at_launch
-    softmax, end = source.index("= softmax + epilogue\n"), source.index("    }  // !inherited_abort")
-    rest = source[:softmax] + "\n    }\n" + source[end:]
-    rest = re.sub(r'asm volatile\("setmaxnreg[^;]*;[^;]*;', "", rest)
-    (tmp_path / "part.cuh").write_text(rest.replace('#include "ptx.cuh"', '#include "%s"' % os.path.join(build.CSRC, "ptx.cuh")))
-    several = re.search(r"template <([^>]*)>\s*__global__ void __launch_bounds__\(384, 2\)", source).group(1).count(",")
-    kinds = [f"{d}{flag}" for d in (64, 128) for flag in ((", true", ", false") if several else ("",))]
-    (tmp_path / "part.cu").write_text('#include "part.cuh"\nvoid* kernels[] = {%s};\n' % ", ".join(
-        f"reinterpret_cast<void*>(salad::salad_fused_kernel<{k}>)" for k in kinds))
-    done = subprocess.run(["nvcc", "-gencode", "arch=compute_100a,code=sm_100a", "-O3", "-std=c++17", "-Xptxas", "-v", "-cubin",
-                           "-o", str(tmp_path / "part.cubin"), str(tmp_path / "part.cu")], capture_output=True, text=True)
-    assert done.returncode == 0, done.stderr[-2000:]
-    took = [int(n) for n in re.findall(r"Used (\d+) registers", done.stderr)]
-    assert len(took) == len(kinds) and max(took) <= dec, (took, dec)
+def test_no_registers_change_hands():
+    """No kernel hands registers over between its warps: ptxas 12.9 lost values that live across setmaxnreg in forms of the attention
+    kernel (wrong outputs, no warning), and the same sources without it were right."""
+    csrc = os.path.join(ROOT, "paper_2601_16515_b200", "csrc")
+    for name in sorted(os.listdir(csrc)):
+        assert "setmaxnreg" not in re.sub(r"//[^\n]*", "", open(os.path.join(csrc, name)).read()), name
 
 
 def test_tensor_memory_loads_wait_where_they_load():
