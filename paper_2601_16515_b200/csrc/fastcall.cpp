@@ -55,7 +55,7 @@ PyObject* call(int (*fn)(A...), PyObject* const* args, Py_ssize_t n) {
 #define SALAD_FAST(X) \
     X(salad_fused_fwd) X(salad_fused_drop_fwd) X(salad_sparse_attn_fwd) X(salad_linear_attn_fwd) X(salad_linear_state_fwd) \
     X(salad_fused_prepared_fwd) X(salad_fused_rope_fwd) X(salad_linear_attn_rope_fwd) X(salad_fused_proj_fwd) \
-    X(salad_topk_mask_build) X(salad_dynamic_scale) X(salad_proj_combine_fwd)
+    X(salad_topk_mask_build) X(salad_dynamic_scale) X(salad_proj_combine_fwd) X(salad_fused_stswa_fwd)
 
 #define X(name) \
     decltype(&name) g_##name = nullptr; \

@@ -490,8 +490,8 @@ def salad_fused_stswa_fwd(q, k, v, grid, head_flags, row_ptr, col_idx, static_sc
     if out is None:
         out = torch.empty_like(q)
     tau = float("-inf") if drop_tau is None else float(drop_tau)
-    _call("salad_fused_stswa_fwd", q, stream, _ptr(q), _ptr(k), _ptr(v), _ptr(out), B, H, N, d, T, Hs, Ws, flags,
-          _ptr(row_ptr), _ptr(col_idx), _ptr(static_scale), _ptr(dyn_scale), tau, float(softmax_scale), float(eps),
+    _call("salad_fused_stswa_fwd", q, stream, _ptr(q), _ptr(k), _ptr(v), _ptr(out), B, H, N, d, T, Hs, Ws,
+          ctypes.addressof(flags), _ptr(row_ptr), _ptr(col_idx), _ptr(static_scale), _ptr(dyn_scale), tau, float(softmax_scale), float(eps),
           _ptr(workspace), workspace.numel(), _ptr(status))
     return out
 

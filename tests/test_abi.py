@@ -202,3 +202,14 @@ def test_without_the_native_module(lib, tmp_path, monkeypatch):
             "assert salad._enter('salad_fused_fwd', None, *good[1:]) == salad.SALAD_ERR_INVALID_ARG\n"
             "assert salad._enter('salad_fused_fwd', *good[:18], n - 1, None, None) == salad.SALAD_ERR_WORKSPACE\n")
     subprocess.run([sys.executable, "-c", code], cwd=ROOT, check=True)
+
+
+def test_stswa_call_bypasses_ctypes(lib):
+    """The ST-SWA call, whose head flags are host memory, takes the way of the other calls of every layer, with ctypes' answers."""
+    flags = (ctypes.c_int32 * 2)(0, 1)
+    p, n = 1 << 20, lib._lib.salad_stswa_workspace_bytes(1, 2, 4, 16, 16, 64)
+    good = [p, p, p, p, 1, 2, 1024, 64, 4, 16, 16, ctypes.addressof(flags), p, p, p, p, 0.5, 0.0, 1e-6, p, n, None, None]
+    for change in ({0: None}, {3: p + 8}, {6: 1023}, {7: 96}, {8: 65}, {11: None}, {17: -1.0}, {18: float("nan")}, {19: p + 1}, {20: n - 1}):
+        args = [change.get(i, a) for i, a in enumerate(good)]
+        rc = lib._fast["salad_fused_stswa_fwd"](*args)
+        assert isinstance(rc, int) and rc == lib._lib.salad_fused_stswa_fwd(*args) and rc < 0, change
