@@ -1,6 +1,6 @@
 // Python's way into the entry points that a layer calls on every step: the same functions of libsalad as through ctypes,
 // with their arguments converted here by their C++ types instead of by ctypes' interpreter (a call with its 21 arguments
-// costs 0.3 us instead of 2.5, of the 15 us that the host spends on the smallest fused call).  Addresses come from the
+// costs 0.2 us instead of 2.5, of the 15 us that the host spends on the smallest fused call).  Addresses come from the
 // loaded library (bind), so nothing is linked.  What these conversions do not take (anything but plain integers, floats
 // and None) they leave to ctypes: the answer is None then and nothing has been called.
 #define PY_SSIZE_T_CLEAN
