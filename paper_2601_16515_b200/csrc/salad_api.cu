@@ -416,11 +416,13 @@ int launch_fused(const Problem& P, const KvMaps& kv, const Workspace& w, const D
     }
     fp.row_ptr = P.row_ptr; fp.col_idx = P.col_idx;
     fp.BH = BH;
-    // Where K and V of all heads fit in half of the 126 MB L2, the items go by expense over all heads: 12 heads of 2310 tokens
-    // 32.4 -> 28.0 us (attention alone 27.1 -> 23.4, rotary 37.7 -> 31.7), 4158 tokens 45.8 -> 43.2, 7854 tokens (48 MB) 112 -> 108;
-    // 40 heads of 900 tokens 39.9 -> 35.9, of 2310 tokens 75.8 -> 72.0.  Beyond, K and V come from memory more than once: 12 heads of
-    // 16464 tokens (101 MB) 243 against 265 us.
-    fp.by_rank = int64_t(BH) * P.N * D * 4 <= (int64_t(64) << 20) ? 1 : 0;
+    // Where K and V of all heads take no more than 48 MB of the 126 MB L2, the items go by expense over all heads: one list for
+    // all, 12 heads of 2310 tokens 32.4 -> 28.0 us (attention alone 27.1 -> 23.4, rotary 37.7 -> 31.7), 4158 tokens 45.8 -> 43.2, 7854
+    // tokens (48 MB) 112 -> 108; lists per head, 24 heads of 1936 tokens (23 MB) 30.5 -> 29.4, of 3465 (41 MB) 46.0 -> 43.1, 12 heads of
+    // 15318 at d = 64 (45 MB) 127 -> 122.  From there it gains nothing, then loses, K and V coming from memory more than once:
+    // all blocks kept, 5 heads of 20384 tokens (50 MB) 961 -> 964, 40 of 2852 (56 MB) 187 -> 192; 4 of 38880 (76 MB) 309 -> 326; 12 of
+    // 16464 (101 MB) 243 -> 265.
+    fp.by_rank = int64_t(BH) * P.N * D * 4 <= (int64_t(48) << 20) ? 1 : 0;
     fp.order = nullptr;
     if (P.mode & MODE_SPARSE) fp.order = reinterpret_cast<const int32_t*>(ws + w.off_order);   // written by run()
     fp.static_scale = P.static_scale; fp.dyn_scale = P.dyn_scale;

@@ -1522,3 +1522,21 @@ def test_a_cta_with_several_items(salad, d, Bq, longest):
     again = salad.salad_fused_fwd(qd, kd, vd, rp_d, ci_d, B * H, lam_d, s_d, Bq=Bq, drop_tau=0.5)
     clean = [h for h in range(H) if h not in (0, 7, 23)]
     assert torch.equal(again[0, clean], out[0, clean]) and torch.equal(again[1], out[1])
+
+
+# The order of the work items changes with the size of K and V (48 MB): a call above the line gives the bits of its parts below it.
+@pytest.mark.parametrize("d,Bq,N,H", [(128, 128, 2049, 48), (128, 64, 1290, 80), (64, 128, 4100, 49), (64, 64, 3137, 64)])
+def test_order_of_the_items(salad, d, Bq, N, H):
+    assert H * N * d * 4 > 48 << 20 >= (H // 3 + 1) * N * d * 4
+    q, k, v = (x.cuda() for x in rand_qkv(1, H, N, d, d + Bq + N))
+    nQb, nKb = -(-N // Bq), -(-N // 64)
+    rp, ci = random_csr(H * nQb, nKb, d + N, lo=0, hi=5)
+    lse = torch.empty((1, H, N), device="cuda")
+    whole = salad.salad_sparse_attn_fwd(q, k, v, *dev_csr(rp, ci), H, Bq=Bq, lse=lse)
+    for a in range(0, H, H // 3 + 1):
+        b = min(H, a + H // 3 + 1)
+        rows = rp[a * nQb:b * nQb + 1]
+        part_lse = torch.empty((1, b - a, N), device="cuda")
+        part = salad.salad_sparse_attn_fwd(*(x[:, a:b].contiguous() for x in (q, k, v)), *dev_csr(rows - rows[0], ci[rows[0]:rows[-1]]),
+                                           b - a, Bq=Bq, lse=part_lse)
+        assert torch.equal(part, whole[:, a:b]) and torch.equal(part_lse, lse[:, a:b])
