@@ -1487,12 +1487,12 @@ def test_linear_call_stops_on_a_reported_failure(salad, d):
     assert torch.equal(salad.salad_linear_attn_fwd(q, k, v, workspace=ws), want)
 
 
-# ------------------------------------------------------------------------------ several items per CTA
+# ------------------------------------------------------------------------------ more work items than the chip takes at once
 
 @pytest.mark.parametrize("d,Bq,longest", [(128, 128, 5), (128, 64, 3), (64, 128, 2), (64, 64, 4)])
 def test_a_cta_with_several_items(salad, d, Bq, longest):
-    # More work items than the chip takes at once, with lists of 0 to `longest` blocks in any order (the parity of the
-    # buffers changes from item to item), half of the items without a linear branch, a ragged end.
+    # More work items than the chip takes at once, so that CTAs follow one another on an SM (and may be made to take several
+    # items), with lists of 0 to `longest` blocks in any order, half of the items without a linear branch, a ragged end.
     B, H, N = 2, 40, 1290
     q, k, v = rand_qkv(B, H, N, d, 5 * d + Bq)
     nQb, nKb = -(-N // Bq), -(-N // 64)
